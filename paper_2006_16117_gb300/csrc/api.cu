@@ -216,19 +216,21 @@ void upload_pencil(DeviceArena& ar, cudaStream_t st, Pencil& P, const std::vecto
     P.T += P.T & 1;  // even: block rows stay 16-byte aligned in complex64
     P.nb = (int)((n + P.T - 1) / P.T);
     P.b_kind = b_kind;
-    // couplings to the next block row, column-compressed per block
-    const int T = P.T, nb = P.nb;
+    // couplings to the inner neighbour, column-compressed per block
+    P.mid = P.nb / 2;
+    const int T = P.T, nb = P.nb, mid = P.mid;
     std::vector<int32_t> up_ptr((size_t)nb * (T + 1), 0), up_row, up_idx;
     {
         std::vector<std::vector<std::pair<int32_t, int32_t>>> cols(T);
-        for (int k = 0; k + 1 < nb; ++k) {
+        for (int k = 0; k < nb; ++k) {
             for (auto& c : cols) c.clear();
-            for (int i = 0; i < T; ++i) {
+            const int64_t b0 = (int64_t)(k < mid ? k + 1 : k - 1) * T;  // the inner neighbour's columns
+            for (int i = 0; i < T && k != mid; ++i) {
                 int64_t g = (int64_t)k * T + i;
                 if (g >= n) break;
                 for (int64_t e = rp[g]; e < rp[g + 1]; ++e) {
                     int64_t j = ci[e];
-                    if (j >= (int64_t)(k + 1) * T) cols[j - (int64_t)(k + 1) * T].push_back({i, (int32_t)e});
+                    if (j >= b0 && j < b0 + T) cols[j - b0].push_back({i, (int32_t)e});
                 }
             }
             size_t base = (size_t)k * (T + 1);
@@ -242,14 +244,16 @@ void upload_pencil(DeviceArena& ar, cudaStream_t st, Pencil& P, const std::vecto
             }
         }
     }
-    // couplings to the previous block row
+    // couplings to the outer neighbour (both neighbours of mid)
     std::vector<int32_t> Lptr(n + 1, 0), Lcol, Lidx;
     for (int64_t g = 0; g < n; ++g) {
         const int64_t k = g / T;
         for (int64_t e = rp[g]; e < rp[g + 1]; ++e) {
             const int64_t j = ci[e];
-            if (k > 0 && j < k * T && j >= (k - 1) * T) {
-                Lcol.push_back((int32_t)(j - (k - 1) * T));
+            const bool below = j < k * T, above = j >= (k + 1) * T;
+            if ((below && k <= mid) || (above && k >= mid)) {
+                const int64_t c = below ? j - (k - 1) * T : j - (k + 1) * T;
+                Lcol.push_back((int32_t)(above && k == mid ? c + T : c));
                 Lidx.push_back((int32_t)e);
             }
         }
@@ -525,9 +529,10 @@ bool solve_nodes(sim_ctx* h, int dir, const std::vector<double2>& z, const doubl
     if (!P.sep) {
         auto& fac = h->nfactors[dir];
         if ((int)fac.size() < N) fac.resize(N, nullptr);
+        const size_t bytes = factor_storage_bytes(P, h->opt.precision);
         for (int j = 0; j < N; ++j)
             if (!fac[j]) {
-                cudaError_t e = cudaMalloc(&fac[j], h->factor_bytes);
+                cudaError_t e = cudaMalloc(&fac[j], bytes);
                 if (e != cudaSuccess) throw CudaError{e, "cudaMalloc of a node factorisation"};
             }
         SIM_CUDA(cudaMemcpyAsync(h->d_nfptrs[dir], fac.data(), sizeof(void*) * N, cudaMemcpyHostToDevice, h->st));
@@ -819,8 +824,7 @@ sim_status sim_create(const sim_csr* A, const sim_csr* B, const sim_options* opt
             }
         }
         SIM_CUDA(cudaStreamSynchronize(h->st));
-        const size_t cs = o.precision == SIM_FP64 ? sizeof(double2) : sizeof(float2);
-        h->factor_bytes = ((size_t)2 * nb * (size_t)T * T + (size_t)P.nnzL + (size_t)n + 16) * cs;
+        h->factor_bytes = factor_storage_bytes(P, o.precision);
         ensure_shift_capacity(h.get());
         h->d_f = h->arena.get<double2>("f", n);
         h->stats.n = n;

@@ -1,11 +1,15 @@
-// Block Thomas factorisation of A - σB on thread-block clusters.
+// Block-tridiagonal factorisation of K = A - σB on thread-block clusters.
 //
-// Same factors as k_factor (krylov.cu): Dinv_k = D_k^{-1} with
-// D_k = A_kk - σB_kk - L_k E_{k-1}, and E_k = Dinv_k U_k, plus the shifted
-// values of the couplings L_k.  The blocks form a serial chain and every block
-// is T pivots long, so the time of a pivot bounds the factorisation.
+// Same factors as k_factor (krylov.cu): the blocks are eliminated from both ends
+// to the middle block mid, Dinv_k = D_k^{-1} with
+//   D_k = K_kk - K_{k,outer(k)} E_{outer(k)}   (mid: minus both neighbours' terms),
+//   E_k = Dinv_k K_{k,inner(k)},
+// plus the shifted values of the outer couplings.  The blocks of a side form a
+// serial chain and every block is T pivots long, so the time of a pivot bounds
+// the factorisation, and two sides halve it: one launch factors the sides, one
+// cluster each, and a second one the middle block of every shift.
 //
-// A cluster of Cf CTAs factors one shift.  CTA q keeps Tc columns of D_k (all
+// A cluster of Cf CTAs factors one side of one shift.  CTA q keeps Tc columns of D_k (all
 // T rows) in shared memory, so a pivot search never leaves its CTA.  The
 // in-place Gauss-Jordan inversion runs in panels of B columns:
 //   panel   the owner's threads hold one row of the panel each, in registers;
@@ -31,10 +35,11 @@
 // complex128: the panel's own multiply-adds, T·B·B of them on one SM, are cheap
 // in FP32 and as dear as the whole update in FP64.
 //
-// Measured for one shift, against rows over the cluster with two cluster barriers
-// a pivot: T = 200, nb = 200 complex64 138 -> 39.7 ms (2,050 clocks a pivot, about
-// 1,000 of them the pivot itself); T = 98, nb = 97 complex128 106 -> 31.6 ms;
-// T = 30, nb = 30 complex128 5.6 -> 2.2 ms (16 nodes of T = 64: 56 -> 10 ms).
+// Measured for one shift, T = 200, nb = 200 complex64: 138 ms with rows over the
+// cluster and two cluster barriers a pivot, 39.7 with the panels (2,050 clocks a
+// pivot, about 1,000 of them the pivot itself), 20.1 from both ends; T = 98, nb =
+// 97 complex128: 106, 31.6, 16.0 ms; T = 30, nb = 30 complex128: 5.6, 2.2, 1.2 ms.
+// 55 shifts of T = 200 complex64 in two calls: 372 -> 80 ms.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -223,25 +228,29 @@ template <class F> __device__ __forceinline__ void for_elements(int rows, int co
     }
 }
 
-// S -= L_k E_{k-1}, my columns (Ep at my first column); each row's first coupling is staged
+// S -= K_{k,outer} E_outer, my columns (Ep and for mid's second neighbour Ep2 at my
+// first column); each row's first coupling is staged
 template <class C> struct SubCouplings {
     using Value = C;
     C* S;
     int ld, T;
-    const C* Ep;
+    const C *Ep, *Ep2;
     const C* l0v;
     const int *l0c, *llo, *lhi;
     const C* Lval;
     const int32_t* Lcol;
-    __device__ __forceinline__ C load(int i, int c) const { return Ep[(size_t)l0c[i] * T + c]; }
+    __device__ __forceinline__ C at(int col, int c) const {
+        return col < T ? Ep[(size_t)col * T + c] : Ep2[(size_t)(col - T) * T + c];
+    }
+    __device__ __forceinline__ C load(int i, int c) const { return at(l0c[i], c); }
     __device__ __forceinline__ void use(int i, int c, C v) const {
         C acc = cmul(l0v[i], v);
-        for (int e = llo[i]; e < lhi[i]; ++e) acc = cfma(Lval[e], Ep[(size_t)Lcol[e] * T + c], acc);
+        for (int e = llo[i]; e < lhi[i]; ++e) acc = cfma(Lval[e], at(Lcol[e], c), acc);
         S[(size_t)i * ld + c] = csub(S[(size_t)i * ld + c], acc);
     }
 };
 
-// E_k = Dinv_k U_k, my columns; each column's first coupling is staged
+// E_k = Dinv_k K_{k,inner}, my columns; each column's first coupling is staged
 template <class C> struct FormE {
     using Value = C;
     const Pencil& P;
@@ -264,12 +273,17 @@ template <class C> struct FormE {
 
 template <class C, int B, int CT, int NT>
 __global__ void __launch_bounds__(NT, 1) k_factor_cl(Pencil P, const int* shift_list, const double2* sigma,
-                                                      void* const* fptrs, int* err, int Tc) {
+                                                      void* const* fptrs, int* err, int Tc, int phase) {
     cg::cluster_group cl = cg::this_cluster();
     const int Cf = (int)cl.num_blocks();
     const int q = (int)cl.block_rank();
-    const int T = P.T, nb = P.nb;
-    const int s = shift_list[blockIdx.x / Cf];
+    const int T = P.T, nb = P.nb, mid = P.mid;
+    // phase 0: blocks 0 .. mid-1 (side 0) or nb-1 .. mid+1 (side 1, launched if there
+    // are any); phase 1: block mid
+    const int sides = phase == 0 && mid + 1 < nb ? 2 : 1, side = (int)(blockIdx.x / Cf) % sides;
+    const int len = phase ? 1 : (side ? nb - 1 - mid : mid);
+    const int kfirst = phase ? mid : (side ? nb - 1 : 0), kstep = side ? -1 : 1;
+    const int s = shift_list[blockIdx.x / Cf / sides];
     C* Dinv = reinterpret_cast<C*>(fptrs[s]);
     C* E = Dinv + (size_t)nb * T * T;
     C* Lval = Dinv + factor_lval_offset(P);
@@ -298,11 +312,15 @@ __global__ void __launch_bounds__(NT, 1) k_factor_cl(Pencil P, const int* shift_
     int* pnew = uhi + Tc;                      // [B] pivot rows of the panel being factored
     int* ctr = pnew + B;
 
-    for (int64_t e = tid + (int64_t)q * nt; e < P.nnzL; e += (int64_t)nt * Cf)
-        Lval[e] = from_c128<C>(sval(P, P.Lidx[e], sg));
     {
+        // the couplings of my rows
+        const int klo = side ? kfirst - (len - 1) : kfirst;
+        const int64_t g_lo = (int64_t)klo * T, g_hi = min(P.n, (int64_t)(klo + len) * T);
+        const int64_t e_hi = P.Lptr[g_hi];
+        for (int64_t e = P.Lptr[g_lo] + tid + (int64_t)q * nt; e < e_hi; e += (int64_t)nt * Cf)
+            Lval[e] = from_c128<C>(sval(P, P.Lidx[e], sg));
         C* L0val = Dinv + factor_l0_offset(P);
-        for (int64_t g = tid + (int64_t)q * nt; g < P.n; g += (int64_t)nt * Cf) {
+        for (int64_t g = g_lo + tid + (int64_t)q * nt; g < g_hi; g += (int64_t)nt * Cf) {
             const int e0 = P.Lptr[g];
             L0val[g] = from_c128<C>(P.Lptr[g + 1] > e0 ? sval(P, P.Lidx[e0], sg) : make_double2(0.0, 0.0));
         }
@@ -452,18 +470,19 @@ __global__ void __launch_bounds__(NT, 1) k_factor_cl(Pencil P, const int* shift_
         S[(size_t)r * ld + c] = v;
     };
 
-    for (int k = 0; k < nb; ++k) {
+    for (int t = 0; t < len; ++t) {
+        const int k = kfirst + t * kstep;
         const int64_t g0 = (int64_t)k * T;
         C* Dk = Dinv + (size_t)k * T * T;
-        C* scr = E + (size_t)k * T * T;  // G's way to the other CTAs (E_{nb-1}, never used, for the last block)
-        // 1. my columns of D_k = K_kk - L_k E_{k-1}
+        C* scr = E + (size_t)k * T * T;  // G's way to the other CTAs (E_mid's place is free)
+        // 1. my columns of D_k = K_kk - K_{k,outer} E_outer
         for (int idx = tid; idx < T * ld; idx += nt) S[idx] = zc<C>();
         for (int i = tid; i < T; i += nt) {
             const int64_t g = g0 + i;
             used[i] = 0;
             int lo = 0, hi = 0, col = 0;
             C v = zc<C>();
-            if (k > 0 && g < P.n) {
+            if (g < P.n) {
                 lo = P.Lptr[g];
                 hi = P.Lptr[g + 1];
                 if (hi > lo) {
@@ -476,7 +495,7 @@ __global__ void __launch_bounds__(NT, 1) k_factor_cl(Pencil P, const int* shift_
             llo[i] = lo + 1;
             lhi[i] = hi;
         }
-        if (k < nb - 1) {  // the first coupling of my columns of U_k, for step 4
+        if (k != mid) {  // the first coupling of my columns of K_{k,inner}, for step 4
             const int32_t* cp = P.up_ptr + (size_t)k * (T + 1);
             for (int c = tid; c < myc; c += nt) {
                 const int lo = cp[c0 + c], hi = cp[c0 + c + 1];
@@ -508,9 +527,11 @@ __global__ void __launch_bounds__(NT, 1) k_factor_cl(Pencil P, const int* shift_
             }
         }
         __syncthreads();
-        if (k > 0 && myc > 0) {
-            const C* Ep = E + (size_t)(k - 1) * T * T + c0;  // my columns, written by this CTA
-            for_elements(T, myc, SubCouplings<C>{S, ld, T, Ep, l0v, l0c, llo, lhi, Lval, P.Lcol});
+        if ((phase ? nb > 1 : t > 0) && myc > 0) {
+            // my columns, written by this CTA (phase 1: by the launch before)
+            const C* Ep = E + (size_t)(phase ? max(mid - 1, 0) : k - kstep) * T * T + c0;
+            const C* Ep2 = E + (size_t)min(mid + 1, nb - 1) * T * T + c0;
+            for_elements(T, myc, SubCouplings<C>{S, ld, T, Ep, Ep2, l0v, l0c, llo, lhi, Lval, P.Lcol});
         }
         __syncthreads();
         // 2. Gauss-Jordan in panels
@@ -585,8 +606,8 @@ __global__ void __launch_bounds__(NT, 1) k_factor_cl(Pencil P, const int* shift_
             cluster_wait();
         }
         __syncthreads();
-        // 4. my columns of E_k = Dinv_k U_k
-        if (k < nb - 1 && myc > 0) {
+        // 4. my columns of E_k = Dinv_k K_{k,inner}
+        if (k != mid && myc > 0) {
             C* Ek = E + (size_t)k * T * T + c0;
             for_elements(T, myc, FormE<C>{P, sg, T, Dk, Ek, u0v, u0c, ulo, uhi});
             __syncthreads();
@@ -629,7 +650,7 @@ cudaLaunchConfig_t factor_config(int clusters, const FactorShape& f, cudaStream_
     return cfg;
 }
 
-using FactorKernel = void (*)(Pencil, const int*, const double2*, void* const*, int*, int);
+using FactorKernel = void (*)(Pencil, const int*, const double2*, void* const*, int*, int, int);
 
 FactorKernel factor_kernel(size_t cs, int B, int threads) {
     if (cs == sizeof(double2)) return threads <= 384 ? k_factor_cl<double2, 4, 4, 384> : k_factor_cl<double2, 4, 4, 512>;
@@ -708,7 +729,8 @@ bool factor_shifts_cluster(const Pencil& P, int precision, const int* d_shift_li
     if (count <= 0) return true;
     const size_t cs = precision == SIM_FP64 ? sizeof(double2) : sizeof(float2);
     if (P.T < 2 || P.T > 32 * FC_MAXW || admit_bytes(P.T, cs) > 220 * 1024) return false;
-    const FactorShape f = choose_factor_shape(P.T, cs, count);
+    const int sides = (P.mid > 0) + (P.mid + 1 < P.nb);
+    const FactorShape f = choose_factor_shape(P.T, cs, count * std::max(1, sides));
     if (f.Cf == 0) return false;
     if (!g_ferr) {
         SIM_CUDA(cudaMalloc(&g_ferr, sizeof(int)));
@@ -717,10 +739,12 @@ bool factor_shifts_cluster(const Pencil& P, int precision, const int* d_shift_li
     FactorKernel kern = factor_kernel(cs, f.B, f.threads);
     SIM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem));
     cudaLaunchAttribute attr[1];
-    const cudaLaunchConfig_t cfg = factor_config(count, f, st, attr);
     kprof_begin("factor", st);
-    SIM_CUDA(cudaLaunchKernelEx(&cfg, kern, P, d_shift_list, d_sigma, d_factor_ptrs, g_ferr, f.Tc));
-    SIM_LAUNCH_CHECK();
+    for (int phase = sides > 0 ? 0 : 1; phase < 2; ++phase) {
+        const cudaLaunchConfig_t cfg = factor_config(phase ? count : count * sides, f, st, attr);
+        SIM_CUDA(cudaLaunchKernelEx(&cfg, kern, P, d_shift_list, d_sigma, d_factor_ptrs, g_ferr, f.Tc, phase));
+        SIM_LAUNCH_CHECK();
+    }
     const double TT = (double)P.T * P.T;
     kprof_end("factor", st, count * (2.0 * P.nb * TT * cs), count * 8.0 * P.nb * TT * P.T);
     return true;

@@ -30,15 +30,23 @@ struct Pencil {
     const double2* Ka = nullptr;
     const double2* Kb = nullptr;
     const double2* Bdiag = nullptr;  // b_kind == 1: B's diagonal (complex128[n])
-    // couplings to block row k+1 in column-compressed form, one segment per
+    // The block elimination runs from both ends to the middle block mid: blocks
+    // below mid come before their upper neighbour, blocks above it before their
+    // lower one.  inner(k) is the neighbour on the way to mid, outer(k) the one
+    // on the way to the end.
+    // couplings to block row inner(k) in column-compressed form, one segment per
     // block row: for block k, entries [up_ptr[k*(T+1)+c], up_ptr[k*(T+1)+c+1])
-    // hold (row-in-block, value index) of column c of the block (k, k+1).
+    // hold (row-in-block, value index) of column c of the block (k, inner(k));
+    // none for mid.
+    int mid = 0;
     const int32_t* up_ptr = nullptr;
     const int32_t* up_row = nullptr;
     const int32_t* up_idx = nullptr;
-    // couplings to block row k-1, per row g: entries [Lptr[g], Lptr[g+1]) with
-    // column Lcol (relative to the start of block k-1) and value index Lidx.
-    // Each shift's factor stores the shifted values Lval (after E).
+    // couplings to block row outer(k), per row g: entries [Lptr[g], Lptr[g+1]) with
+    // column Lcol (relative to the start of that block) and value index Lidx; a
+    // row of block mid lists those to block mid-1 and then those to block mid+1,
+    // the latter's columns from T on.  Each shift's factor stores the shifted
+    // values Lval (after E).
     const int32_t* Lptr = nullptr;
     const int32_t* Lcol = nullptr;
     const int32_t* Lidx = nullptr;
@@ -54,6 +62,13 @@ struct Pencil {
     // shifted residual is about ε (||A|| + |σ| ||B||) ||x||
     double anorm = 0.0, bnorm = 0.0;
 };
+
+// Bytes of one shift's factorisation: Dinv and E (2 nb T² entries; E_mid's place
+// is scratch), Lval and L0val.
+inline size_t factor_storage_bytes(const Pencil& P, int precision) {
+    const size_t cs = precision == SIM_FP64 ? sizeof(double2) : sizeof(float2);
+    return ((size_t)2 * P.nb * (size_t)P.T * P.T + (size_t)P.nnzL + (size_t)P.n + 16) * cs;
+}
 
 // Offset (in elements of the factor type) of Lval inside a shift's factor.
 __host__ __device__ inline size_t factor_lval_offset(const Pencil& P) { return (size_t)2 * P.nb * P.T * P.T; }
@@ -104,7 +119,8 @@ constexpr int GS_THREADS = 256;
 
 // ---- krylov.cu ------------------------------------------------------------
 // Factor A - σB for the listed shifts into block form Dinv_k = D_k^{-1},
-// E_k = Dinv_k U_k (block Thomas).  factors[s] points to 2*nb*T*T entries of C.
+// E_k = Dinv_k K_{k,inner(k)} (block elimination from both ends).  factors[s]
+// points to factor_storage_bytes().
 void factor_shifts(const Pencil& P, int precision, const int* d_shift_list, int count,
                    const double2* d_sigma, void* const* d_factor_ptrs, cudaStream_t st);
 

@@ -2,12 +2,14 @@
 // (A - σB) and its inverse, and the Arnoldi process for M = (A - σB)^{-1} B
 // (Sec. 2, Eqs. AzBxf, IMxb, eq:arnoldi).
 //
-//  * factor_shifts  : block-tridiagonal (block Thomas) factorisation of A - σB
-//                     for many shifts at once, one CTA per shift; each
+//  * factor_shifts  : block-tridiagonal factorisation of A - σB, eliminated
+//                     from both ends to the middle block, for many shifts at
+//                     once, one CTA per shift (the blocks that the cluster
+//                     kernel of factor_cluster.cu does not hold); each
 //                     diagonal Schur complement D_k is inverted by Gauss–Jordan
 //                     with partial pivoting.  Storage: Dinv_k = D_k^{-1} and
-//                     E_k = Dinv_k U_k, both dense T×T, in complex128 (FP64
-//                     mode) or complex64 (mixed mode).
+//                     E_k = Dinv_k K_{k,inner(k)}, both dense T×T, in complex128
+//                     (FP64 mode) or complex64 (mixed mode).
 //  * (the solve x = (A - σB)^{-1} r through those factors is the cluster
 //    kernel of solve_cluster.cu)
 //  * inner_solve    : batched FGMRES(k) in FP64 with the factorisation as right
@@ -74,7 +76,10 @@ __global__ void __launch_bounds__(FACTOR_THREADS) k_factor(Pencil P, const int* 
             L0val[g] = P.Lptr[g + 1] > e0 ? from_c128<C>(shifted_val(P, P.Lidx[e0], sg)) : czero<C>();
         }
     }
-    for (int k = 0; k < nb; ++k) {
+    // from both ends to the middle: 0 .. mid-1, then nb-1 .. mid+1, then mid
+    const int mid = P.mid;
+    for (int t = 0; t < nb; ++t) {
+        const int k = t < mid ? t : (t < nb - 1 ? nb - 1 - (t - mid) : mid);
         C* D = Dinv + (size_t)k * TT;
         const int64_t g0 = (int64_t)k * T;
         for (int i = warp; i < T; i += nw)
@@ -92,8 +97,10 @@ __global__ void __launch_bounds__(FACTOR_THREADS) k_factor(Pencil P, const int* 
             }
         }
         __syncthreads();
-        if (k > 0) {
-            const C* Ep = E + (size_t)(k - 1) * TT;
+        {
+            // E of the outer neighbour; mid: block mid-1's, columns from T on block mid+1's
+            const C* Ep = E + (size_t)(k <= mid ? max(k - 1, 0) : min(k + 1, nb - 1)) * TT;
+            const C* Ep2 = E + (size_t)min(k + 1, nb - 1) * TT;
             const C* Lval = Dinv + factor_lval_offset(P);
             for (int i = warp; i < T; i += nw) {
                 const int64_t g = g0 + i;
@@ -101,7 +108,10 @@ __global__ void __launch_bounds__(FACTOR_THREADS) k_factor(Pencil P, const int* 
                 const int e0 = P.Lptr[g], e1 = P.Lptr[g + 1];
                 for (int c = lane; c < T; c += 32) {
                     C acc = czero<C>();
-                    for (int e = e0; e < e1; ++e) acc = cfma(Lval[e], Ep[(size_t)P.Lcol[e] * T + c], acc);
+                    for (int e = e0; e < e1; ++e) {
+                        const int col = P.Lcol[e];
+                        acc = cfma(Lval[e], col < T ? Ep[(size_t)col * T + c] : Ep2[(size_t)(col - T) * T + c], acc);
+                    }
                     D[(size_t)i * T + c] = csub(D[(size_t)i * T + c], acc);
                 }
             }
@@ -176,8 +186,8 @@ __global__ void __launch_bounds__(FACTOR_THREADS) k_factor(Pencil P, const int* 
                 __syncthreads();
             }
         }
-        // E_k = Dinv_k U_k, U_k = (A - σB)_{k,k+1} in column-compressed form
-        if (k < nb - 1) {
+        // E_k = Dinv_k K_{k,inner(k)}, that block in column-compressed form
+        if (k != mid) {
             C* Ek = E + (size_t)k * TT;
             const int32_t* cp = P.up_ptr + (size_t)k * (T + 1);
             for (int rr = warp; rr < T; rr += nw)

@@ -32,15 +32,34 @@ def _block_matrix(T, blocks, seed):
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 @pytest.mark.parametrize("T", [2, 4, 8, 10, 16, 18, 30, 32, 34, 64, 66, 96, 128, 130, 160, 256, 258, 280])
 def test_factor_of_permuted_blocks(precision, T):
+    _check(_block_matrix(T, 4, 40 + T), T, 5, precision)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("T", [2, 18, 34])
+@pytest.mark.parametrize("blocks", [1, 2, 3, 5])
+def test_chains_of_few_blocks(precision, T, blocks):
+    """Two to six block rows: sides of the two-ended elimination of uneven
+    length, down to one block and none."""
+    _check(_block_matrix(T, blocks, 90 + T), T, blocks + 1, precision)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("n", [1, 2])
+def test_a_single_block(precision, n):
+    A = sp.csr_matrix(np.array([[2.0 + 1j, 0.5], [-0.25j, 3.0]])[:n, :n])
+    _check(A, 2, 1, precision)
+
+
+def _check(A, T, nb, precision):
     if not torch.cuda.is_available():
         pytest.skip("no GPU")
     import paper_2006_16117_gb300 as simlib
 
-    A = _block_matrix(T, 4, 40 + T)
     A.sort_indices()
     n = A.shape[0]
     s = simlib.Sim((A.indptr, A.indices, A.data), None, simlib.sim_default_options(precision=precision))
-    assert s.stats()["block_size"] == T
+    assert s.stats()["block_size"] == T and s.stats()["num_blocks"] == nb
     rng = np.random.default_rng(7)
     r = rng.standard_normal(n) + 1j * rng.standard_normal(n)
     sigma = 0.3 - 0.2j
