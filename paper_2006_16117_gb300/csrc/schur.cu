@@ -14,7 +14,7 @@
 // paper's own formula (the eigendecomposition H_m = P D P^{-1}) gives the same
 // quantities; the Schur form is its unitary, backward-stable counterpart.
 //
-// k_schur: one warp per shift, the shifted QR algorithm of k_ritz applied to
+// k_schur: one CTA per shift, the shifted QR algorithm of k_ritz applied to
 // whole rows and columns with the rotations accumulated into the two rows of Z
 // the level needs (the first and the last: a row of Z evolves on its own
 // under the column rotations).
@@ -45,74 +45,159 @@ __device__ __forceinline__ double2 csqrt_s(double2 z) {
     return make_double2(re, z.y < 0.0 ? -im : im);
 }
 
-__device__ __forceinline__ double2 conj_s(double2 a) { return make_double2(a.x, -a.y); }
-
 }  // namespace
 
-// Shared memory: A [m][m] row-major, then rows 0 and n-1 of Z.
-__global__ void __launch_bounds__(32) k_schur(const double2* Hall, int m, const int* meff_all, const double* beta_all,
-                                              int s0, double2* Tall, double2* Call, double2* Qall, int* ok_all) {
+// 1 / sqrt(d) for a d well inside the range of normal numbers: an FP32 seed y0 of
+// d scaled by an even power of two (exponent arithmetic), then one third-order
+// Newton step y0 + y0 t (1/2 + 3/8 t) with t = 1 - d y0^2: five FP64 operations.
+__device__ __forceinline__ double rsqrt_nr(double d) {
+    const uint32_t hd = (uint32_t)__double2hiint(d), ld = (uint32_t)__double2loint(d);
+    const int e = ((int)(hd >> 20) - 1023) & ~1;  // even; d 2^-e in [1, 4)
+    const float f = __uint_as_float((((hd >> 20) - 1023u - (uint32_t)e + 127u) << 23) | ((hd & 0xFFFFFu) << 3) | (ld >> 29));
+    const uint32_t g = __float_as_uint(rsqrtf(f));  // (0.5, 1]
+    const double y0 = __hiloint2double((int)((((g >> 23) - 127u + 1023u - (uint32_t)(e / 2)) << 20) | ((g & 0x7FFFFFu) >> 3)),
+                                       (int)(g << 29));
+    const double t = fma(-(d * y0), y0, 1.0);
+    return fma(y0 * t, fma(0.375, t, 0.5), y0);
+}
+
+// The FP64 pipe takes 64 clocks of its scheduler for a warp instruction, however
+// few lanes are active, so k_schur spreads every rotation over lanes and warps
+// (m = 50: 20.8 ms on one warp, most of it scalar code of lane 0, now 3.7 ms):
+//  * update warps: a thread computes one real component of one rotated pair (three
+//    FP64 instructions).  Step k applies left rotation k to rows k, k+1 and, two
+//    steps behind, right rotation k-2 to columns k-2, k-1 of the rows that left
+//    rotations no longer touch, and to the two rows of Z.
+//  * a generator warp runs one rotation ahead: in step k it rotates column k+1's
+//    pair itself (nobody else touches that column in step k) and forms rotation
+//    k+1 from it, its sums, square roots and products side by side in four lanes
+//    (13 dependent FP64 instructions instead of about 150).
+//  * the deflation test takes a lane per subdiagonal, in the norm |re| + |im|.
+constexpr int SC_UPD = 256;           // update threads: 4 per pair, at most m + 3 pairs
+constexpr int SC_THREADS = SC_UPD + 32;
+
+// Shared memory: A [n][ld] row-major, then rows 0 and n-1 of Z as rows n, n+1 (ld odd).
+__global__ void __launch_bounds__(SC_THREADS) k_schur(const double2* Hall, int m, const int* meff_all,
+                                                      const double* beta_all, int s0, double2* Tall, double2* Call,
+                                                      double2* Qall, int* ok_all) {
     const int s = s0 + blockIdx.x;
     const int n = meff_all[s];
     const double2* Hs = Hall + (size_t)s * (m + 1) * m;  // column-major, leading dimension m + 1
     extern __shared__ double2 sh_schur[];
     double2* A = sh_schur;
-    double2* Z0 = sh_schur + (size_t)m * m;  // row 0 of Z
-    double2* Zl = Z0 + m;                    // row n-1 of Z
+    const int ld = m | 1;
     __shared__ double gc[64];
     __shared__ double2 gs[64];
     __shared__ double2 s_mu;
     __shared__ int s_l;
-    const int lane = threadIdx.x;
-    for (int idx = lane; idx < n * n; idx += 32) {
-        const int r = idx / n, c = idx % n;
-        A[r * m + c] = (r <= c + 1) ? Hs[(size_t)c * (m + 1) + r] : make_double2(0.0, 0.0);
-    }
-    for (int c = lane; c < n; c += 32) {
-        Z0[c] = make_double2(c == 0 ? 1.0 : 0.0, 0.0);
-        Zl[c] = make_double2(c == n - 1 ? 1.0 : 0.0, 0.0);
-    }
+    __shared__ double s_nrm[SC_THREADS / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool gen = warp == SC_UPD / 32;
+    int fail = (n < 1 || n > 60) ? 1 : 0;
     double nrm = 0.0;
-    for (int idx = lane; idx < n * n; idx += 32) nrm = fmax(nrm, cabs_s(A[(idx / n) * m + idx % n]));
+    if (!fail) {
+        for (int idx = tid; idx < n * n; idx += SC_THREADS) {
+            const int r = idx / n, c = idx % n;
+            const double2 h = (r <= c + 1) ? Hs[(size_t)c * (m + 1) + r] : make_double2(0.0, 0.0);
+            A[r * ld + c] = h;
+            nrm = fmax(nrm, fabs(h.x) + fabs(h.y));
+        }
+        for (int c = tid; c < n; c += SC_THREADS) {
+            A[n * ld + c] = make_double2(c == 0 ? 1.0 : 0.0, 0.0);
+            A[(n + 1) * ld + c] = make_double2(c == n - 1 ? 1.0 : 0.0, 0.0);
+        }
+    }
     for (int o = 16; o > 0; o >>= 1) nrm = fmax(nrm, __shfl_xor_sync(0xffffffffu, nrm, o));
-    __syncwarp();
-    int hi = n - 1, its = 0, sweeps = 0, fail = (n < 1 || n > 64) ? 1 : 0;
-    while (!fail && hi > 0) {
-        if (lane == 0) {
-            int l = hi;
-            while (l > 0) {
-                const double sub = cabs_s(A[l * m + l - 1]);
-                double d = cabs_s(A[(l - 1) * m + l - 1]) + cabs_s(A[l * m + l]);
-                if (d == 0.0) d = nrm;
-                if (sub <= DBL_EPSILON * d) break;
-                --l;
+    if (lane == 0) s_nrm[warp] = nrm;
+    __syncthreads();
+    for (int w = 0; w < SC_THREADS / 32; ++w) nrm = fmax(nrm, s_nrm[w]);
+
+    // rotation k from (a, b) = (A[k][k], A[k+1][k]), by the generator warp
+    auto generate = [&](int k, double2 a, double2 b) {
+        // lane 0: |a|^2, 1: |b|^2, 2: re(a conj b), 3: im(a conj b)
+        const double p = lane == 1 ? b.x : (lane == 3 ? a.y : a.x), q = lane == 0 ? a.x : b.x;
+        const double r = lane == 1 ? b.y : (lane == 3 ? -a.x : a.y), t = lane == 0 ? a.y : b.y;
+        const double d = fma(r, t, p * q);
+        const double na2 = __shfl_sync(0xffffffffu, d, 0), nb2 = __shfl_sync(0xffffffffu, d, 1);
+        const double h2 = na2 + nb2;
+        if (na2 > 1e-280 && h2 < 1e280) {
+            const double rs = rsqrt_nr(lane == 0 ? na2 : h2);
+            const double pr = __shfl_sync(0xffffffffu, rs, 0) * __shfl_sync(0xffffffffu, rs, 1);  // 1 / (|a| h)
+            const double v = d * pr;  // lane 0: |a| / h, 2 and 3: a conj(b) / (|a| h)
+            if (lane == 0) gc[k] = v;
+            if (lane == 2) gs[k].x = v;
+            if (lane == 3) gs[k].y = v;
+        } else if (lane == 0) {
+            const double na = cabs_s(a), nb = cabs_s(b);
+            double c;
+            double2 sn;
+            if (nb == 0.0) {
+                c = 1.0;
+                sn = make_double2(0.0, 0.0);
+            } else if (na == 0.0) {
+                c = 0.0;
+                sn = make_double2(b.x / nb, -b.y / nb);
+            } else {
+                const double h = hypot(na, nb);
+                c = na / h;
+                const double2 ua = make_double2(a.x / na, a.y / na);
+                sn = cmul(ua, make_double2(b.x / h, -b.y / h));
             }
-            if (l > 0) A[l * m + l - 1] = make_double2(0.0, 0.0);
-            s_l = l;
-            if (l != hi) {
-                // Wilkinson shift from the trailing 2×2 block, exceptional every 10 sweeps
-                const double2 p = A[(hi - 1) * m + hi - 1], q = A[(hi - 1) * m + hi];
-                const double2 r = A[hi * m + hi - 1], t = A[hi * m + hi];
-                double2 mu = t;
-                if (its > 0 && its % 10 == 0) {
-                    mu.x += 0.75 * cabs_s(r);
-                } else {
-                    const double2 d = make_double2(0.5 * (p.x - t.x), 0.5 * (p.y - t.y));
-                    const double2 qr = cmul(q, r);
-                    const double2 disc = csqrt_s(cadd(cmul(d, d), qr));
-                    const double2 den1 = cadd(d, disc), den2 = csub(d, disc);
-                    const double2 den = cabs_s(den1) >= cabs_s(den2) ? den1 : den2;
-                    if (cabs_s(den) > 0.0) mu = csub(t, cdiv(qr, den));
-                }
-                s_mu = mu;
-            }
+            gc[k] = c;
+            gs[k] = sn;
         }
         __syncwarp();
+    };
+    // component cmp (x'.re, x'.im, y'.re, y'.im) of the rotated pair:
+    //   left  x' = c x + s y,        y' = c y - conj(s) x
+    //   right x' = c x + conj(s) y,  y' = c y - s x
+    auto rotated = [&](int cmp, bool left, double c, double2 sn, double2 x, double2 y) {
+        const bool first = cmp < 2, im = cmp & 1;
+        const double2 o = first ? x : y, e = first ? y : x;
+        const double sx = first ? sn.x : -sn.x;
+        const double sy = (im == left) ? sn.y : -sn.y;
+        return fma(sy, im ? e.x : e.y, fma(sx, im ? e.y : e.x, c * (im ? o.y : o.x)));
+    };
+
+    int hi = n - 1, its = 0, sweeps = 0;
+    while (!fail && hi > 0) {
+        if (warp == 0) {
+            // the largest l with a negligible subdiagonal A[l][l-1], l <= hi (0: none)
+            int best = 0;
+            for (int k = lane + 1; k <= hi; k += 32) {
+                const double2 u = A[k * ld + k - 1], d0 = A[(k - 1) * ld + k - 1], d1 = A[k * ld + k];
+                double d = (fabs(d0.x) + fabs(d0.y)) + (fabs(d1.x) + fabs(d1.y));
+                if (d == 0.0) d = nrm;
+                if (fabs(u.x) + fabs(u.y) <= DBL_EPSILON * d) best = k;
+            }
+            best = __reduce_max_sync(0xffffffffu, best);
+            if (lane == 0) {
+                if (best > 0) A[best * ld + best - 1] = make_double2(0.0, 0.0);
+                s_l = best;
+            }
+        } else if (gen && lane == 0) {
+            // Wilkinson shift from the trailing 2×2 block, exceptional every 10 sweeps
+            const double2 p = A[(hi - 1) * ld + hi - 1], q = A[(hi - 1) * ld + hi];
+            const double2 r = A[hi * ld + hi - 1], t = A[hi * ld + hi];
+            double2 mu = t;
+            if (its > 0 && its % 10 == 0) {
+                mu.x += 0.75 * cabs_s(r);
+            } else {
+                const double2 d = make_double2(0.5 * (p.x - t.x), 0.5 * (p.y - t.y));
+                const double2 qr = cmul(q, r);
+                const double2 disc = csqrt_s(cadd(cmul(d, d), qr));
+                const double2 den1 = cadd(d, disc), den2 = csub(d, disc);
+                const double2 den = cabs2(den1) >= cabs2(den2) ? den1 : den2;
+                if (den.x != 0.0 || den.y != 0.0) mu = csub(t, cdiv(qr, den));
+            }
+            s_mu = mu;
+        }
+        __syncthreads();
         const int l = s_l;
         if (l == hi) {
             --hi;
             its = 0;
-            __syncwarp();
+            __syncthreads();  // s_l read before it is rewritten
             continue;
         }
         if (++sweeps > 30 * n) {
@@ -121,75 +206,67 @@ __global__ void __launch_bounds__(32) k_schur(const double2* Hall, int m, const 
         }
         ++its;
         const double2 mu = s_mu;
-        for (int k = l + lane; k <= hi; k += 32) A[k * m + k] = csub(A[k * m + k], mu);
-        __syncwarp();
-        // left: G_k zeroes A[k+1][k] of the active block; applied to whole rows k, k+1
-        for (int k = l; k < hi; ++k) {
-            if (lane == 0) {
-                const double2 a = A[k * m + k], b = A[(k + 1) * m + k];
-                const double na = cabs_s(a), nb = cabs_s(b);
-                double c;
-                double2 sn;
-                if (nb == 0.0) {
-                    c = 1.0;
-                    sn = make_double2(0.0, 0.0);
-                } else if (na == 0.0) {
-                    c = 0.0;
-                    sn = make_double2(b.x / nb, -b.y / nb);
-                } else {
-                    const double h = hypot(na, nb);
-                    c = na / h;
-                    const double2 ua = make_double2(a.x / na, a.y / na);
-                    sn = cmul(ua, make_double2(b.x / h, -b.y / h));
+        for (int k = l + tid; k <= hi; k += SC_THREADS) A[k * ld + k] = csub(A[k * ld + k], mu);
+        __syncthreads();
+        if (gen) generate(l, A[l * ld + l], A[(l + 1) * ld + l]);
+        __syncthreads();
+        // step k: left rotation k, and right rotation k-2 on the rows it has left behind
+        for (int k = l; k <= hi + 1; ++k) {
+            const bool dol = k < hi, dor = k - 2 >= l;
+            if (gen) {
+                if (k + 1 < hi) {
+                    // column k+1 of left rotation k, then rotation k+1
+                    double2* px = A + k * ld + k + 1;
+                    double2* py = px + ld;
+                    const double2 x = *px, y = *py;
+                    const double v = rotated(lane & 3, true, gc[k], gs[k], x, y);
+                    const double2 a = make_double2(__shfl_sync(0xffffffffu, v, 2), __shfl_sync(0xffffffffu, v, 3));
+                    if (lane < 4) (lane < 2 ? reinterpret_cast<double*>(px) : reinterpret_cast<double*>(py))[lane & 1] = v;
+                    generate(k + 1, a, A[(k + 2) * ld + k + 1]);
                 }
-                gc[k - l] = c;
-                gs[k - l] = sn;
+            } else {
+                // left: columns k .. n-1 (but k+1 where the generator has it); right: rows 0 .. k-1, Z's two
+                const int nl = dol ? n - k : 0, rows = min(k, hi + 1), nrt = dor ? rows + 2 : 0;
+                for (int it = tid >> 2; it < nl + nrt; it += SC_UPD / 4) {
+                    const bool left = it < nl;
+                    const int kk = left ? k : k - 2;
+                    double2 *px, *py;
+                    if (left) {
+                        px = A + k * ld + k + it;
+                        py = px + ld;
+                    } else {
+                        const int row = it - nl < rows ? it - nl : n + (it - nl - rows);
+                        px = A + row * ld + kk;
+                        py = px + 1;
+                    }
+                    const bool skip = left && it == 1 && k + 1 < hi;
+                    const unsigned quad = 0xFu << (lane & ~3);
+                    const double2 x = *px, y = *py;
+                    const double v = rotated(tid & 3, left, gc[kk], gs[kk], x, y);
+                    __syncwarp(quad);  // the pair's four lanes have read it
+                    if (!skip) (tid & 2 ? reinterpret_cast<double*>(py) : reinterpret_cast<double*>(px))[tid & 1] = v;
+                }
             }
-            __syncwarp();
-            const double c = gc[k - l];
-            const double2 sn = gs[k - l];
-            for (int j = k + lane; j < n; j += 32) {
-                const double2 x = A[k * m + j], y = A[(k + 1) * m + j];
-                A[k * m + j] = cadd(make_double2(c * x.x, c * x.y), cmul(sn, y));
-                A[(k + 1) * m + j] = csub(make_double2(c * y.x, c * y.y), cmul(conj_s(sn), x));
-            }
-            __syncwarp();
+            __syncthreads();
         }
-        // right: columns k, k+1 of every row above the active block's subdiagonal, and of Z
-        for (int k = l; k < hi; ++k) {
-            const double c = gc[k - l];
-            const double2 sn = gs[k - l];
-            const int rmax = min(k + 1, hi);
-            for (int i = lane; i <= rmax; i += 32) {
-                const double2 x = A[i * m + k], y = A[i * m + k + 1];
-                A[i * m + k] = cadd(make_double2(c * x.x, c * x.y), cmul(conj_s(sn), y));
-                A[i * m + k + 1] = csub(make_double2(c * y.x, c * y.y), cmul(sn, x));
-            }
-            if (lane < 2) {
-                double2* Zr = lane == 0 ? Z0 : Zl;
-                const double2 x = Zr[k], y = Zr[k + 1];
-                Zr[k] = cadd(make_double2(c * x.x, c * x.y), cmul(conj_s(sn), y));
-                Zr[k + 1] = csub(make_double2(c * y.x, c * y.y), cmul(sn, x));
-            }
-            __syncwarp();
-        }
-        for (int k = l + lane; k <= hi; k += 32) A[k * m + k] = cadd(A[k * m + k], mu);
-        __syncwarp();
+        for (int k = l + tid; k <= hi; k += SC_THREADS) A[k * ld + k] = cadd(A[k * ld + k], mu);
+        __syncthreads();
     }
+    const double2 *Z0 = A + n * ld, *Zl = A + (n + 1) * ld;
     double2* T = Tall + (size_t)s * m * m;
     const double beta = beta_all[s];
     if (!fail) {
-        for (int idx = lane; idx < n * n; idx += 32) {
+        for (int idx = tid; idx < n * n; idx += SC_THREADS) {
             const int r = idx / n, c = idx % n;
-            T[r * m + c] = c >= r ? A[r * m + c] : make_double2(0.0, 0.0);
+            T[r * m + c] = c >= r ? A[r * ld + c] : make_double2(0.0, 0.0);
         }
-        for (int i = lane; i < n; i += 32) {
+        for (int i = tid; i < n; i += SC_THREADS) {
             const double2 z0 = Z0[i];
             Call[(size_t)s * m + i] = make_double2(beta * z0.x, -beta * z0.y);
             Qall[(size_t)s * m + i] = Zl[i];
         }
     }
-    if (lane == 0) ok_all[s] = fail ? 0 : 1;
+    if (tid == 0) ok_all[s] = fail ? 0 : 1;
 }
 
 // 8 nodes per square, 4 squares per warp, SE_WARPS warps per CTA; x_j of every
@@ -349,9 +426,9 @@ __global__ void __launch_bounds__(SE_WARPS * 32) k_eval_schur(ShiftTable st, Lev
 void schur_shifts(const double2* H, int m, const int* meff, const double* beta, int s0, int count, double2* T,
                   double2* C, double2* Q, int* ok, cudaStream_t st) {
     if (count <= 0) return;
-    const size_t sm = ((size_t)m * m + 2 * (size_t)m) * sizeof(double2);
+    const size_t sm = (size_t)(m + 2) * (m | 1) * sizeof(double2);
     SIM_CUDA(cudaFuncSetAttribute(k_schur, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    k_schur<<<count, 32, sm, st>>>(H, m, meff, beta, s0, T, C, Q, ok);
+    k_schur<<<count, SC_THREADS, sm, st>>>(H, m, meff, beta, s0, T, C, Q, ok);
     SIM_LAUNCH_CHECK();
 }
 
