@@ -217,7 +217,9 @@ void upload_pencil(DeviceArena& ar, cudaStream_t st, Pencil& P, const std::vecto
     P.nb = (int)((n + P.T - 1) / P.T);
     P.b_kind = b_kind;
     // couplings to the inner neighbour, column-compressed per block
-    P.mid = P.nb / 2;
+    // From both ends, but for short chains: two launches of half the steps cost more
+    // than one chain of fewer than 8 blocks.
+    P.mid = P.nb < 8 ? P.nb - 1 : P.nb / 2;
     const int T = P.T, nb = P.nb, mid = P.mid;
     std::vector<int32_t> up_ptr((size_t)nb * (T + 1), 0), up_row, up_idx;
     {
