@@ -49,6 +49,7 @@
 
 #include "internal.h"
 #include "factor_cluster.h"
+#include "fp64.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -79,35 +80,6 @@ __device__ __forceinline__ float2 crecip(float2 a) {
     r = fmaf(r, fmaf(-d, r, 1.0f), r) * s;  // one Newton step
     return make_float2(x * r, -y * r);
 }
-// Seven FP64 operations (a warp's FP64 instruction takes 64 clocks of its scheduler):
-// the scalings by powers of two are exponent arithmetic, and 1/d is one third-order
-// Newton step, r + r (e + e^2) with e = 1 - d r, from an FP32 reciprocal (e^3 < 2^-66).
-__device__ __forceinline__ double2 crecip(double2 a) {
-    const uint32_t hx = (uint32_t)__double2hiint(a.x), hy = (uint32_t)__double2hiint(a.y);
-    const int ex = (int)((hx >> 20) & 2047u), ey = (int)((hy >> 20) & 2047u), e = max(ex, ey);
-    if (e < 64 || e > 1983) {  // far out: by division
-        const double s = e < 64 ? 0x1p+960 : 0x1p-960;
-        const double x = a.x * s, y = a.y * s, d = x * x + y * y;
-        return make_double2(x / d * s, -(y / d) * s);
-    }
-    const int k = 1023 - e;  // a 2^k has its larger part in [1, 2)
-    const double x = ex + k > 0 ? __hiloint2double((int)(hx + ((uint32_t)k << 20)), __double2loint(a.x)) : 0.0;
-    const double y = ey + k > 0 ? __hiloint2double((int)(hy + ((uint32_t)k << 20)), __double2loint(a.y)) : 0.0;
-    const double d = fma(x, x, y * y);  // [1, 8)
-    // d to FP32 and its reciprocal back to FP64 by exponent arithmetic
-    const uint32_t hd = (uint32_t)__double2hiint(d), ld = (uint32_t)__double2loint(d);
-    const float f = __uint_as_float(((((hd >> 20) & 2047u) - 1023u + 127u) << 23) | ((hd & 0xFFFFFu) << 3) | (ld >> 29));
-    const uint32_t g = __float_as_uint(1.0f / f);
-    const double r0 = __hiloint2double((int)((((g >> 23) - 127u + 1023u) << 20) | ((g & 0x7FFFFFu) >> 3)), (int)(g << 29));
-    const double t = fma(-d, r0, 1.0);
-    const double r = fma(r0, fma(t, t, t), r0);
-    const double ix = x * r, iy = -(y * r);
-    const uint32_t hix = (uint32_t)__double2hiint(ix), hiy = (uint32_t)__double2hiint(iy);
-    const int eix = (int)((hix >> 20) & 2047u) + k, eiy = (int)((hiy >> 20) & 2047u) + k;
-    return make_double2(eix > 0 ? __hiloint2double((int)(hix + ((uint32_t)k << 20)), __double2loint(ix)) : 0.0,
-                        eiy > 0 ? __hiloint2double((int)(hiy + ((uint32_t)k << 20)), __double2loint(iy)) : 0.0);
-}
-
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 __device__ __forceinline__ void bar_panel(int threads) {

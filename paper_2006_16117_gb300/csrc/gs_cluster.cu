@@ -1,22 +1,34 @@
-// Batched classical Gram–Schmidt, applied twice (CGS2) or with the
+// Batched classical Gram–Schmidt, applied twice (CGS2), once, or with the
 // Daniel–Gragg–Kaufman–Stewart test for the second pass, in one launch: the
 // orthogonalisation of w against the cnt basis vectors of its job, the norm,
-// the Arnoldi breakdown test and the normalisation (Sec. 3.1's Arnoldi
-// process; the inner FGMRES uses the same step).
+// the Arnoldi breakdown test, the normalisation and the FGMRES step (Sec. 3.1's
+// Arnoldi process; the inner FGMRES uses the same step).
 //
-// One thread-block cluster per job.  CTA q of the cluster owns rows
-// [q*256*E, (q+1)*256*E) and keeps its piece of w in shared memory (E values
-// per thread, two CTAs per SM), so w is read once and written once; every
-// pass over the basis is one streaming read.  The complex multiply-adds are
-// FP64 and on this GPU the FP64 pipe, not HBM, bounds the step; the update
-// streams all basis vectors per element so that many loads are in flight.  The dot products and norms are summed in the CTA
-// (shuffles, then shared memory) and across the cluster by reading each peer
-// CTA's partials through distributed shared memory, in rank order — every
-// CTA forms the same totals and takes the same decisions.  The only waits are
-// the hardware cluster barriers.
+// One thread-block cluster per job.  CTA q of the cluster owns E·NT consecutive
+// rows and keeps its piece of w in shared memory, so w is read once and written
+// once; every pass over the basis is one streaming read.  The complex
+// multiply-adds are FP64 and on this GPU the FP64 pipe (two lanes a clock per
+// SM), not HBM, bounds the step: the cluster is as large as the number of jobs
+// leaves room for, and the sums over lanes are made for eight vectors at a time.
+// The partial sums are added in the CTA and across the cluster by reading each
+// peer CTA's through distributed shared memory, in rank order — every CTA forms
+// the same totals and takes the same decisions.  The only waits are the hardware
+// cluster barriers; the partial sums alternate between two buffers, so that a
+// pass needs one of them.
+//
+// gram_schmidt() takes this form or the grid kernels (gs_grid.cu), whichever an
+// estimate says is faster: this one cannot use more than 16 SMs a job.  n up to
+// 3,600 (six pencils, one to three jobs a call): 52 -> 23 us a call, the Givens
+// step's own kernel (7 us) and a copy of w included.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+#include <atomic>
+#include <cmath>
+#include <limits>
+
 #include "gs.h"
+#include "gs_finish.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -24,225 +36,227 @@ namespace sim {
 
 namespace {
 
-constexpr int GC_THREADS = 256;
-constexpr int GC_WARPS = GC_THREADS / 32;
-constexpr int GC_MAXV = 64;  // basis vectors per call (cnt), plus two norm slots below
+constexpr int GC_MAXT = 256;
+constexpr int GC_WARPS = GC_MAXT / 32;
+constexpr int GC_MAXV = 64;   // basis vectors per call (cnt)
+constexpr int GC_MAXE = 20;   // rows per thread: two CTAs' pieces of w fit an SM
 
 struct GcShared {
-    double2 red[GC_WARPS][GC_MAXV + 2];  // per-warp sums
-    double2 part[GC_MAXV + 2];           // this CTA's sums (read by the peers)
-    double2 tot[GC_MAXV + 2];            // cluster totals
-    double2 h1[GC_MAXV];                 // first-pass coefficients
+    double red[GC_WARPS][2 * GC_MAXV + 4];  // per-warp sums, (re, im) per value
+    double part[2][2 * GC_MAXV + 4];        // this CTA's sums (read by the peers)
+    double2 tot[GC_MAXV + 2];               // cluster totals
+    double2 h1[GC_MAXV];                    // coefficients so far
     double fro[GC_WARPS];
 };
 
-// Sum V values (each thread's contribution in v(i), i < V) over the CTA and
-// the cluster; the totals land in S.tot[0..V).
-template <class F>
-__device__ __forceinline__ void cluster_sum(cg::cluster_group& cl, GcShared& S, int V, F v) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = 0; i < V; ++i) {
-        const double2 x = warp_sum(v(i));
-        if (lane == 0) S.red[warp][i] = x;
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < V; i += GC_THREADS) {
-        double2 s = S.red[0][i];
-        for (int w = 1; w < GC_WARPS; ++w) s = cadd(s, S.red[w][i]);
-        S.part[i] = s;
-    }
-    cl.sync();  // every CTA's partials are written
-    const int nr = (int)cl.num_blocks();
-    for (int i = threadIdx.x; i < V; i += GC_THREADS) {
-        double2 s = make_double2(0.0, 0.0);
-        for (int r = 0; r < nr; ++r) s = cadd(s, cl.map_shared_rank(S.part, r)[i]);
-        S.tot[i] = s;
-    }
-    cl.sync();  // the peers have read our partials; the totals are visible
-}
-
-template <int E>
-__global__ void __launch_bounds__(GC_THREADS, 2) k_gs_cluster(GSArgs a) {
+__global__ void __launch_bounds__(GC_MAXT, 2) k_gs_cluster(GSArgs a, int E) {
     cg::cluster_group cl = cg::this_cluster();
     const int Cg = (int)cl.num_blocks();
     const int q = (int)cl.block_rank();
     const int job = a.active[blockIdx.x / Cg];
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, NT = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = NT >> 5;
     __shared__ GcShared S;
-    extern __shared__ double2 wsm[];  // [E][GC_THREADS]: this CTA's rows of w
+    extern __shared__ double2 wsm[];  // [E][NT]: this CTA's rows of w
     const double2* B = a.basis + (size_t)job * a.bstride;
     double2* w = a.w + (size_t)job * a.wstride;
-    const int64_t base = (int64_t)q * GC_THREADS * E + tid;
+    const double2* src = a.src ? a.src + (size_t)job * a.sstride : w;
+    const int64_t base = (int64_t)q * NT * E + tid;
     const int cnt = a.cnt;
+    // rows of this thread: e < Er are below n
+    const int Er = base < a.n ? (int)min((int64_t)E, (a.n - base + NT - 1) / NT) : 0;
 
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int64_t r = base + (int64_t)e * GC_THREADS;
-        wsm[e * GC_THREADS + tid] = r < a.n ? w[r] : make_double2(0.0, 0.0);
-    }
+#pragma unroll 4
+    for (int e = 0; e < E; ++e)
+        wsm[e * NT + tid] = e < Er ? src[base + (int64_t)e * NT] : make_double2(0.0, 0.0);
     auto sq = [&]() {
         double s = 0.0;
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            const double2 v = wsm[e * GC_THREADS + tid];
-            s += v.x * v.x + v.y * v.y;
+        for (int e = 0; e < Er; ++e) {
+            const double2 v = wsm[e * NT + tid];
+            s = fma(v.x, v.x, fma(v.y, v.y, s));
         }
-        return make_double2(s, 0.0);
+        return s;
+    };
+    int buf = 0;
+    // totals of V values whose warps' sums are in S.red
+    auto totals = [&](int V) {
+        __syncthreads();
+        for (int t = tid; t < 2 * V; t += NT) {
+            double s = S.red[0][t];
+            for (int i = 1; i < nw; ++i) s += S.red[i][t];
+            S.part[buf][t] = s;
+        }
+        cl.sync();  // every CTA's sums are written
+        for (int t = tid; t < 2 * V; t += NT) {
+            double s = 0.0;
+            for (int r = 0; r < Cg; ++r) s += cl.map_shared_rank(&S.part[buf][0], r)[t];
+            reinterpret_cast<double*>(S.tot)[t] = s;
+        }
+        buf ^= 1;  // a peer may still read these: the next sums go to the other buffer
+        __syncthreads();
+    };
+    auto put_norm = [&](int at, double v) {
+        v = warp_sum(v);
+        if (lane == 0) {
+            S.red[warp][2 * at] = v;
+            S.red[warp][2 * at + 1] = 0.0;
+        }
     };
     // h_i = conj(q_i) . w for i < cnt (and ||w||^2 in slot cnt if `with_norm`)
     auto dots = [&](bool with_norm) {
-        cluster_sum(cl, S, cnt + (with_norm ? 1 : 0), [&](int i) -> double2 {
-            if (i == cnt) return sq();
-            const double2* qv = B + (size_t)i * a.n;
-            double2 acc = make_double2(0.0, 0.0), acc2 = make_double2(0.0, 0.0);
-#pragma unroll 10
-            for (int e = 0; e < E; ++e) {
-                const int64_t r = base + (int64_t)e * GC_THREADS;
-                if (r < a.n) {
-                    const double2 x = qv[r];
-                    const double2 v = wsm[e * GC_THREADS + tid];
-                    double2& c = (e & 1) ? acc2 : acc;
-                    c.x = fma(x.x, v.x, c.x);
-                    c.x = fma(x.y, v.y, c.x);
-                    c.y = fma(x.x, v.y, c.y);
-                    c.y = fma(-x.y, v.x, c.y);
-                }
+        for_groups(cnt, [&](auto tag, int i0) {
+            constexpr int G = decltype(tag)::value;
+            double2 acc[G];
+#pragma unroll
+            for (int g = 0; g < G; ++g) acc[g] = make_double2(0.0, 0.0);
+            const double2* qv = B + (size_t)i0 * a.n + base;
+#pragma unroll 2
+            for (int e = 0; e < Er; ++e) {
+                const double2 v = wsm[e * NT + tid];
+#pragma unroll
+                for (int g = 0; g < G; ++g) conj_mac(acc[g], qv[(size_t)g * a.n + (int64_t)e * NT], v);
             }
-            return cadd(acc, acc2);
+            const double2 s = warp_sum_group<G>(acc);
+            if ((lane & (32 / G - 1)) == 0) {
+                const int i = i0 + lane / (32 / G);
+                S.red[warp][2 * i] = s.x;
+                S.red[warp][2 * i + 1] = s.y;
+            }
         });
+        if (with_norm) put_norm(cnt, sq());
+        totals(cnt + (with_norm ? 1 : 0));
     };
     // w -= sum_i q_i h_i with h in S.tot[0..cnt): per element, all i
     auto update = [&]() {
-#pragma unroll 2
-        for (int e = 0; e < E; ++e) {
-            const int64_t r = base + (int64_t)e * GC_THREADS;
-            if (r >= a.n) continue;
-            double2 v = wsm[e * GC_THREADS + tid];
-            const double2* qv = B + r;
-            for (int i = 0; i < cnt; ++i) {
-                const double2 x = qv[(size_t)i * a.n];
-                const double2 hi = S.tot[i];
-                v.x = fma(-x.x, hi.x, v.x);
-                v.x = fma(x.y, hi.y, v.x);
-                v.y = fma(-x.x, hi.y, v.y);
-                v.y = fma(-x.y, hi.x, v.y);
-            }
-            wsm[e * GC_THREADS + tid] = v;
+        for (int e = 0; e < Er; ++e) {
+            double2 v = wsm[e * NT + tid];
+            const double2* qv = B + base + (int64_t)e * NT;
+#pragma unroll 8
+            for (int i = 0; i < cnt; ++i) sub_mac(v, qv[(size_t)i * a.n], S.tot[i]);
+            wsm[e * NT + tid] = v;
         }
+    };
+    auto norm2 = [&]() {
+        put_norm(0, sq());
+        totals(1);
+        return S.tot[0].x;
     };
 
     double nn = 0.0;  // ||w||^2 after the last pass
     if (cnt == 0) {
-        cluster_sum(cl, S, 1, [&](int) { return sq(); });
-        nn = S.tot[0].x;
+        nn = norm2();
     } else {
         dots(a.dgks != 0);
         const double nb = a.dgks ? S.tot[cnt].x : 0.0;  // ||w||^2 before the first pass
-        for (int i = tid; i < cnt; i += GC_THREADS) S.h1[i] = S.tot[i];
+        for (int i = tid; i < cnt; i += NT) S.h1[i] = S.tot[i];
         update();
-        // the barriers in cluster_sum order S.h1's writes before its reads below
+        // the barriers in totals order S.h1's writes before its reads below
         bool second = !a.single;
         if (a.dgks || a.single) {
-            cluster_sum(cl, S, 1, [&](int) { return sq(); });
-            nn = S.tot[0].x;
+            nn = norm2();
             if (a.dgks && !a.single) second = !(nn > 0.5 * nb);
         }
         if (second) {
             dots(false);
             // S.tot now holds the second-pass coefficients
-            for (int i = tid; i < cnt; i += GC_THREADS) S.h1[i] = cadd(S.h1[i], S.tot[i]);
+            for (int i = tid; i < cnt; i += NT) S.h1[i] = cadd(S.h1[i], S.tot[i]);
             update();
-            cluster_sum(cl, S, 1, [&](int) { return sq(); });
-            nn = S.tot[0].x;
+            nn = norm2();
         }
         __syncthreads();  // S.h1 complete
     }
     const double hn = sqrt(nn);
     bool broken = !(hn > 0.0);
     if (a.Hfull) {
-        // ||H(0:j, 0:j)||_F, column j being the coefficients just computed
-        const double2* H = a.Hfull + (size_t)job * a.Hstride;
-        const int jj = a.j, rows = a.j + 1;
-        double f = 0.0;
-        for (int idx = tid; idx < jj * rows; idx += GC_THREADS) f += cabs2(H[(size_t)(idx / rows) * a.Hld + idx % rows]);
-        for (int r = tid; r < rows; r += GC_THREADS) f += cabs2(S.h1[r]);
-        f = warp_sum(f);
-        if ((tid & 31) == 0) S.fro[tid >> 5] = f;
-        __syncthreads();
-        double ft = 0.0;
-        for (int w2 = 0; w2 < GC_WARPS; ++w2) ft += S.fro[w2];
-        if (hn <= a.btol * sqrt(ft)) broken = true;
+        const double f = hess_frobenius2(a, job, S.h1, [&](double v) {
+            v = warp_sum(v);
+            if (lane == 0) S.fro[warp] = v;
+            __syncthreads();
+            double t = 0.0;
+            for (int i = 0; i < nw; ++i) t += S.fro[i];
+            return t;
+        });
+        if (hn <= a.btol * sqrt(f)) broken = true;
     }
-    if (q == 0) {
-        double2* hc = a.hcol + (size_t)job * a.hstride;
-        for (int i = tid; i < cnt; i += GC_THREADS) hc[i] = S.h1[i];
-        if (tid == 0) {
-            hc[cnt] = make_double2((broken && a.Hfull) ? 0.0 : hn, 0.0);
-            if (broken && a.meff) a.meff[job] = a.j + 1;
-            if (broken && a.istat) a.istat[job * IS_N + IS_BROKEN] = 1;
-        }
-    }
+    if (q == 0 && warp == 0) gs_finish(a, job, S.h1, hn, broken);
     const double inv = broken ? 1.0 : 1.0 / hn;
-#pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int64_t r = base + (int64_t)e * GC_THREADS;
-        const double2 v = wsm[e * GC_THREADS + tid];
-        if (r < a.n) w[r] = broken ? v : cscale(v, inv);
+#pragma unroll 4
+    for (int e = 0; e < Er; ++e) {
+        const double2 v = wsm[e * NT + tid];
+        w[base + (int64_t)e * NT] = broken ? v : cscale(v, inv);
     }
+    cl.sync();  // no CTA leaves while a peer reads its sums
 }
 
-template <int E>
-void launch_gc(const GSArgs& a, int nactive, int Cg, cudaStream_t st) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(nactive * Cg);
-    cfg.blockDim = dim3(GC_THREADS);
-    cfg.dynamicSmemBytes = (size_t)E * GC_THREADS * sizeof(double2);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = Cg;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    static bool smem_set = false;  // per instantiation
-    if (!smem_set) {
-        SIM_CUDA(cudaFuncSetAttribute(k_gs_cluster<E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)cfg.dynamicSmemBytes));
-        smem_set = true;
-    }
-    SIM_CUDA(cudaLaunchKernelEx(&cfg, k_gs_cluster<E>, a));
-    SIM_LAUNCH_CHECK();
+struct ClusterShape {
+    int Cg = 0, E = 0, NT = 256;
+    double cost = std::numeric_limits<double>::infinity();
+};
+
+// Cluster size and rows per thread: as many CTAs a job as the GPU holds at two per
+// SM, at most 16 (the hardware's limit) and no more than there are rows for.  The
+// estimate charges each SM's FP64 instructions 64 clocks a warp on its four
+// schedulers and 2,500 clocks a pass for the sums across the cluster.
+ClusterShape cluster_shape(int64_t n, int cnt, int passes, int nactive) {
+    ClusterShape s;
+    s.NT = n <= 128 * 16 ? 128 : 256;
+    const int need = cdiv_up(n, (int64_t)s.NT * GC_MAXE);
+    if (need > 16 || cnt > GC_MAXV) return s;
+    const int room = std::max(1, 2 * 152 / std::max(1, nactive));
+    s.Cg = std::max(need, std::min(std::min(16, room), cdiv_up(n, s.NT)));
+    s.E = cdiv_up(n, (int64_t)s.NT * s.Cg);
+    s.Cg = cdiv_up(n, (int64_t)s.NT * s.E);
+    const double per_warp = s.E * (4.0 * cnt * passes + 6.0) + 1.2 * cnt * passes + 20.0;
+    const double per_sm = std::ceil((double)nactive * s.Cg / 152.0);
+    s.cost = per_warp * 64.0 * (s.NT / 128) * per_sm + (passes + 1.0) * 2500.0;
+    return s;
 }
 
 }  // namespace
 
-bool gs_cluster(const GSArgs& a, int nactive, cudaStream_t st) {
-    if (nactive <= 0) return true;
-    if (a.cnt < 0 || a.cnt > GC_MAXV) return false;
-    static const int Es[] = {4, 8, 12, 16, 20};
-    int E = 0;
-    for (int e : Es)
-        if ((int64_t)GC_THREADS * e * 8 >= a.n) {
-            E = e;
-            break;
-        }
-    if (E == 0) return false;
-    const int Cg = cdiv_up(a.n, (int64_t)GC_THREADS * E);
+double gs_cluster_cost(int64_t n, int cnt, int passes, int nactive) {
+    return cluster_shape(n, cnt, passes, nactive).cost;
+}
+
+void gs_cluster(const GSArgs& a, int nactive, cudaStream_t st) {
+    const int passes = a.cnt == 0 ? 0 : (a.dgks || a.single ? 2 : 4);
+    const ClusterShape s = cluster_shape(a.n, a.cnt, passes, nactive);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nactive * s.Cg);
+    cfg.blockDim = dim3(s.NT);
+    cfg.dynamicSmemBytes = (size_t)s.E * s.NT * sizeof(double2);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = s.Cg;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    static std::atomic<uint64_t> ready{0};  // devices whose kernel attributes are set
+    int dev = 0;
+    SIM_CUDA(cudaGetDevice(&dev));
+    if (dev > 63 || !(ready.load() >> dev & 1)) {
+        SIM_CUDA(cudaFuncSetAttribute(k_gs_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      GC_MAXE * GC_MAXT * (int)sizeof(double2)));
+        SIM_CUDA(cudaFuncSetAttribute(k_gs_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        if (dev <= 63) ready.fetch_or(1ull << dev);
+    }
+    SIM_CUDA(cudaLaunchKernelEx(&cfg, k_gs_cluster, a, s.E));
+    SIM_LAUNCH_CHECK();
+}
+
+void gram_schmidt(const GSArgs& a, int nactive, cudaStream_t st) {
+    if (nactive <= 0) return;
+    const int passes = a.cnt == 0 ? 0 : (a.dgks || a.single ? 2 : 4);
     // algorithmic bytes: w read and written once; the basis streamed once per
     // pass (two passes with the selective test in its usual outcome, four for CGS2)
-    const double passes = a.cnt == 0 ? 0.0 : ((a.dgks || a.single) ? 2.0 : 4.0);
     kprof_begin("gram_schmidt", st);
-    switch (E) {
-        case 4: launch_gc<4>(a, nactive, Cg, st); break;
-        case 8: launch_gc<8>(a, nactive, Cg, st); break;
-        case 12: launch_gc<12>(a, nactive, Cg, st); break;
-        case 16: launch_gc<16>(a, nactive, Cg, st); break;
-        default: launch_gc<20>(a, nactive, Cg, st); break;
-    }
-    kprof_end("gram_schmidt", st, nactive * (passes * a.cnt + 2.0) * a.n * sizeof(double2),
+    if (gs_cluster_cost(a.n, a.cnt, passes, nactive) <= gs_grid_cost(a.n, a.cnt, passes, nactive))
+        gs_cluster(a, nactive, st);
+    else
+        gs_grid(a, nactive, st);
+    kprof_end("gram_schmidt", st, nactive * ((double)passes * a.cnt + 2.0) * a.n * sizeof(double2),
               nactive * 8.0 * (passes * a.cnt + 1.0) * a.n);
-    return true;
 }
 
 }  // namespace sim

@@ -75,6 +75,28 @@ __host__ __device__ inline size_t factor_lval_offset(const Pencil& P) { return (
 // Offset of L0val (n values: the first coupling's shifted value of each row, 0 if none).
 __host__ __device__ inline size_t factor_l0_offset(const Pencil& P) { return factor_lval_offset(P) + (size_t)P.nnzL; }
 
+// Host side of a job space, kept with its buffers: pinned memory (the device
+// writes istat and worst, the host fills act), the list last uploaded and the
+// iterations every job of the last solve took.
+struct JobHost {
+    int J = 0;
+    int* istat = nullptr;
+    double* worst = nullptr;
+    int* act = nullptr;
+    cudaEvent_t act_ev = nullptr;  // the last upload from `act`
+    std::vector<int> uploaded;
+    int usual_steps = 0;
+    JobHost() = default;
+    JobHost(const JobHost&) = delete;
+    JobHost& operator=(const JobHost&) = delete;
+    ~JobHost() {
+        if (istat) cudaFreeHost(istat);
+        if (worst) cudaFreeHost(worst);
+        if (act) cudaFreeHost(act);
+        if (act_ev) cudaEventDestroy(act_ev);
+    }
+};
+
 // Workspace of a batch of Krylov jobs (one job = one Arnoldi process for
 // one shift and one starting vector).  All vectors are complex128 of length n,
 // job j's vector v at base + j*stride + v*n.
@@ -96,10 +118,22 @@ struct JobSpace {
     double2* g = nullptr;      // [J][k+1]
     double* scal = nullptr;    // [J][8]: rnorm0, res_est, res_true, ...
     int* istat = nullptr;      // [J][8]: steps in cycle, total iters, flags
-    double2* partial = nullptr;  // [J][nchunk][max(m+2, k+2)] partial dot products
-    int nchunk = 0;
-    int pstride = 0;           // per-job partial stride = nchunk * pw
-    int pw = 0;                // partial width
+    double2* y = nullptr;      // [J][k] the cycle's least-squares solution
+    // Gram-Schmidt scratch (gs_grid.cu)
+    double2* partial = nullptr;
+    int pw = 0;                // values per chunk of partial
+    double2* hsum = nullptr;   // [2][J][pw]
+    double* fin = nullptr;     // [J]
+    int* need = nullptr;       // [J]
+    int* ticket = nullptr;     // [J]
+    // partial sums of ||x||^2 and ||r||^2, one per 256 rows
+    int nblk = 0;
+    double* xpart = nullptr;   // [J][nblk]
+    double* rpart = nullptr;   // [J][nblk]
+    // host side: pinned memory that the kernels write flags and results to
+    struct JobHost* host = nullptr;
+    int* h_istat = nullptr;    // [J][IS_N]: the flags the host waits for; all fields after a cycle
+    double* h_worst = nullptr; // [J] last explicit relative residual
     int* d_jobshift = nullptr; // [J] shift id of each slot
     int* d_active = nullptr;   // [J] active slot list
     const int* h_jobshift = nullptr;  // [J] the same ids in host memory (owned by the caller)
@@ -113,9 +147,6 @@ __host__ __device__ inline int vs_count(int k) { return VS_Q0 + 2 * k + 1; }
 // scal / istat fields
 enum { SC_RNORM0 = 0, SC_RES = 1, SC_GAMMA = 2, SC_WORST = 3, SC_N = 8 };
 enum { IS_STEPS = 0, IS_ITERS = 1, IS_DONE = 2, IS_CYCLE_DONE = 3, IS_BROKEN = 4, IS_STALL = 5, IS_LOOSE = 6, IS_N = 8 };
-
-constexpr int GS_CHUNK = 4096;   // rows per CTA in the Gram–Schmidt kernels (16 per thread)
-constexpr int GS_THREADS = 256;
 
 // ---- krylov.cu ------------------------------------------------------------
 // Factor A - σB for the listed shifts into block form Dinv_k = D_k^{-1},

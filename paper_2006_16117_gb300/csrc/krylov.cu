@@ -234,18 +234,35 @@ void factor_shifts(const Pencil& P, int precision, const int* d_shift_list, int 
 // ---------------------------------------------------------------------------
 // sparse applies
 // ---------------------------------------------------------------------------
+// ||v||^2 over the CTA's (256) threads to *out
+__device__ __forceinline__ void block_norm2(double2 v, double* out) {
+    __shared__ double red[8];
+    const double s = warp_sum(fma(v.x, v.x, v.y * v.y));
+    __syncthreads();  // an earlier sum has been read
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = red[0];
+        for (int w = 1; w < 8; ++w) t += red[w];
+        *out = t;
+    }
+}
+
 // y = (A - σB) x, or y = rhs - (A - σB) x when rhs_slot >= 0, for SPMV_RJ
 // active jobs per thread: a thread owns one row and reads its indices and
 // values once for all of its jobs (the jobs' shifts differ only on B's
 // entries), then gathers each job's x.  Every job's row sum runs over the
 // row's entries in order, so the result does not depend on SPMV_RJ, which the
 // autotuner picks per matrix (1, 2, 4 or 8).
+// With a right-hand side each CTA also leaves ||y||^2 of its rows in js.rpart.
 template <int SPMV_RJ>
 __global__ void __launch_bounds__(256) k_spmv_jobs(Pencil P, JobSpace js, int x_slot, int y_slot, int rhs_slot,
                                                    const double2* sigma, int nactive) {
-    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int jb = blockIdx.y * SPMV_RJ;
-    if (g >= P.n) return;
+    if (rhs_slot < 0 && row >= P.n) return;
+    const bool in = row < P.n;
+    const int64_t g = in ? row : P.n - 1;  // the last CTA's spare threads only take part in the sums
     const int nj = min(SPMV_RJ, nactive - jb);
     const double2* x[SPMV_RJ];
     double2 sg[SPMV_RJ], acc[SPMV_RJ];
@@ -292,7 +309,8 @@ __global__ void __launch_bounds__(256) k_spmv_jobs(Pencil P, JobSpace js, int x_
         const int job = js.d_active[jb + r];
         double2 v = acc[r];
         if (rhs_slot >= 0) v = csub(js.vec[(size_t)job * js.vstride + (size_t)rhs_slot * js.n + g], v);
-        js.vec[(size_t)job * js.vstride + (size_t)y_slot * js.n + g] = v;
+        if (in) js.vec[(size_t)job * js.vstride + (size_t)y_slot * js.n + g] = v;
+        if (rhs_slot >= 0) block_norm2(in ? v : make_double2(0.0, 0.0), js.rpart + (size_t)job * js.nblk + blockIdx.x);
     }
 }
 
@@ -364,393 +382,30 @@ __global__ void k_apply_B_jobs(Pencil P, JobSpace js, int j, int y_slot) {
 }
 
 // ---------------------------------------------------------------------------
-// batched classical Gram–Schmidt, applied twice (CGS2), FP64
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ void block_reduce_vec(double2* red, int cnt, int nw) {
-    for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-        double2 s = red[i * nw];
-        for (int w = 1; w < nw; ++w) s = cadd(s, red[i * nw + w]);
-        red[i * nw] = s;
-    }
-}
-
-constexpr int GS_PER = GS_CHUNK / GS_THREADS;
-
-__device__ __forceinline__ void gs_partial_dots(const GSArgs& a, const double2* B, const double2 (&wv)[GS_PER],
-                                                int64_t r0, double2* red, double2* out) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int i = 0; i < a.cnt; ++i) {
-        const double2* q = B + (size_t)i * a.n;
-        double2 acc = make_double2(0.0, 0.0);
-#pragma unroll
-        for (int t = 0; t < GS_PER; ++t) {
-            int64_t r = r0 + threadIdx.x + t * GS_THREADS;
-            if (r < a.n) {
-                double2 qv = q[r];
-                acc.x = fma(qv.x, wv[t].x, acc.x);
-                acc.x = fma(qv.y, wv[t].y, acc.x);
-                acc.y = fma(qv.x, wv[t].y, acc.y);
-                acc.y = fma(-qv.y, wv[t].x, acc.y);
-            }
-        }
-        acc = warp_sum(acc);
-        if (lane == 0) red[i * nw + warp] = acc;
-    }
-    if (a.dgks) {  // partial ||w||^2 as value cnt
-        double nn = 0.0;
-#pragma unroll
-        for (int t = 0; t < GS_PER; ++t) nn += wv[t].x * wv[t].x + wv[t].y * wv[t].y;
-        nn = warp_sum(nn);
-        if (lane == 0) red[a.cnt * nw + warp] = make_double2(nn, 0.0);
-    }
-    __syncthreads();
-    block_reduce_vec(red, a.cnt + (a.dgks ? 1 : 0), nw);
-    __syncthreads();
-    for (int i = threadIdx.x; i < a.cnt + (a.dgks ? 1 : 0); i += blockDim.x) out[i] = red[i * nw];
-}
-
-// pass-1 partial dot products  h_i = Σ_rows conj(q_i) w
-__global__ void __launch_bounds__(GS_THREADS) k_gs_dots(GSArgs a) {
-    const int job = a.active[blockIdx.y];
-    const int chunk = blockIdx.x;
-    const double2* B = a.basis + (size_t)job * a.bstride;
-    const double2* w = a.w + (size_t)job * a.wstride;
-    extern __shared__ double2 red[];
-    const int64_t r0 = (int64_t)chunk * GS_CHUNK;
-    double2 wv[GS_PER];
-#pragma unroll
-    for (int t = 0; t < GS_PER; ++t) {
-        int64_t r = r0 + threadIdx.x + t * GS_THREADS;
-        wv[t] = r < a.n ? w[r] : make_double2(0.0, 0.0);
-    }
-    gs_partial_dots(a, B, wv, r0, red, a.pout + ((size_t)job * a.nchunk + chunk) * a.pw);
-}
-
-// reduce pass partials -> h; w -= Σ q_i h_i; then either the next pass's
-// partial dots (next_dots = 1) or the partial squared norm.  hcol = h or += h.
-__global__ void __launch_bounds__(GS_THREADS) k_gs_update(GSArgs a, int accumulate, int next_dots) {
-    const int job = a.active[blockIdx.y];
-    const int chunk = blockIdx.x;
-    const double2* B = a.basis + (size_t)job * a.bstride;
-    double2* w = a.w + (size_t)job * a.wstride;
-    extern __shared__ double2 sm[];
-    double2* h = sm;                 // [cnt]
-    double2* red = sm + a.cnt + 1;   // [cnt*nw]
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const double2* Pin = a.pin + (size_t)job * a.nchunk * a.pw;
-    double2* out = a.pout + ((size_t)job * a.nchunk + chunk) * a.pw;
-    if (a.dgks && accumulate) {
-        // second pass: needed only if the first one lost more than half of ||w||^2
-        __shared__ int s_skip;
-        if (threadIdx.x == 0) {
-            double na = 0.0;
-            for (int c = 0; c < a.nchunk; ++c) na += Pin[(size_t)c * a.pw + a.cnt].x;
-            const double nb = Pin[a.cnt + 1].x;
-            s_skip = na > 0.5 * nb;
-        }
-        __syncthreads();
-        if (s_skip) {
-            if (threadIdx.x == 0) out[0] = Pin[(size_t)chunk * a.pw + a.cnt];  // this chunk's ||w||^2
-            return;
-        }
-    }
-    for (int i = threadIdx.x; i < a.cnt; i += blockDim.x) {
-        double2 s = make_double2(0.0, 0.0);
-        for (int c = 0; c < a.nchunk; ++c) s = cadd(s, Pin[(size_t)c * a.pw + i]);
-        h[i] = s;
-    }
-    if (a.dgks && !accumulate && chunk == 0 && threadIdx.x == 0) {
-        double nb = 0.0;
-        for (int c = 0; c < a.nchunk; ++c) nb += Pin[(size_t)c * a.pw + a.cnt].x;
-        out[a.cnt + 1] = make_double2(nb, 0.0);  // ||w||^2 before the first pass, for the test above
-    }
-    __syncthreads();
-    if (chunk == 0) {
-        double2* hc = a.hcol + (size_t)job * a.hstride;
-        for (int i = threadIdx.x; i < a.cnt; i += blockDim.x) hc[i] = accumulate ? cadd(hc[i], h[i]) : h[i];
-    }
-    const int64_t r0 = (int64_t)chunk * GS_CHUNK;
-    double2 wv[GS_PER];
-#pragma unroll
-    for (int t = 0; t < GS_PER; ++t) {
-        int64_t r = r0 + threadIdx.x + t * GS_THREADS;
-        wv[t] = r < a.n ? w[r] : make_double2(0.0, 0.0);
-    }
-    for (int i = 0; i < a.cnt; ++i) {
-        const double2* q = B + (size_t)i * a.n;
-        const double2 hi = h[i];
-#pragma unroll
-        for (int t = 0; t < GS_PER; ++t) {
-            int64_t r = r0 + threadIdx.x + t * GS_THREADS;
-            if (r < a.n) {
-                double2 qv = q[r];
-                wv[t].x = fma(-qv.x, hi.x, wv[t].x);
-                wv[t].x = fma(qv.y, hi.y, wv[t].x);
-                wv[t].y = fma(-qv.x, hi.y, wv[t].y);
-                wv[t].y = fma(-qv.y, hi.x, wv[t].y);
-            }
-        }
-    }
-#pragma unroll
-    for (int t = 0; t < GS_PER; ++t) {
-        int64_t r = r0 + threadIdx.x + t * GS_THREADS;
-        if (r < a.n) w[r] = wv[t];
-    }
-    if (next_dots) {
-        gs_partial_dots(a, B, wv, r0, red, out);
-    } else {
-        double acc = 0.0;
-#pragma unroll
-        for (int t = 0; t < GS_PER; ++t) acc += wv[t].x * wv[t].x + wv[t].y * wv[t].y;
-        acc = warp_sum(acc);
-        if (lane == 0) red[warp] = make_double2(acc, 0.0);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double s = 0.0;
-            for (int w2 = 0; w2 < nw; ++w2) s += red[w2].x;
-            out[0] = make_double2(s, 0.0);
-        }
-    }
-}
-
-// partial ||w||^2 of each chunk (w read only), into pout[chunk]
-__global__ void __launch_bounds__(GS_THREADS) k_gs_norm_partial(GSArgs a) {
-    const int job = a.active[blockIdx.y];
-    const int chunk = blockIdx.x;
-    const double2* w = a.w + (size_t)job * a.wstride;
-    __shared__ double red[GS_THREADS / 32];
-    const int64_t r0 = (int64_t)chunk * GS_CHUNK;
-    double acc = 0.0;
-    for (int t = 0; t < GS_PER; ++t) {
-        const int64_t r = r0 + threadIdx.x + t * GS_THREADS;
-        if (r < a.n) {
-            const double2 v = w[r];
-            acc += v.x * v.x + v.y * v.y;
-        }
-    }
-    acc = warp_sum(acc);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double sum = 0.0;
-        for (int i = 0; i < GS_THREADS / 32; ++i) sum += red[i];
-        a.pout[((size_t)job * a.nchunk + chunk) * a.pw] = make_double2(sum, 0.0);
-    }
-}
-
-// reduce norm partials, write the subdiagonal entry and normalise w in place
-// (Arnoldi: breakdown test h_{j+1,j} <= btol * ||H_{1:j+1,1:j+1}||_F).
-__global__ void __launch_bounds__(GS_THREADS) k_gs_finish(GSArgs a) {
-    const int job = a.active[blockIdx.y];
-    const int chunk = blockIdx.x;
-    double2* w = a.w + (size_t)job * a.wstride;
-    __shared__ double s_hn;
-    __shared__ int s_broken;
-    if (threadIdx.x == 0) {
-        const double2* Pin = a.pin + (size_t)job * a.nchunk * a.pw;
-        double s = 0.0;
-        for (int c = 0; c < a.nchunk; ++c) s += Pin[(size_t)c * a.pw].x;
-        double hn = sqrt(s);
-        int broken = !(hn > 0.0);
-        if (a.Hfull) {
-            const double2* H = a.Hfull + (size_t)job * a.Hstride;
-            double f = 0.0;
-            for (int c = 0; c <= a.j; ++c)
-                for (int r = 0; r <= a.j; ++r) f += cabs2(H[(size_t)c * a.Hld + r]);
-            if (hn <= a.btol * sqrt(f)) broken = 1;
-        }
-        s_hn = hn;
-        s_broken = broken;
-        if (chunk == 0) {
-            double2* hc = a.hcol + (size_t)job * a.hstride;
-            hc[a.cnt] = make_double2((broken && a.Hfull) ? 0.0 : hn, 0.0);
-            if (broken && a.meff) a.meff[job] = a.j + 1;
-            if (broken && a.istat) a.istat[job * IS_N + IS_BROKEN] = 1;
-        }
-    }
-    __syncthreads();
-    if (s_broken) return;
-    const double inv = 1.0 / s_hn;
-    const int64_t r0 = (int64_t)chunk * GS_CHUNK;
-    for (int t = 0; t < GS_PER; ++t) {
-        int64_t r = r0 + threadIdx.x + t * GS_THREADS;
-        if (r < a.n) w[r] = cscale(w[r], inv);
-    }
-}
-
-// one CGS2 step on the active jobs: partial buffers A = partial, B = partial + half
-static void gs_run(GSArgs a, double2* partial, size_t half, int nactive, cudaStream_t st) {
-    if (gs_cluster(a, nactive, st)) return;
-    kprof_begin("gram_schmidt", st);
-    dim3 grid(a.nchunk, nactive);
-    const int nw = GS_THREADS / 32;
-    size_t sm_dots = (size_t)(a.cnt + 2) * nw * sizeof(double2) + 64;
-    size_t sm_upd = ((size_t)a.cnt + 1 + (size_t)(a.cnt + 2) * nw) * sizeof(double2) + 64;
-    double2* A = partial;
-    double2* Bf = partial + half;
-    if (a.single) {  // one pass: dots, update with the norm, finish
-        a.dgks = 0;
-        a.pout = A;
-        k_gs_dots<<<grid, GS_THREADS, sm_dots, st>>>(a);
-        SIM_LAUNCH_CHECK();
-        a.pin = A;
-        a.pout = Bf;
-        k_gs_update<<<grid, GS_THREADS, sm_upd, st>>>(a, 0, 0);
-        SIM_LAUNCH_CHECK();
-        a.pin = Bf;
-        k_gs_finish<<<grid, GS_THREADS, 0, st>>>(a);
-        SIM_LAUNCH_CHECK();
-        kprof_end("gram_schmidt", st, nactive * (2.0 * a.cnt + 4.0) * a.n * sizeof(double2),
-                  nactive * 16.0 * a.cnt * a.n);
-        return;
-    }
-    a.pout = A;
-    k_gs_dots<<<grid, GS_THREADS, sm_dots, st>>>(a);
-    SIM_LAUNCH_CHECK();
-    a.pin = A;
-    a.pout = Bf;
-    k_gs_update<<<grid, GS_THREADS, sm_upd, st>>>(a, 0, 1);
-    SIM_LAUNCH_CHECK();
-    a.pin = Bf;
-    a.pout = A;
-    k_gs_update<<<grid, GS_THREADS, sm_upd, st>>>(a, 1, 0);
-    SIM_LAUNCH_CHECK();
-    a.pin = A;
-    k_gs_finish<<<grid, GS_THREADS, 0, st>>>(a);
-    SIM_LAUNCH_CHECK();
-    kprof_end("gram_schmidt", st, nactive * (4.0 * a.cnt + 6.0) * a.n * sizeof(double2), nactive * 32.0 * a.cnt * a.n);
-}
-
-// ---------------------------------------------------------------------------
 // batched FGMRES(k) with the block factorisation as right preconditioner
 // ---------------------------------------------------------------------------
-__global__ void k_copy_slot(JobSpace js, int src, int dst) {
-    const int job = js.d_active[blockIdx.y];
-    int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= js.n) return;
-    js.vec[(size_t)job * js.vstride + (size_t)dst * js.n + g] = js.vec[(size_t)job * js.vstride + (size_t)src * js.n + g];
-}
-
-__global__ void k_zero_slot(JobSpace js, int dst) {
-    const int job = js.d_active[blockIdx.y];
-    int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= js.n) return;
-    js.vec[(size_t)job * js.vstride + (size_t)dst * js.n + g] = make_double2(0.0, 0.0);
-}
-
-// after the start vector's norm γ landed in g[0]: reset the cycle state
-__global__ void k_gm_cycle_init(JobSpace js, int nactive, int first, double tol) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nactive) return;
-    const int job = js.d_active[t];
-    double2* g = js.g + (size_t)job * (js.k + 1);
-    double* sc = js.scal + (size_t)job * SC_N;
-    int* is = js.istat + (size_t)job * IS_N;
-    const double gamma = g[0].x;
-    for (int i = 1; i <= js.k; ++i) g[i] = make_double2(0.0, 0.0);
-    if (first) {
-        sc[SC_RNORM0] = gamma;
-        is[IS_ITERS] = 0;
-        is[IS_DONE] = 0;
-        is[IS_STALL] = 0;
-        is[IS_LOOSE] = 0;
-    }
-    sc[SC_GAMMA] = gamma;
-    sc[SC_RES] = gamma;
-    is[IS_STEPS] = 0;
-    const int conv = !(gamma > tol * sc[SC_RNORM0]);
-    is[IS_CYCLE_DONE] = conv;
-    if (conv) is[IS_DONE] = 1;
-}
-
-// Givens update of Hessenberg column i; residual estimate |g_{i+1}|
-__global__ void k_gm_givens(JobSpace js, int nactive, int i, double tol, int max_iter) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nactive) return;
-    const int job = js.d_active[t];
-    const int k = js.k;
-    double2* col = js.Hg + (size_t)job * (k + 1) * k + (size_t)i * (k + 1);
-    double2* cs = js.cs + (size_t)job * k;
-    double2* sn = js.sn + (size_t)job * k;
-    double2* g = js.g + (size_t)job * (k + 1);
-    double* sc = js.scal + (size_t)job * SC_N;
-    int* is = js.istat + (size_t)job * IS_N;
-    const double hn = col[i + 1].x;
-    for (int q = 0; q < i; ++q) {
-        const double c = cs[q].x;
-        const double2 s = sn[q];
-        double2 a = col[q], b = col[q + 1];
-        col[q] = cadd(cscale(a, c), cmul(s, b));
-        col[q + 1] = csub(cscale(b, c), cconjmul(s, a));
-    }
-    double2 a = col[i], b = col[i + 1];
-    const double na = cabsd(a), nbv = cabsd(b);
-    double c;
-    double2 s;
-    if (na == 0.0) {
-        c = 0.0;
-        s = make_double2(1.0, 0.0);
-    } else {
-        const double nu = hypot(na, nbv);
-        c = na / nu;
-        const double2 ph = cscale(a, 1.0 / na);
-        s = cscale(cmulc(ph, b), 1.0 / nu);  // (a/|a|) conj(b) / nu
-    }
-    cs[i] = make_double2(c, 0.0);
-    sn[i] = s;
-    col[i] = cadd(cscale(a, c), cmul(s, b));
-    col[i + 1] = make_double2(0.0, 0.0);
-    const double2 gi = g[i];
-    g[i] = cscale(gi, c);
-    g[i + 1] = make_double2(-(s.x * gi.x + s.y * gi.y), -(s.x * gi.y - s.y * gi.x));  // -conj(s) g_i
-    const double res = cabsd(g[i + 1]);
-    sc[SC_RES] = res;
-    is[IS_STEPS] = i + 1;
-    is[IS_ITERS] += 1;
-    is[IS_CYCLE_DONE] = (res <= tol * sc[SC_RNORM0]) || !(hn > 0.0) || (i + 1 == k) || (is[IS_ITERS] >= max_iter);
-}
-
-// x += Z y with R y = g (R: the rotated Hessenberg, order = steps)
-__global__ void k_gm_update_x(JobSpace js) {
+// x = Z y (+ x after the first cycle), y from the end of the cycle (gs_finish.cuh);
+// each CTA leaves ||x||^2 of its rows in js.xpart
+__global__ void __launch_bounds__(256) k_gm_update_x(JobSpace js, int first) {
     const int job = js.d_active[blockIdx.y];
     const int k = js.k;
-    __shared__ double2 y[64];
-    __shared__ int steps;
-    if (threadIdx.x == 0) {
-        const int* is = js.istat + (size_t)job * IS_N;
-        steps = is[IS_STEPS];
-        const double2* R = js.Hg + (size_t)job * (k + 1) * k;
-        const double2* g = js.g + (size_t)job * (k + 1);
-        for (int r = steps - 1; r >= 0; --r) {
-            double2 acc = g[r];
-            for (int c = r + 1; c < steps; ++c) acc = csub(acc, cmul(R[(size_t)c * (k + 1) + r], y[c]));
-            double2 d = R[(size_t)r * (k + 1) + r];
-            y[r] = (d.x == 0.0 && d.y == 0.0) ? make_double2(0.0, 0.0) : cdiv(acc, d);
-        }
+    const int steps = js.istat[(size_t)job * IS_N + IS_STEPS];
+    const int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    double2 x = make_double2(0.0, 0.0);
+    if (gi < js.n) {
+        double2* base = js.vec + (size_t)job * js.vstride + gi;
+        if (!first) x = base[(size_t)VS_X * js.n];
+        const double2* z = base + (size_t)vs_Z(k) * js.n;
+#pragma unroll 4
+        for (int q = 0; q < steps; ++q) x = cfma(z[(size_t)q * js.n], js.y[(size_t)job * k + q], x);
+        base[(size_t)VS_X * js.n] = x;
     }
-    __syncthreads();
-    int64_t gi = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gi >= js.n) return;
-    double2* base = js.vec + (size_t)job * js.vstride;
-    double2 x = base[(size_t)VS_X * js.n + gi];
-    for (int q = 0; q < steps; ++q) x = cfma(base[(size_t)(vs_Z(k) + q) * js.n + gi], y[q], x);
-    base[(size_t)VS_X * js.n + gi] = x;
+    block_norm2(x, js.xpart + (size_t)job * js.nblk + blockIdx.x);
 }
 
-// explicit residual norm from partials (buffer pin), and ||x|| (buffer pinx):
-// done if <= tol * rnorm0
-__global__ void k_gm_check(JobSpace js, int nactive, const double2* pin, const double2* pinx, int nchunk, int pw,
-                           double tol, int max_iter, const double2* sigma, double anorm, double bnorm) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nactive) return;
-    const int job = js.d_active[t];
-    const double2* P = pin + (size_t)job * nchunk * pw;
-    const double2* PX = pinx + (size_t)job * nchunk * pw;
-    double s = 0.0, sx = 0.0;
-    for (int c = 0; c < nchunk; ++c) {
-        s += P[(size_t)c * pw].x;
-        sx += PX[(size_t)c * pw].x;
-    }
+// The end of a cycle of one job with the squared residual norm s and ||x||^2 = sx.
+__device__ void gm_check_job(const JobSpace& js, int job, double s, double sx, double tol, int max_iter,
+                             const double2* sigma, double anorm, double bnorm) {
     double* sc = js.scal + (size_t)job * SC_N;
     int* is = js.istat + (size_t)job * IS_N;
     const double r = sqrt(s);
@@ -784,100 +439,110 @@ __global__ void k_gm_check(JobSpace js, int nactive, const double2* pin, const d
     }
 }
 
-namespace {
-struct Pinned {
-    int* ist = nullptr;
-    double* sc = nullptr;
-    int* act = nullptr;
-    int cap = 0;
-    cudaEvent_t act_ev = nullptr;  // the last upload from `act`
-    void ensure(int J) {
-        if (J <= cap) return;
-        if (ist) cudaFreeHost(ist);
-        if (sc) cudaFreeHost(sc);
-        if (act) cudaFreeHost(act);
-        SIM_CUDA(cudaMallocHost(&ist, sizeof(int) * IS_N * J));
-        SIM_CUDA(cudaMallocHost(&sc, sizeof(double) * SC_N * J));
-        SIM_CUDA(cudaMallocHost(&act, sizeof(int) * J));
-        cap = J;
+// explicit residual norm and ||x|| from their partial sums, one CTA per job: done
+// if <= tol * rnorm0; the job's state goes to the host's copy
+__global__ void __launch_bounds__(256) k_gm_check(JobSpace js, double tol, int max_iter, const double2* sigma,
+                                                  double anorm, double bnorm) {
+    const int job = js.d_active[blockIdx.x];
+    double s = 0.0, sx = 0.0;
+    for (int c = threadIdx.x; c < js.nblk; c += 256) {
+        s += js.rpart[(size_t)job * js.nblk + c];
+        sx += js.xpart[(size_t)job * js.nblk + c];
     }
-};
-Pinned g_pin;
+    s = warp_sum(s);
+    sx = warp_sum(sx);
+    __shared__ double red[2][8];
+    if ((threadIdx.x & 31) == 0) {
+        red[0][threadIdx.x >> 5] = s;
+        red[1][threadIdx.x >> 5] = sx;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    s = sx = 0.0;
+    for (int w = 0; w < 8; ++w) {
+        s += red[0][w];
+        sx += red[1][w];
+    }
+    gm_check_job(js, job, s, sx, tol, max_iter, sigma, anorm, bnorm);
+    for (int i = 0; i < IS_N; ++i) js.h_istat[job * IS_N + i] = js.istat[job * IS_N + i];
+    js.h_worst[job] = js.scal[(size_t)job * SC_N + SC_WORST];
+}
 
+namespace {
+
+// The active list on the device, in this order (nothing to do if it is there).
 void upload_active(const JobSpace& js, const std::vector<int>& a, cudaStream_t st) {
-    g_pin.ensure(js.J);
+    JobHost& h = *js.host;
+    if (h.uploaded == a) return;
     // the previous upload must have left the pinned buffer before it is refilled
-    if (g_pin.act_ev) SIM_CUDA(cudaEventSynchronize(g_pin.act_ev));
-    else SIM_CUDA(cudaEventCreateWithFlags(&g_pin.act_ev, cudaEventDisableTiming));
-    for (size_t i = 0; i < a.size(); ++i) g_pin.act[i] = a[i];
-    SIM_CUDA(cudaMemcpyAsync(js.d_active, g_pin.act, sizeof(int) * a.size(), cudaMemcpyHostToDevice, st));
-    SIM_CUDA(cudaEventRecord(g_pin.act_ev, st));
+    SIM_CUDA(cudaEventSynchronize(h.act_ev));
+    std::copy(a.begin(), a.end(), h.act);
+    SIM_CUDA(cudaMemcpyAsync(js.d_active, h.act, sizeof(int) * a.size(), cudaMemcpyHostToDevice, st));
+    SIM_CUDA(cudaEventRecord(h.act_ev, st));
+    h.uploaded = a;
 }
 
-void read_state(const JobSpace& js, cudaStream_t st) {
-    g_pin.ensure(js.J);
-    SIM_CUDA(cudaMemcpyAsync(g_pin.ist, js.istat, sizeof(int) * IS_N * js.J, cudaMemcpyDeviceToHost, st));
-    SIM_CUDA(cudaMemcpyAsync(g_pin.sc, js.scal, sizeof(double) * SC_N * js.J, cudaMemcpyDeviceToHost, st));
-    SIM_CUDA(cudaStreamSynchronize(st));
-}
-
-// ||slot|| of active jobs into hcol[0] (stride), and scale slot by 1/||slot||
-void norm_and_scale(const JobSpace& js, int nactive, double2* w_base, int64_t wstride, double2* hcol,
-                    int64_t hstride, cudaStream_t st) {
-    GSArgs a{};
-    a.basis = nullptr;
-    a.bstride = 0;
-    a.w = w_base;
-    a.wstride = wstride;
-    a.hcol = hcol;
-    a.hstride = hstride;
-    a.cnt = 0;
+GSArgs gs_args(const JobSpace& js) {
+    GSArgs a;
     a.n = js.n;
-    a.pw = js.pw;
-    a.nchunk = js.nchunk;
     a.active = js.d_active;
-    if (gs_cluster(a, nactive, st)) return;
-    dim3 grid(js.nchunk, nactive);
-    const int nw = GS_THREADS / 32;
-    a.pout = js.partial;
-    k_gs_update<<<grid, GS_THREADS, (size_t)(1 + nw) * sizeof(double2) + 64, st>>>(a, 0, 0);
-    SIM_LAUNCH_CHECK();
-    a.pin = js.partial;
-    k_gs_finish<<<grid, GS_THREADS, 0, st>>>(a);
-    SIM_LAUNCH_CHECK();
+    a.h_istat = js.h_istat;
+    a.part = js.partial;
+    a.pw = js.pw;
+    a.hsum = js.hsum;
+    a.fin = js.fin;
+    a.need = js.need;
+    a.ticket = js.ticket;
+    a.J = js.J;
+    return a;
 }
+
+GmArgs gm_args(const JobSpace& js, int mode, int i, int first, double tol, int max_iter) {
+    GmArgs g;
+    g.mode = mode;
+    g.k = js.k;
+    g.i = i;
+    g.first = first;
+    g.tol = tol;
+    g.max_iter = max_iter;
+    g.Hg = js.Hg;
+    g.cs = js.cs;
+    g.sn = js.sn;
+    g.g = js.g;
+    g.y = js.y;
+    g.scal = js.scal;
+    g.istat = js.istat;
+    return g;
+}
+
 }  // namespace
 
 bool inner_solve(const Pencil& P, const sim_options& opt, JobSpace& js, const std::vector<int>& jobs,
                  const double2* d_sigma, void* const* d_factor_ptrs, cudaStream_t st, InnerStats& stats) {
     if (jobs.empty()) return true;
     const int k = js.k;
-    const dim3 rows_grid_1(cdiv_up(js.n, 256), 1);
-    const size_t half = (size_t)js.J * js.nchunk * js.pw;
     auto rows_grid = [&](int na) { return dim3(cdiv_up(js.n, 256), na); };
-    (void)rows_grid_1;
+    const int* ist = js.h_istat;
     std::vector<int> cyc = jobs;  // jobs that start a cycle
-    upload_active(js, cyc, st);
-    k_zero_slot<<<rows_grid((int)cyc.size()), 256, 0, st>>>(js, VS_X);
-    SIM_LAUNCH_CHECK();
-    k_copy_slot<<<rows_grid((int)cyc.size()), 256, 0, st>>>(js, VS_RHS, VS_R);
-    SIM_LAUNCH_CHECK();
     bool first = true;
     bool ok = true;
+    // Iterations that every job of the last solve took: the host issues that many
+    // without waiting for the flags in between (a job whose cycle has ended takes no
+    // further columns, whatever is computed for it).
+    int& usual = js.host->usual_steps;
     while (!cyc.empty()) {
-        const int nc = (int)cyc.size();
         upload_active(js, cyc, st);
-        k_copy_slot<<<rows_grid(nc), 256, 0, st>>>(js, VS_R, VS_Q0);
-        SIM_LAUNCH_CHECK();
-        norm_and_scale(js, nc, js.vec + (size_t)VS_Q0 * js.n, js.vstride, js.g, k + 1, st);
-        k_gm_cycle_init<<<cdiv_up(nc, 128), 128, 0, st>>>(js, nc, first ? 1 : 0, opt.inner_tol);
-        SIM_LAUNCH_CHECK();
-        first = false;
-        read_state(js, st);
-        std::vector<int> act;
-        for (int j : cyc)
-            if (!g_pin.ist[j * IS_N + IS_CYCLE_DONE]) act.push_back(j);
-        std::vector<int> in_cycle = act;
+        {
+            // q_0 = r / ||r||, the cycle's state
+            GSArgs a = gs_args(js);
+            a.w = js.vec + (size_t)VS_Q0 * js.n;
+            a.wstride = js.vstride;
+            a.src = js.vec + (size_t)(first ? VS_RHS : VS_R) * js.n;
+            a.sstride = js.vstride;
+            a.gm = gm_args(js, GmArgs::START, 0, first ? 1 : 0, opt.inner_tol, opt.inner_max_iter);
+            gram_schmidt(a, (int)cyc.size(), st);
+        }
+        std::vector<int> act = cyc;
         for (int i = 0; i < k && !act.empty(); ++i) {
             const int na = (int)act.size();
             upload_active(js, act, st);
@@ -888,73 +553,51 @@ bool inner_solve(const Pencil& P, const sim_options& opt, JobSpace& js, const st
                 throw std::runtime_error("LIMIT:block size " + std::to_string(P.T) +
                                          " too large for the cluster block solve's shared memory");
             launch_spmv(P, js, na, vs_Z(k) + i, VS_Q0 + i + 1, -1, d_sigma, st);
-            GSArgs a{};
+            GSArgs a = gs_args(js);
             a.basis = js.vec + (size_t)VS_Q0 * js.n;
             a.bstride = js.vstride;
             a.w = js.vec + (size_t)(VS_Q0 + i + 1) * js.n;
             a.wstride = js.vstride;
-            a.hcol = js.Hg + (size_t)i * (k + 1);
-            a.hstride = (int64_t)(k + 1) * k;
             a.cnt = i + 1;
-            a.n = js.n;
-            a.pw = js.pw;
-            a.nchunk = js.nchunk;
-            a.active = js.d_active;
             a.dgks = 1;
-            gs_run(a, js.partial, half, na, st);
-            k_gm_givens<<<cdiv_up(na, 128), 128, 0, st>>>(js, na, i, opt.inner_tol, opt.inner_max_iter);
-            SIM_LAUNCH_CHECK();
-            read_state(js, st);
+            a.gm = gm_args(js, GmArgs::STEP, i, 0, opt.inner_tol, opt.inner_max_iter);
+            gram_schmidt(a, na, st);
+            if (first && i + 1 < usual) continue;
+            SIM_CUDA(cudaStreamSynchronize(st));
             std::vector<int> next;
             for (int j : act)
-                if (!g_pin.ist[j * IS_N + IS_CYCLE_DONE]) next.push_back(j);
+                if (!ist[j * IS_N + IS_CYCLE_DONE]) next.push_back(j);
             act.swap(next);
         }
-        if (in_cycle.empty()) break;
-        const int ni = (int)in_cycle.size();
-        upload_active(js, in_cycle, st);
-        k_gm_update_x<<<rows_grid(ni), 256, 0, st>>>(js);
+        const int ni = (int)cyc.size();
+        upload_active(js, cyc, st);
+        k_gm_update_x<<<rows_grid(ni), 256, 0, st>>>(js, first ? 1 : 0);
         SIM_LAUNCH_CHECK();
         launch_spmv(P, js, ni, VS_X, VS_R, VS_RHS, d_sigma, st);
-        {
-            GSArgs a{};
-            a.w = js.vec + (size_t)VS_R * js.n;
-            a.wstride = js.vstride;
-            a.cnt = 0;
-            a.n = js.n;
-            a.pw = js.pw;
-            a.nchunk = js.nchunk;
-            a.active = js.d_active;
-            a.pout = js.partial;
-            const int nw = GS_THREADS / 32;
-            k_gs_update<<<dim3(js.nchunk, ni), GS_THREADS, (size_t)(1 + nw) * sizeof(double2) + 64, st>>>(a, 0, 0);
-            SIM_LAUNCH_CHECK();
-            // ||x||^2 partials into the second half, for the rounding floor
-            a.w = js.vec + (size_t)VS_X * js.n;
-            a.pout = js.partial + half;
-            k_gs_norm_partial<<<dim3(js.nchunk, ni), GS_THREADS, 0, st>>>(a);
-            SIM_LAUNCH_CHECK();
-        }
-        k_gm_check<<<cdiv_up(ni, 128), 128, 0, st>>>(js, ni, js.partial, js.partial + half, js.nchunk, js.pw,
-                                                     opt.inner_tol, opt.inner_max_iter, d_sigma, P.anorm, P.bnorm);
+        k_gm_check<<<ni, 256, 0, st>>>(js, opt.inner_tol, opt.inner_max_iter, d_sigma, P.anorm, P.bnorm);
         SIM_LAUNCH_CHECK();
-        read_state(js, st);
+        SIM_CUDA(cudaStreamSynchronize(st));
+        if (first) {
+            usual = k;
+            for (int j : cyc) usual = std::min(usual, ist[j * IS_N + IS_STEPS]);
+        }
+        first = false;
         std::vector<int> again;
-        for (int j : in_cycle) {
-            int d = g_pin.ist[j * IS_N + IS_DONE];
+        for (int j : cyc) {
+            int d = ist[j * IS_N + IS_DONE];
             if (d == 0) again.push_back(j);
             if (d == -1) ok = false;
         }
         cyc.swap(again);
     }
     for (int j : jobs) {
-        int it = g_pin.ist[j * IS_N + IS_ITERS];
+        int it = ist[j * IS_N + IS_ITERS];
         stats.solves += 1;
         stats.iters += it;
         stats.max_iters = std::max(stats.max_iters, it);
-        stats.worst = std::max(stats.worst, g_pin.sc[j * SC_N + SC_WORST]);
-        stats.loose += g_pin.ist[j * IS_N + IS_LOOSE];
-        if (g_pin.ist[j * IS_N + IS_DONE] != 1) ok = false;
+        stats.worst = std::max(stats.worst, js.h_worst[j]);
+        stats.loose += ist[j * IS_N + IS_LOOSE];
+        if (ist[j * IS_N + IS_DONE] != 1) ok = false;
     }
     return ok;
 }
@@ -962,19 +605,13 @@ bool inner_solve(const Pencil& P, const sim_options& opt, JobSpace& js, const st
 // ---------------------------------------------------------------------------
 // Arnoldi with CGS2 for all jobs of the space
 // ---------------------------------------------------------------------------
-__global__ void k_copy_to_V(JobSpace js, int src_slot, int j) {
-    const int job = js.d_active[blockIdx.y];
-    int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= js.n) return;
-    js.V[((size_t)job * (js.m + 1) + j) * js.n + g] = js.vec[(size_t)job * js.vstride + (size_t)src_slot * js.n + g];
-}
-
 __global__ void k_arnoldi_init(JobSpace js, int nactive) {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nactive) return;
     const int job = js.d_active[t];
     js.meff[job] = js.m;
     js.istat[job * IS_N + IS_BROKEN] = 0;
+    js.h_istat[job * IS_N + IS_BROKEN] = 0;
     double2* H = js.H + (size_t)job * (js.m + 1) * js.m;
     for (int e = 0; e < (js.m + 1) * js.m; ++e) H[e] = make_double2(0.0, 0.0);
 }
@@ -996,15 +633,20 @@ bool arnoldi(const Pencil& P, const sim_options& opt, JobSpace& js, const double
     upload_active(js, all, st);
     k_arnoldi_init<<<cdiv_up(J, 128), 128, 0, st>>>(js, J);
     SIM_LAUNCH_CHECK();
-    k_copy_to_V<<<rows_grid(J), 256, 0, st>>>(js, VS_X, 0);
-    SIM_LAUNCH_CHECK();
-    // beta = ||b||, v_1 = b / beta   (the norm lands in g[job*(k+1)] as scratch)
-    norm_and_scale(js, J, js.V, (int64_t)(m + 1) * js.n, js.g, js.k + 1, st);
+    {
+        // beta = ||b||, v_1 = b / beta   (the norm lands in g[job*(k+1)] as scratch)
+        GSArgs a = gs_args(js);
+        a.w = js.V;
+        a.wstride = (int64_t)(m + 1) * js.n;
+        a.src = js.vec + (size_t)VS_X * js.n;
+        a.sstride = js.vstride;
+        a.hcol = js.g;
+        a.hstride = js.k + 1;
+        gram_schmidt(a, J, st);
+    }
     k_store_beta<<<cdiv_up(J, 128), 128, 0, st>>>(js, J);
     SIM_LAUNCH_CHECK();
-    const size_t half = (size_t)js.J * js.nchunk * js.pw;
     std::vector<int> act = all;
-    std::vector<int> broken(J, 0);
     for (int j = 0; j < m && !act.empty(); ++j) {
         const int na = (int)act.size();
         upload_active(js, act, st);
@@ -1012,20 +654,16 @@ bool arnoldi(const Pencil& P, const sim_options& opt, JobSpace& js, const double
         SIM_LAUNCH_CHECK();
         ok = inner_solve(P, opt, js, act, d_sigma, d_factor_ptrs, st, stats) && ok;
         upload_active(js, act, st);
-        k_copy_to_V<<<rows_grid(na), 256, 0, st>>>(js, VS_X, j + 1);
-        SIM_LAUNCH_CHECK();
-        GSArgs a{};
+        GSArgs a = gs_args(js);
         a.basis = js.V;
         a.bstride = (int64_t)(m + 1) * js.n;
         a.w = js.V + (size_t)(j + 1) * js.n;
         a.wstride = (int64_t)(m + 1) * js.n;
+        a.src = js.vec + (size_t)VS_X * js.n;
+        a.sstride = js.vstride;
         a.hcol = js.H + (size_t)j * (m + 1);
         a.hstride = (int64_t)(m + 1) * m;
         a.cnt = j + 1;
-        a.n = js.n;
-        a.pw = js.pw;
-        a.nchunk = js.nchunk;
-        a.active = js.d_active;
         a.Hfull = js.H;
         a.Hstride = (int64_t)(m + 1) * m;
         a.Hld = m + 1;
@@ -1034,11 +672,11 @@ bool arnoldi(const Pencil& P, const sim_options& opt, JobSpace& js, const double
         a.meff = js.meff;
         a.istat = js.istat;
         a.single = single_pass ? 1 : 0;
-        gs_run(a, js.partial, half, na, st);
-        read_state(js, st);
+        gram_schmidt(a, na, st);
+        SIM_CUDA(cudaStreamSynchronize(st));
         std::vector<int> next;
         for (int q : act)
-            if (!g_pin.ist[q * IS_N + IS_BROKEN]) next.push_back(q);
+            if (!js.h_istat[q * IS_N + IS_BROKEN]) next.push_back(q);
         act.swap(next);
     }
     SIM_CUDA(cudaStreamSynchronize(st));
@@ -1072,13 +710,24 @@ JobSpace make_jobspace(DeviceArena& ar, cudaStream_t st, int J, int k, int m, in
     js.g = ar.get<double2>(tag + "g", (int64_t)J * (js.k + 1));
     js.scal = ar.get<double>(tag + "scal", (int64_t)J * SC_N);
     js.istat = ar.get<int>(tag + "istat", (int64_t)J * IS_N);
-    js.nchunk = cdiv_up(js.n, GS_CHUNK);
+    js.y = ar.get<double2>(tag + "y", (int64_t)J * js.k);
     js.pw = std::max(js.m + 2, js.k + 2);
-    js.partial = ar.get<double2>(tag + "partial", (int64_t)2 * J * js.nchunk * js.pw);
+    js.partial = ar.get<double2>(tag + "partial", gs_grid_partials(js.n, J, js.pw));
+    js.hsum = ar.get<double2>(tag + "hsum", (int64_t)2 * J * js.pw);
+    js.fin = ar.get<double>(tag + "fin", J);
+    js.need = ar.get<int>(tag + "need", J);
+    js.ticket = ar.get<int>(tag + "ticket", J);
+    js.nblk = cdiv_up(js.n, 256);
+    js.xpart = ar.get<double>(tag + "xpart", (int64_t)J * js.nblk);
+    js.rpart = ar.get<double>(tag + "rpart", (int64_t)J * js.nblk);
+    js.host = ar.job_host(tag, J);
+    js.h_istat = js.host->istat;
+    js.h_worst = js.host->worst;
     js.d_jobshift = ar.get<int>(tag + "jobshift", J);
     js.d_active = ar.get<int>(tag + "active", J);
     SIM_CUDA(cudaMemsetAsync(js.istat, 0, sizeof(int) * J * IS_N, st));
     SIM_CUDA(cudaMemsetAsync(js.scal, 0, sizeof(double) * J * SC_N, st));
+    SIM_CUDA(cudaMemsetAsync(js.ticket, 0, sizeof(int) * J, st));
     return js;
 }
 

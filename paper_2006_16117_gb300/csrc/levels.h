@@ -74,6 +74,27 @@ public:
         if (!h64_) SIM_CUDA(cudaMallocHost(&h64_, sizeof(int64_t) * 8));
         return h64_;
     }
+    // the host side of job space `tag` with room for J jobs, for a new run of jobs
+    JobHost* job_host(const std::string& tag, int J) {
+        JobHost& h = hosts_[tag];
+        if (h.J < J) {
+            if (h.istat) SIM_CUDA(cudaFreeHost(h.istat));
+            if (h.worst) SIM_CUDA(cudaFreeHost(h.worst));
+            if (h.act) SIM_CUDA(cudaFreeHost(h.act));
+            h.istat = nullptr;
+            h.worst = nullptr;
+            h.act = nullptr;
+            h.J = 0;
+            SIM_CUDA(cudaMallocHost(&h.istat, sizeof(int) * IS_N * J));
+            SIM_CUDA(cudaMallocHost(&h.worst, sizeof(double) * J));
+            SIM_CUDA(cudaMallocHost(&h.act, sizeof(int) * J));
+            h.J = J;
+        }
+        if (!h.act_ev) SIM_CUDA(cudaEventCreateWithFlags(&h.act_ev, cudaEventDisableTiming));
+        h.uploaded.clear();
+        h.usual_steps = 0;
+        return &h;
+    }
     void release(const std::string& name) {
         auto it = bufs_.find(name);
         if (it != bufs_.end()) {
@@ -93,6 +114,7 @@ private:
         size_t bytes;
     };
     std::map<std::string, Buf> bufs_;
+    std::map<std::string, JobHost> hosts_;
     int64_t* h64_ = nullptr;
     size_t total_ = 0;
 };

@@ -28,6 +28,7 @@
 // the direct evaluation (k_eval_level).
 #include <cfloat>
 
+#include "fp64.cuh"
 #include "hess.cuh"
 #include "internal.h"
 #include "levels.h"
@@ -46,20 +47,6 @@ __device__ __forceinline__ double2 csqrt_s(double2 z) {
 }
 
 }  // namespace
-
-// 1 / sqrt(d) for a d well inside the range of normal numbers: an FP32 seed y0 of
-// d scaled by an even power of two (exponent arithmetic), then one third-order
-// Newton step y0 + y0 t (1/2 + 3/8 t) with t = 1 - d y0^2: five FP64 operations.
-__device__ __forceinline__ double rsqrt_nr(double d) {
-    const uint32_t hd = (uint32_t)__double2hiint(d), ld = (uint32_t)__double2loint(d);
-    const int e = ((int)(hd >> 20) - 1023) & ~1;  // even; d 2^-e in [1, 4)
-    const float f = __uint_as_float((((hd >> 20) - 1023u - (uint32_t)e + 127u) << 23) | ((hd & 0xFFFFFu) << 3) | (ld >> 29));
-    const uint32_t g = __float_as_uint(rsqrtf(f));  // (0.5, 1]
-    const double y0 = __hiloint2double((int)((((g >> 23) - 127u + 1023u - (uint32_t)(e / 2)) << 20) | ((g & 0x7FFFFFu) >> 3)),
-                                       (int)(g << 29));
-    const double t = fma(-(d * y0), y0, 1.0);
-    return fma(y0 * t, fma(0.375, t, 0.5), y0);
-}
 
 // The FP64 pipe takes 64 clocks of its scheduler for a warp instruction, however
 // few lanes are active, so k_schur spreads every rotation over lanes and warps
