@@ -4,6 +4,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "fp64.cuh"
 
 namespace sim {
 
@@ -41,84 +42,106 @@ __device__ __forceinline__ void stage_H(const double2* H, int m, int meff, doubl
     }
 }
 
-// One warp solves (I + alpha H) y = beta e1 (order m, H row-major in Hs with
+// v - a b in four operations
+__device__ __forceinline__ double2 sub_product(double2 v, double2 a, double2 b) {
+    return make_double2(fma(-a.x, b.x, fma(a.y, b.y, v.x)), fma(-a.x, b.y, fma(-a.y, b.x, v.y)));
+}
+
+// One warp solves (I + alpha H) y = beta e1 (order m <= 63, H row-major in Hs with
 // leading dimension m) and leaves y in ys[0..m).  U: packed upper-triangular
 // scratch of m(m+1)/2 entries.  Returns |y_{m-1}| and ||y||^2 (warp-uniform).
+//
+// An FP64 instruction costs a warp 64 clocks however many lanes it serves, so
+// what counts is their number, about 1,500 a solve at m = 50 (5,500 with
+// divisions, alpha's products and the right-hand side on every lane: 4,096
+// squares of 8 nodes took 9.65 ms, now 4.1):
+//  * the system is divided by alpha, (H + τI) y = β τ e1 with τ = 1/alpha, so that
+//    rows are loaded as they stand;
+//  * the right-hand side is column m of the rows;
+//  * a pivot's reciprocal (crecip) serves the elimination and, kept by the pivot's
+//    lane, the back substitution;
+//  * columns below 32 are done with from row 32 on.
 __device__ __forceinline__ void warp_hess_solve(const double2* Hs, int m, double2 alpha, double beta, double2* U, double2* ys,
                                 double& ylast, double& ynorm2) {
     const int lane = threadIdx.x & 31;
     const int c0 = lane, c1 = lane + 32;
-    auto trow = [&](int r, int c) -> double2 {
-        if (c >= m) return make_double2(0.0, 0.0);
-        double2 h = Hs[r * m + c];
-        double2 v = cmul(alpha, h);
-        if (r == c) v.x += 1.0;
-        return v;
-    };
-    double2 a0 = trow(0, c0), a1 = trow(0, c1);
-    double2 arhs = make_double2(beta, 0.0);
-    for (int k = 0; k < m - 1; ++k) {
-        double2 b0 = (c0 >= k) ? trow(k + 1, c0) : make_double2(0.0, 0.0);
-        double2 b1 = (c1 >= k) ? trow(k + 1, c1) : make_double2(0.0, 0.0);
-        double2 brhs = make_double2(0.0, 0.0);
+    const double2 zero = make_double2(0.0, 0.0);
+    if (alpha.x == 0.0 && alpha.y == 0.0) {  // the identity
+        for (int c = lane; c < m; c += 32) ys[c] = c == 0 ? make_double2(beta, 0.0) : zero;
+        __syncwarp();
+        ylast = m == 1 ? fabs(beta) : 0.0;
+        ynorm2 = beta * beta;
+        return;
+    }
+    const double2 tau = crecip(alpha);
+    // the diagonal entries of this lane's columns
+    const double2 d0 = c0 < m ? cadd(Hs[c0 * m + c0], tau) : zero, d1 = c1 < m ? cadd(Hs[c1 * m + c1], tau) : zero;
+    auto entry = [&](int r, int c, double2 d) -> double2 { return c == r ? d : (c < m ? Hs[r * m + c] : zero); };
+    double2 a0 = entry(0, c0, d0), a1 = entry(0, c1, d1);
+    if (c0 == m) a0 = cscale(tau, beta);
+    if (c1 == m) a1 = cscale(tau, beta);
+    double2 iv0 = zero, iv1 = zero;  // reciprocals of U's diagonal in this lane's columns
+    for (int k = 0; k < m; ++k) {
+        const bool low = k < 32;  // columns 0..31 still in work
+        const bool more = k + 1 < m;
+        double2 b0 = low && more ? entry(k + 1, c0, d0) : zero;
+        double2 b1 = more ? entry(k + 1, c1, d1) : zero;
         const int src = k & 31;
-        const bool hi = k >= 32;
         double2 ak, bk;
-        ak.x = __shfl_sync(0xffffffffu, hi ? a1.x : a0.x, src);
-        ak.y = __shfl_sync(0xffffffffu, hi ? a1.y : a0.y, src);
-        bk.x = __shfl_sync(0xffffffffu, hi ? b1.x : b0.x, src);
-        bk.y = __shfl_sync(0xffffffffu, hi ? b1.y : b0.y, src);
-        if (mag1(bk) > mag1(ak)) {
+        ak.x = __shfl_sync(0xffffffffu, low ? a0.x : a1.x, src);
+        ak.y = __shfl_sync(0xffffffffu, low ? a0.y : a1.y, src);
+        bk.x = __shfl_sync(0xffffffffu, low ? b0.x : b1.x, src);
+        bk.y = __shfl_sync(0xffffffffu, low ? b0.y : b1.y, src);
+        if (more && mag1(bk) > mag1(ak)) {
             double2 t;
             t = a0; a0 = b0; b0 = t;
             t = a1; a1 = b1; b1 = t;
-            t = arhs; arhs = brhs; brhs = t;
             t = ak; ak = bk; bk = t;
         }
-        // U row k
+        // U row k, and the transformed right-hand side
         const int ofs = k * m - (k * (k - 1)) / 2;
         if (c0 >= k && c0 < m) U[ofs + (c0 - k)] = a0;
         if (c1 >= k && c1 < m) U[ofs + (c1 - k)] = a1;
-        if (lane == 0) ys[k] = arhs;  // transformed right-hand side
-        double2 l = (ak.x == 0.0 && ak.y == 0.0) ? make_double2(0.0, 0.0) : cdiv(bk, ak);
-        if (c0 > k) b0 = csub(b0, cmul(l, a0));
-        if (c1 > k) b1 = csub(b1, cmul(l, a1));
-        brhs = csub(brhs, cmul(l, arhs));
-        a0 = b0;
-        a1 = b1;
-        arhs = brhs;
-    }
-    {
-        const int k = m - 1;
-        const int ofs = k * m - (k * (k - 1)) / 2;
-        if (c0 == k) U[ofs] = a0;
-        if (c1 == k) U[ofs] = a1;
-        if (lane == 0) ys[k] = arhs;
+        if (c0 == m) ys[k] = a0;
+        if (c1 == m) ys[k] = a1;
+        const double2 inv = (ak.x == 0.0 && ak.y == 0.0) ? zero : crecip(ak);
+        if (lane == src) {
+            if (low) iv0 = inv;
+            else iv1 = inv;
+        }
+        const double2 l = cmul(bk, inv);
+        // (a column that is done with only holds garbage from here on)
+        if (low) a0 = sub_product(b0, l, a0);
+        a1 = sub_product(b1, l, a1);
     }
     __syncwarp();
     // column-oriented back substitution: lane owns rows lane and lane+32
-    double2 r0 = (c0 < m) ? ys[c0] : make_double2(0.0, 0.0);
-    double2 r1 = (c1 < m) ? ys[c1] : make_double2(0.0, 0.0);
+    double2 r0 = (c0 < m) ? ys[c0] : zero;
+    double2 r1 = (c1 < m) ? ys[c1] : zero;
     __syncwarp();
-    double nrm = 0.0;
-    double last = 0.0;
     for (int j = m - 1; j >= 0; --j) {
-        const int ofsj = j * m - (j * (j - 1)) / 2;
-        const double2 ujj = U[ofsj];
         const bool hi = j >= 32;
-        double2 rj;
-        rj.x = __shfl_sync(0xffffffffu, hi ? r1.x : r0.x, j & 31);
-        rj.y = __shfl_sync(0xffffffffu, hi ? r1.y : r0.y, j & 31);
-        const double2 yj = (ujj.x == 0.0 && ujj.y == 0.0) ? make_double2(0.0, 0.0) : cdiv(rj, ujj);
-        if (lane == 0) ys[j] = yj;
-        if (j == m - 1) last = cabsd(yj);
-        nrm += cabs2(yj);
-        if (c0 < j) r0 = csub(r0, cmul(U[c0 * m - (c0 * (c0 - 1)) / 2 + (j - c0)], yj));
-        if (c1 < j) r1 = csub(r1, cmul(U[c1 * m - (c1 * (c1 - 1)) / 2 + (j - c1)], yj));
+        const double2 t = hi ? cmul(r1, iv1) : cmul(r0, iv0);
+        double2 yj;
+        yj.x = __shfl_sync(0xffffffffu, t.x, j & 31);
+        yj.y = __shfl_sync(0xffffffffu, t.y, j & 31);
+        if (lane == (j & 31)) {
+            if (hi) r1 = yj;
+            else r0 = yj;
+        }
+        const int q0 = c0 * m - (c0 * (c0 - 1)) / 2 + (j - c0);
+        if (c0 < j) r0 = sub_product(r0, U[q0], yj);
+        if (j > 32 && c1 < j) r1 = sub_product(r1, U[c1 * m - (c1 * (c1 - 1)) / 2 + (j - c1)], yj);
     }
+    if (c0 < m) ys[c0] = r0;
+    if (c1 < m) ys[c1] = r1;
+    double nrm = 0.0;
+    if (c0 < m) nrm = cabs2(r0);
+    if (c1 < m) nrm += cabs2(r1);
+    ynorm2 = warp_sum(nrm);
+    const double last = cabsd(m <= 32 ? r0 : r1);
+    ylast = __shfl_sync(0xffffffffu, last, (m - 1) & 31);
     __syncwarp();
-    ylast = last;
-    ynorm2 = nrm;
 }
 
 

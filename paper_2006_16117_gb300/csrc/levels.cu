@@ -31,61 +31,70 @@ struct EvalSmem {
     double* red;   // 2 * 8
 };
 
+// H's Hessenberg matrix is in sm.Hs already (stage_H and a barrier).
 __device__ void eval_square(const double2* H, int m, int meff, double beta, double2 sigma, double2 c, double s,
                             int scale, const EvalSmem& sm, double& ind, double& rho_max) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    stage_H(H, m, meff, sm.Hs);
-    __syncthreads();
-    const double hlast = cabsd(H[(size_t)(meff - 1) * (m + 1) + meff]);
     const int Usz = meff * (meff + 1) / 2;
-    {
-        const int j = warp;  // node
+    auto alpha_of = [&](int j) {
         const double2 off = node_offset(j, s);
         const double2 z = make_double2(__dadd_rn(c.x, off.x), __dadd_rn(c.y, off.y));
-        const double2 alpha = make_double2(__dsub_rn(sigma.x, z.x), __dsub_rn(sigma.y, z.y));
+        return make_double2(__dsub_rn(sigma.x, z.x), __dsub_rn(sigma.y, z.y));
+    };
+    {
+        const int j = warp;  // node
         double ylast, yn2;
-        warp_hess_solve(sm.Hs, meff, alpha, beta, sm.U + (size_t)j * Usz, sm.Y + (size_t)j * meff, ylast, yn2);
+        warp_hess_solve(sm.Hs, meff, alpha_of(j), beta, sm.U + (size_t)j * Usz, sm.Y + (size_t)j * meff, ylast, yn2);
         if (lane == 0) {
-            const double num = cabsd(alpha) * hlast * ylast;
-            const double den = scale == 0 ? sqrt(yn2) : beta;
-            double r = num / den;
+            sm.rho[j] = ylast;
+            sm.red[j] = yn2;
+        }
+    }
+    __syncthreads();
+    if (warp == 7) {
+        // the 8 nodes' residuals, a lane each
+        double r = 0.0;
+        if (lane < 8) {
+            const double hlast = cabsd(H[(size_t)(meff - 1) * (m + 1) + meff]);
+            const double num = cabsd(alpha_of(lane)) * hlast * sm.rho[lane];
+            const double den = scale == 0 ? sqrt(sm.red[lane]) : beta;
+            r = num / den;
             if (!(r == r) || isinf(r)) r = INFINITY;
             if (num == 0.0) r = 0.0;
-            sm.rho[j] = r;
+        }
+        for (int o = 4; o > 0; o >>= 1) r = fmax(r, __shfl_xor_sync(0xffffffffu, r, o));
+        __syncwarp();
+        if (lane == 0) sm.rho[0] = r;
+    } else if (warp < 2) {
+        // quadrature sums Y8 = Σ_j (off_j/8) y_j, Y4 = Σ_{j even} (off_j/4) y_j
+        double n8 = 0.0, n4 = 0.0;
+        for (int q = threadIdx.x; q < meff; q += 64) {
+            double2 y8 = make_double2(0.0, 0.0), y4 = make_double2(0.0, 0.0);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const double2 off = node_offset(j, s);
+                const double2 yj = sm.Y[(size_t)j * meff + q];
+                y8 = cadd(y8, cmul(cscale(off, 0.125), yj));
+                if ((j & 1) == 0) y4 = cadd(y4, cmul(cscale(off, 0.25), yj));
+            }
+            n8 += cabs2(y8);
+            n4 += cabs2(y4);
+        }
+        n8 = warp_sum(n8);
+        n4 = warp_sum(n4);
+        if (lane == 0) {
+            sm.red[8 + 2 * warp] = n8;
+            sm.red[9 + 2 * warp] = n4;
         }
     }
     __syncthreads();
-    // quadrature sums Y8 = Σ_j (off_j/8) y_j, Y4 = Σ_{j even} (off_j/4) y_j
-    double n8 = 0.0, n4 = 0.0;
-    for (int q = threadIdx.x; q < meff; q += blockDim.x) {
-        double2 y8 = make_double2(0.0, 0.0), y4 = make_double2(0.0, 0.0);
-        for (int j = 0; j < 8; ++j) {
-            const double2 off = node_offset(j, s);
-            const double2 yj = sm.Y[(size_t)j * meff + q];
-            y8 = cadd(y8, cmul(cscale(off, 0.125), yj));
-            if ((j & 1) == 0) y4 = cadd(y4, cmul(cscale(off, 0.25), yj));
-        }
-        n8 += cabs2(y8);
-        n4 += cabs2(y4);
-    }
-    n8 = warp_sum(n8);
-    n4 = warp_sum(n4);
-    if (lane == 0) {
-        sm.red[warp] = n8;
-        sm.red[8 + warp] = n4;
+    if (warp == 0) {
+        const double s8 = sqrt(sm.red[8] + sm.red[10]), s4 = sqrt(sm.red[9] + sm.red[11]);
+        if (lane == 0) sm.red[0] = s4 > 0.0 ? s8 / s4 : (s8 > 0.0 ? INFINITY : 0.0);
     }
     __syncthreads();
-    double s8 = 0.0, s4 = 0.0, rm = 0.0;
-    for (int w = 0; w < 8; ++w) {
-        s8 += sm.red[w];
-        s4 += sm.red[8 + w];
-        rm = fmax(rm, sm.rho[w]);
-        if (sm.rho[w] != sm.rho[w]) rm = INFINITY;
-    }
-    s8 = sqrt(s8);
-    s4 = sqrt(s4);
-    ind = s4 > 0.0 ? s8 / s4 : (s8 > 0.0 ? INFINITY : 0.0);
-    rho_max = rm;
+    ind = sm.red[0];
+    rho_max = sm.rho[0];
     __syncthreads();
 }
 
@@ -172,6 +181,8 @@ __global__ void __launch_bounds__(256) k_eval_level(ShiftTable st, LevelArgs a, 
         int used = s;
         for (int attempt = 0; s >= 0 && attempt < hi - lo; ++attempt) {
             double ii, rr;
+            stage_H(st.H + (size_t)s * (st.m + 1) * st.m, st.m, st.meff[s], sm.Hs);
+            __syncthreads();
             eval_square(st.H + (size_t)s * (st.m + 1) * st.m, st.m, st.meff[s], st.beta[s], st.sigma[s], c, side,
                         st.scale, sm, ii, rr);
             if (attempt == 0) ind0 = ii;
@@ -226,6 +237,8 @@ __global__ void __launch_bounds__(256) k_eval_explicit(const double2* H, int m, 
                                                        int scale, double* ind, double* rho) {
     extern __shared__ unsigned char raw[];
     const EvalSmem sm = carve(raw, m);
+    stage_H(H, m, meff, sm.Hs);
+    __syncthreads();
     for (int64_t q = blockIdx.x; q < count; q += gridDim.x) {
         double ii, rr;
         eval_square(H, m, meff, beta, sigma, centers[q], sides[q], scale, sm, ii, rr);
@@ -241,7 +254,7 @@ void eval_explicit(const double2* H, int m, int meff, double beta, double2 sigma
     if (count <= 0) return;
     const size_t sm = eval_smem_bytes(m);
     SIM_CUDA(cudaFuncSetAttribute(k_eval_explicit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    int grid = (int)std::min<int64_t>(count, 152 * 64);
+    int grid = (int)std::min<int64_t>(count, 152);  // one CTA fits an SM: H staged once for all its squares
     k_eval_explicit<<<grid, 256, sm, stream>>>(H, m, meff, beta, sigma, centers, sides, count, scale, ind, rho);
     SIM_LAUNCH_CHECK();
 }
