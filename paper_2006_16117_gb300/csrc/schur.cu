@@ -18,7 +18,7 @@
 // whole rows and columns with the rotations accumulated into the two rows of Z
 // the level needs (the first and the last: a row of Z evolves on its own
 // under the column rotations).
-// k_eval_schur: one lane per quadrature node (a warp holds the 8 nodes of 4
+// k_eval_schur: one lane per quadrature node (a CTA holds the 8 nodes of 4
 // squares), so every FP64 instruction does useful work in all lanes; T's
 // entries are warp-uniform loads when the 4 squares share a shift (children
 // of one square do).  The squares their own shift does not resolve are then
@@ -256,9 +256,16 @@ __global__ void __launch_bounds__(SC_THREADS) k_schur(const double2* Hall, int m
     if (tid == 0) ok_all[s] = fail ? 0 : 1;
 }
 
-// 8 nodes per square, 4 squares per warp, SE_WARPS warps per CTA; x_j of every
-// lane in shared memory as [i][lane] (conflict-free 16-byte accesses).
+// 4 squares of 8 nodes per CTA, a lane per node in each of its SE_WARPS warps, the
+// rows of the triangular solve dealt out to the warps (row i to warp i mod 4), so
+// that one square's chain uses all four FP64 pipes of an SM: a level often holds
+// fewer squares than the GPU has warps, and then the time is one warp's chain
+// (m = 50, 1,300 squares: 373 us a level with whole solves per warp, now about 190).  Column by column from
+// the last: the owner of row i forms x_i from its sum and sends it round through
+// shared memory; every warp then adds T_ri x_i to its rows r < i, whose T_ri it
+// loaded one column ahead.
 constexpr int SE_WARPS = 4;
+constexpr int SE_ROWS = 13;  // rows per warp: m <= 52
 
 // ALL = false: item t is square t against its own shift; a square it resolves
 //   gets its results, the others todo[q] = 1.
@@ -269,17 +276,14 @@ template <bool ALL>
 __global__ void __launch_bounds__(SE_WARPS * 32) k_eval_schur(ShiftTable st, LevelArgs a, uint8_t* todo,
                                                               const int64_t* list, int smax, int64_t nitems,
                                                               double* rind, double* rrho, uint8_t* rbad) {
-    const double2* Tall = st.schT;
-    const double2* Call = st.schC;
-    const double2* Qall = st.schQ;
     const int* ok_all = st.schOK;
-    extern __shared__ double2 sh_x[];
+    __shared__ double2 xs[2][32];             // x_i of every node, alternating
+    __shared__ double red[SE_WARPS][5][32];   // yl (2), ||x||^2, the quadrature sums' squares
+    __shared__ int s_bad;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int m = st.m;
-    double2* xs = sh_x + (size_t)warp * m * 32;
     const int j = lane & 7;  // node
-    const int64_t nwarps = (int64_t)gridDim.x * SE_WARPS;
-    for (int64_t t0 = ((int64_t)blockIdx.x * SE_WARPS + warp) * 4; t0 < nitems; t0 += nwarps * 4) {
+    for (int64_t t0 = (int64_t)blockIdx.x * 4; t0 < nitems; t0 += (int64_t)gridDim.x * 4) {
         const int64_t t = t0 + (lane >> 3);
         int64_t q = t;
         bool active = t < nitems;
@@ -307,106 +311,158 @@ __global__ void __launch_bounds__(SE_WARPS * 32) k_eval_schur(ShiftTable st, Lev
             }
             good = ok_all[s] != 0;
             n = good ? st.meff[s] : 0;
+        } else {
+            s = 0;
         }
         const double2 c = square_center(re_lo, im_lo, side, active ? a.ix[q] : 0, active ? a.iy[q] : 0);
         const double2 off = node_offset(j, side);
         const double2 z = make_double2(__dadd_rn(c.x, off.x), __dadd_rn(c.y, off.y));
         const double2 sig = active ? st.sigma[s] : make_double2(0.0, 0.0);
         const double2 alpha = make_double2(__dsub_rn(sig.x, z.x), __dsub_rn(sig.y, z.y));
-        const double2 w8 = cscale(off, 0.125), w4 = (j & 1) == 0 ? cscale(off, 0.25) : make_double2(0.0, 0.0);
-        const double2* T = Tall + (size_t)s * m * m;
-        const double2* Cv = Call + (size_t)s * m;
-        const double2* Qv = Qall + (size_t)s * m;
-        int nmax = n;
-        for (int o = 16; o > 0; o >>= 1) nmax = max(nmax, __shfl_xor_sync(0xffffffffu, nmax, o));
+        const double2 w8 = cscale(off, 0.125);
+        const double2* T = st.schT + (size_t)s * m * m;
+        const double2* Cv = st.schC + (size_t)s * m;
+        const double2* Qv = st.schQ + (size_t)s * m;
+        const int nmax = __reduce_max_sync(0xffffffffu, n);  // every warp holds the same nodes
+        if (threadIdx.x == 0) s_bad = 0;
+        // this warp's rows r = warp + 4 u: sums, reciprocals of 1 + α T_rr, next column's T
+        double2 acc[SE_ROWS], tn[SE_ROWS];
+#pragma unroll
+        for (int u = 0; u < SE_ROWS; ++u) {
+            acc[u] = make_double2(0.0, 0.0);
+            const int r = warp + SE_WARPS * u, i = n - 1;
+            tn[u] = r < i ? __ldg(T + (size_t)r * m + i) : make_double2(0.0, 0.0);
+        }
         double2 yl = make_double2(0.0, 0.0);
         double yn2 = 0.0, n8 = 0.0, n4 = 0.0;
-        for (int i = nmax - 1; i >= 0; --i) {
-            double2 xi = make_double2(0.0, 0.0);
-            if (i < n) {
-                // x_i = (c_i - α Σ_{k>i} T_ik x_k) / (1 + α T_ii)
-                double2 acc = make_double2(0.0, 0.0);
-                const double2* Ti = T + (size_t)i * m;
-                int k = i + 1;
-                for (; k + 1 < n; k += 2) {
-                    const double2 t0 = __ldg(Ti + k), t1 = __ldg(Ti + k + 1);
-                    const double2 x0 = xs[(size_t)k * 32 + lane], x1 = xs[(size_t)(k + 1) * 32 + lane];
-                    acc.x = fma(t0.x, x0.x, acc.x);
-                    acc.x = fma(-t0.y, x0.y, acc.x);
-                    acc.y = fma(t0.x, x0.y, acc.y);
-                    acc.y = fma(t0.y, x0.x, acc.y);
-                    acc.x = fma(t1.x, x1.x, acc.x);
-                    acc.x = fma(-t1.y, x1.y, acc.x);
-                    acc.y = fma(t1.x, x1.y, acc.y);
-                    acc.y = fma(t1.y, x1.x, acc.y);
-                }
-                if (k < n) {
-                    const double2 t0 = __ldg(Ti + k);
-                    const double2 x0 = xs[(size_t)k * 32 + lane];
-                    acc.x = fma(t0.x, x0.x, acc.x);
-                    acc.x = fma(-t0.y, x0.y, acc.x);
-                    acc.y = fma(t0.x, x0.y, acc.y);
-                    acc.y = fma(t0.y, x0.x, acc.y);
-                }
-                const double2 tii = __ldg(Ti + i);
-                double2 den = cmul(alpha, tii);
-                den.x += 1.0;
-                const double2 rhs = csub(__ldg(Cv + i), cmul(alpha, acc));
-                if (den.x == 0.0 && den.y == 0.0) good = false;
-                else xi = cdiv(rhs, den);
-                xs[(size_t)i * 32 + lane] = xi;
-                const double2 ql = __ldg(Qv + i);
-                yl = cadd(yl, cmul(ql, xi));
-                yn2 += cabs2(xi);
+        bool zero_pivot = false;
+        // this warp's next row: 1 / (1 + α T_rr) and c_r, made ahead of its turn
+        double2 inv, cr;
+        auto next_row = [&](int r) {
+            inv = cr = make_double2(0.0, 0.0);
+            if (r >= 0 && r < n) {
+                const double2 trr = __ldg(T + (size_t)r * m + r);
+                cr = __ldg(Cv + r);
+                double2 den;
+                den.x = fma(alpha.x, trr.x, fma(-alpha.y, trr.y, 1.0));
+                den.y = fma(alpha.x, trr.y, alpha.y * trr.x);
+                if (den.x == 0.0 && den.y == 0.0) zero_pivot = true;
+                else inv = crecip(den);
             }
-            // the two quadrature sums of component i over the square's 8 lanes
-            double2 p8 = cmul(w8, xi), p4 = cmul(w4, xi);
+        };
+        {
+            const int r = nmax - 1 - ((nmax - 1 - warp) & (SE_WARPS - 1));  // the last row of this warp
+            next_row(r);
+        }
+        __syncthreads();
+        for (int i = nmax - 1; i >= 0; --i) {
+            const bool mine = (i & (SE_WARPS - 1)) == warp;
+            double2 xi = make_double2(0.0, 0.0);
+            if (mine) {
+                // x_i = (c_i - α Σ_{k>i} T_ik x_k) / (1 + α T_ii)
+                double2 sum = make_double2(0.0, 0.0);
+#pragma unroll
+                for (int u = 0; u < SE_ROWS; ++u)
+                    if (u == i / SE_WARPS) sum = acc[u];
+                const double2 rhs = make_double2(fma(-alpha.x, sum.x, fma(alpha.y, sum.y, cr.x)),
+                                                 fma(-alpha.x, sum.y, fma(-alpha.y, sum.x, cr.y)));
+                xi = cmul(rhs, inv);
+                xs[i & 1][lane] = xi;
+            }
+            __syncthreads();
+            const double2 x = xs[i & 1][lane];
+#pragma unroll
+            for (int u = SE_ROWS - 1; u >= 0; --u) {
+                const int r = warp + SE_WARPS * u;
+                if (r < i) {  // warp-uniform
+                    // (a node of a smaller order has x = 0 and T = 0 in the columns beyond it)
+                    acc[u] = cfma(tn[u], x, acc[u]);
+                    tn[u] = r < i - 1 && i - 1 < n ? __ldg(T + (size_t)r * m + i - 1) : make_double2(0.0, 0.0);
+                }
+            }
+            if (mine) {
+                // off the chain: what the level needs of component i, and this warp's next row
+                if (i < n) {
+                    yl = cfma(__ldg(Qv + i), xi, yl);
+                    yn2 = fma(xi.x, xi.x, fma(xi.y, xi.y, yn2));
+                }
+                // the quadrature sums of component i over the square's 8 lanes: lanes with
+                // bit 2 clear sum the real parts, the others the imaginary ones; even
+                // lanes then hold the coarse rule's sum (half of it: its weights are twice
+                // the fine rule's), and all lanes add the odd nodes for the fine rule
+                const double2 p = cmul(w8, xi);
+                const bool up = (lane & 4) != 0;
+                double v = (up ? p.y : p.x) + __shfl_xor_sync(0xffffffffu, up ? p.x : p.y, 4);
+                v += __shfl_xor_sync(0xffffffffu, v, 2);
+                n4 = fma(v, v, n4);
+                v += __shfl_xor_sync(0xffffffffu, v, 1);
+                n8 = fma(v, v, n8);
+                next_row(i - SE_WARPS);
+            }
+        }
+        if (zero_pivot) good = false;
+        red[warp][0][lane] = yl.x;
+        red[warp][1][lane] = yl.y;
+        red[warp][2][lane] = yn2;
+        red[warp][3][lane] = n8;
+        red[warp][4][lane] = n4;
+        if (__any_sync(0xffffffffu, zero_pivot)) {
+            // which nodes: a bit per lane
+            const unsigned b = __ballot_sync(0xffffffffu, zero_pivot);
+            if (lane == 0) atomicOr(&s_bad, (int)b);
+        }
+        __syncthreads();
+        if (warp == 0) {
+            double v[5];
+#pragma unroll
+            for (int e = 0; e < 5; ++e) {
+                v[e] = red[0][e][lane];
+#pragma unroll
+                for (int w = 1; w < SE_WARPS; ++w) v[e] += red[w][e][lane];
+            }
+            if ((unsigned)s_bad >> lane & 1u) good = false;
+            yl = make_double2(v[0], v[1]);
+            yn2 = v[2];
+            // real plus imaginary parts' squares; the coarse rule's from an even lane
+            n8 = v[3] + __shfl_xor_sync(0xffffffffu, v[3], 4);
+            n4 = v[4] + __shfl_xor_sync(0xffffffffu, v[4], 4);
+            n4 = 4.0 * __shfl_sync(0xffffffffu, n4, lane & ~7);
+            // residual of Eq. eq:error at this node, as the direct evaluation forms it
+            double r = 0.0;
+            if (active && good && n > 0) {
+                const double hlast = cabsd(st.H[(size_t)s * (m + 1) * m + (size_t)(n - 1) * (m + 1) + n]);
+                const double num = cabsd(alpha) * hlast * cabsd(yl);
+                const double den = st.scale == 0 ? sqrt(yn2) : st.beta[s];
+                r = num / den;
+                if (!(r == r) || isinf(r)) r = INFINITY;
+                if (num == 0.0) r = 0.0;
+            }
+            int bad = (active && (!good || n == 0)) ? 1 : 0;
+            double rmax = r;
 #pragma unroll
             for (int o = 1; o < 8; o <<= 1) {
-                p8.x += __shfl_xor_sync(0xffffffffu, p8.x, o);
-                p8.y += __shfl_xor_sync(0xffffffffu, p8.y, o);
-                p4.x += __shfl_xor_sync(0xffffffffu, p4.x, o);
-                p4.y += __shfl_xor_sync(0xffffffffu, p4.y, o);
+                rmax = fmax(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
+                bad |= __shfl_xor_sync(0xffffffffu, bad, o);
             }
-            n8 += cabs2(p8);
-            n4 += cabs2(p4);
-        }
-        __syncwarp();
-        // residual of Eq. eq:error at this node, as the direct evaluation forms it
-        double r = 0.0;
-        if (active && good && n > 0) {
-            const double hlast = cabsd(st.H[(size_t)s * (m + 1) * m + (size_t)(n - 1) * (m + 1) + n]);
-            const double num = cabsd(alpha) * hlast * cabsd(yl);
-            const double den = st.scale == 0 ? sqrt(yn2) : st.beta[s];
-            r = num / den;
-            if (!(r == r) || isinf(r)) r = INFINITY;
-            if (num == 0.0) r = 0.0;
-        }
-        int bad = (active && (!good || n == 0)) ? 1 : 0;
-        double rmax = r;
-#pragma unroll
-        for (int o = 1; o < 8; o <<= 1) {
-            rmax = fmax(rmax, __shfl_xor_sync(0xffffffffu, rmax, o));
-            bad |= __shfl_xor_sync(0xffffffffu, bad, o);
-        }
-        if (ALL && t < nitems && j == 0) {
-            const double s8 = sqrt(n8), s4 = sqrt(n4);
-            rind[t] = s4 > 0.0 ? s8 / s4 : (s8 > 0.0 ? INFINITY : 0.0);
-            rrho[t] = active ? rmax : INFINITY;
-            rbad[t] = active ? (uint8_t)bad : (uint8_t)0;
-        }
-        if (!ALL && active && j == 0) {
             const double s8 = sqrt(n8), s4 = sqrt(n4);
             const double ind = s4 > 0.0 ? s8 / s4 : (s8 > 0.0 ? INFINITY : 0.0);
-            if (!bad && rmax <= st.eps) {
-                a.ind[q] = ind;
-                a.mark[q] = ind > st.delta0 ? 1 : 0;
-                a.flag[q] = 0;
-                todo[q] = 0;
-            } else {
-                todo[q] = 1;
+            if (ALL && t < nitems && j == 0) {
+                rind[t] = ind;
+                rrho[t] = active ? rmax : INFINITY;
+                rbad[t] = active ? (uint8_t)bad : (uint8_t)0;
+            }
+            if (!ALL && active && j == 0) {
+                if (!bad && rmax <= st.eps) {
+                    a.ind[q] = ind;
+                    a.mark[q] = ind > st.delta0 ? 1 : 0;
+                    a.flag[q] = 0;
+                    todo[q] = 0;
+                } else {
+                    todo[q] = 1;
+                }
             }
         }
+        __syncthreads();  // red, s_bad and xs are free again
     }
 }
 
@@ -486,12 +542,9 @@ __global__ void k_pick_shift(ShiftTable st, LevelArgs a, const int64_t* list, in
 
 void eval_level_schur(const ShiftTable& st, const LevelArgs& a, uint8_t* todo, cudaStream_t stream) {
     if (a.count <= 0) return;
-    const size_t sm = (size_t)SE_WARPS * st.m * 32 * sizeof(double2);
-    SIM_CUDA(cudaFuncSetAttribute(k_eval_schur<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    const int64_t warps = (a.count + 3) / 4;
-    const int grid = (int)std::min<int64_t>((warps + SE_WARPS - 1) / SE_WARPS, 152 * 16);
+    const int grid = (int)std::min<int64_t>((a.count + 3) / 4, 152 * 64);
     kprof_begin("eval_level_schur", stream);
-    k_eval_schur<false><<<grid, SE_WARPS * 32, sm, stream>>>(st, a, todo, nullptr, 1, a.count, nullptr, nullptr,
+    k_eval_schur<false><<<grid, SE_WARPS * 32, 0, stream>>>(st, a, todo, nullptr, 1, a.count, nullptr, nullptr,
                                                              nullptr);
     SIM_LAUNCH_CHECK();
     // per square: 8 triangular solves of order m (m²/2 complex multiply-adds each)
@@ -510,12 +563,9 @@ void eval_level_schur_retries(const ShiftTable& st, const LevelArgs& a, uint8_t*
     SIM_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), stream));
     k_list_todo<<<cdiv_up(a.count, 256), 256, 0, stream>>>(todo, a.count, list, cnt);
     SIM_LAUNCH_CHECK();
-    const size_t sm = (size_t)SE_WARPS * st.m * 32 * sizeof(double2);
-    SIM_CUDA(cudaFuncSetAttribute(k_eval_schur<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    const int64_t warps = (nitems + 3) / 4;
-    const int grid = (int)std::min<int64_t>((warps + SE_WARPS - 1) / SE_WARPS, 152 * 16);
+    const int grid = (int)std::min<int64_t>((nitems + 3) / 4, 152 * 64);
     kprof_begin("eval_level_schur", stream);
-    k_eval_schur<true><<<grid, SE_WARPS * 32, sm, stream>>>(st, a, todo, list, smax, nitems, rind, rrho, rbad);
+    k_eval_schur<true><<<grid, SE_WARPS * 32, 0, stream>>>(st, a, todo, list, smax, nitems, rind, rrho, rbad);
     SIM_LAUNCH_CHECK();
     k_pick_shift<<<cdiv_up(ntodo, 128), 128, 0, stream>>>(st, a, list, ntodo, smax, rind, rrho, rbad, todo);
     SIM_LAUNCH_CHECK();
