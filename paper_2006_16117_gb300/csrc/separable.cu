@@ -346,6 +346,9 @@ void separable_setup(Separable& S, DeviceArena& ar, cudaStream_t st, const std::
                                                          S.Q32[d], S.rho[d], S.irho[d], S.lam[d]);
         SIM_LAUNCH_CHECK();
         sep_split_tables(S.Q64[d], (int)N, S.Qh[d], S.Ql[d], st);
+        const int64_t Np = (N + 3) / 4 * 4;
+        S.Qp[d] = ar.get<float>(tag + "Qp", Np * Np);
+        sep_pad_table(S.Q32[d], (int)N, S.Qp[d], st);
     }
     int64_t n = 1;
     for (int d = 0; d < S.ndim; ++d) n *= S.dims[d];
@@ -364,7 +367,8 @@ void separable_apply(const Separable& S, int precision, const JobSpace& js, cons
     if (na <= 0) return;
     // the active list is already on the device (js.d_active) in this order
     kprof_begin("separable", st);
-    if (precision == SIM_FP64) apply_t<double, double>(S, js, na, in_slot, out_slot, d_sigma, ar, st);
+    if (precision != SIM_FP64 && S.tc && sep_fused_2d(S, js, na, in_slot, out_slot, d_sigma, st)) {
+    } else if (precision == SIM_FP64) apply_t<double, double>(S, js, na, in_slot, out_slot, d_sigma, ar, st);
     else apply_t<float, float>(S, js, na, in_slot, out_slot, d_sigma, ar, st);
     double flops = 0.0;
     for (int d = 0; d < S.ndim; ++d) flops += 2.0 * 4.0 * (double)js.n * (double)S.dims[d];  // 2 passes, 2 FMA

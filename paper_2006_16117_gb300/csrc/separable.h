@@ -34,6 +34,9 @@ struct Separable {
     // Q split for the tensor cores: Q = Qh + Ql, Qh exact in TF32 (FP32 tables)
     float* Qh[3] = {nullptr, nullptr, nullptr};
     float* Ql[3] = {nullptr, nullptr, nullptr};
+    // Q in FP32 for the fused kernel: rows and columns padded with zeros to a
+    // multiple of 4 (separable_fused.cu)
+    float* Qp[3] = {nullptr, nullptr, nullptr};
     bool tc = false;  // complex64 mode products on the tensor cores (separable_tc.cu)
     // per element, for the complex64 path: Π_d ρ_d^{-j_d} and Π_d ρ_d^{j_d} rounded
     // from FP64, and Σ_d λ_{d,k_d} in FP64 (so the denominator's cancellation
@@ -55,6 +58,12 @@ void separable_setup(Separable& S, DeviceArena& ar, cudaStream_t st, const std::
 // Y = X ×_axis Q for an axis of length N with inner stride P (separable_tc.cu).
 bool sep_mode_tc(const float2* cur, float2* nxt, const float* Qhi, const float* Qlo, int N, int64_t P, int64_t rows,
                  int64_t n, int na, cudaStream_t st);
+// The whole apply of a two-dimensional separable part in one kernel, a cluster per
+// job with its vector in shared memory (separable_fused.cu); false (nothing
+// launched) where the vector does not fit or the separate kernels are faster.
+bool sep_fused_2d(const Separable& S, const JobSpace& js, int na, int in_slot, int out_slot, const double2* d_sigma,
+                  cudaStream_t st);
+void sep_pad_table(const float* Q32, int N, float* Qp, cudaStream_t st);
 void sep_split_tables(const double* Q64, int N, float* Qhi, float* Qlo, cudaStream_t st);
 
 // z_job = (A_s - σ_job b I)^{-1} q_job for the active jobs (vector slots
