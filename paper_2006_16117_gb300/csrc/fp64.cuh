@@ -22,6 +22,28 @@ __device__ __forceinline__ double rsqrt_nr(double d) {
     return fma(y0 * t, fma(0.375, t, 0.5), y0);
 }
 
+// float <-> double by integer arithmetic: the conversion instructions go through
+// the FP64 pipe.  Same values, rounded to nearest even; what is not a normal number
+// on both sides (zero apart) takes the instruction.
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t b = __float_as_uint(f), e = (b >> 23) & 255u;
+    if ((b << 1) == 0u) return __hiloint2double((int)b, 0);
+    if (e == 0u || e == 255u) return (double)f;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + (896u << 20))), (int)(b << 29));
+}
+__device__ __forceinline__ float narrow(double d) {
+    const uint32_t h = (uint32_t)__double2hiint(d), l = (uint32_t)__double2loint(d);
+    const uint32_t e = (h >> 20) & 2047u;
+    if (((h << 1) | l) == 0u) return __uint_as_float(h);
+    if (e < 898u || e > 1149u) return (float)d;
+    uint32_t m = (((h & 0x7FFFFFFFu) - (896u << 20)) << 3) | (l >> 29);
+    const uint32_t rest = l & 0x1FFFFFFFu;
+    m += (rest > 0x10000000u || (rest == 0x10000000u && (m & 1u))) ? 1u : 0u;
+    return __uint_as_float((h & 0x80000000u) | m);
+}
+__device__ __forceinline__ float2 narrow(double2 v) { return make_float2(narrow(v.x), narrow(v.y)); }
+__device__ __forceinline__ double2 widen(float2 v) { return make_double2(widen(v.x), widen(v.y)); }
+
 // v 2^k, zero where v or the result is zero or subnormal
 __device__ __forceinline__ double scale2(double v, int k) {
     const uint32_t h = (uint32_t)__double2hiint(v);

@@ -11,9 +11,9 @@
 // values go back for the second Q_0.  Three cluster barriers an apply.
 //
 // A product is a GEMM of complex rows with a real symmetric matrix on the FP32
-// cores: a thread forms RT rows x 4 outputs, a complex value times a real one in
-// one paired FMA; the rows come from shared memory as broadcasts, Q through L1
-// (coalesced, four rows ahead in registers).  FP32 products need no splitting as
+// cores: a thread forms RT rows x KT outputs, a complex value times a real one in
+// one paired FMA; the rows come from shared memory, Q through a ring of stages
+// there.  FP32 products need no splitting as
 // on the tensor cores, and every value is summed in FP32 over its line in order.
 #include <cooperative_groups.h>
 
@@ -21,6 +21,7 @@
 #include <atomic>
 #include <cmath>
 
+#include "fp64.cuh"
 #include "internal.h"
 #include "levels.h"
 #include "separable.h"
@@ -35,63 +36,142 @@ constexpr int SF_T = 256;
 
 __host__ __device__ constexpr int pad4(int n) { return (n + 3) / 4 * 4; }
 
-// store(r, k, Σ_j X[r][j] Q[j][k]) for r < rows, k < N.  X: [rows][ldx] in shared
-// memory, zero from column N to ldx = pad4(N); Q: pad4(N) x pad4(N), zero beyond N.
-template <int RT, class F>
+__device__ __forceinline__ void copy_async_16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+constexpr int SF_STAGES = 3;
+// rows of Q per stage: three stages within 48 KB
+__host__ __device__ constexpr int stage_rows(int ldq) { return ldq <= 256 ? 16 : (ldq <= 512 ? 8 : 4); }
+__host__ __device__ constexpr size_t stage_floats(int N) { return (size_t)stage_rows(pad4(N)) * pad4(N); }
+
+// f.put(f.column(k), r, Σ_j X[r][j] Q[j][k]) for r < rows, k < N.  X: [rows][ldx] in
+// shared memory, zero from column N to ldx = pad4(N); Q: pad4(N) x pad4(N), zero
+// beyond N, streamed through three stages of shared memory (read directly, its L2
+// latency of about 370 clocks per two reduction steps was the time of a product).
+// A thread forms RT rows x KT columns at a time.  Every thread of the CTA calls it.
+template <int RT, int KT, class F>
 __device__ __forceinline__ void rows_times_q(const float2* X, int ldx, int rows, int N, const float* __restrict__ Q,
-                                             F store) {
-    const int ldq = pad4(N), nk = ldq / 4, nr = (rows + RT - 1) / RT;
-    for (int item = threadIdx.x; item < nk * nr; item += SF_T) {
-        const int k = item % nk * 4, r0 = item / nk * RT;
+                                             float* stage, const F& f) {
+    constexpr int K4 = KT / 4;
+    const int ldq = pad4(N), nk = (ldq + KT - 1) / KT, nr = (rows + RT - 1) / RT, items = nk * nr;
+    const int KC = stage_rows(ldq), nc = (ldq + KC - 1) / KC, per_stage = KC * ldq;
+    auto fill = [&](int c) {
+        if (c < nc) {
+            float* dst = stage + (size_t)(c % SF_STAGES) * per_stage;
+            const float* src = Q + (size_t)c * per_stage;
+            const int units = min(KC, ldq - c * KC) * ldq / 4;
+            for (int i = threadIdx.x; i < units; i += SF_T) copy_async_16(dst + 4 * i, src + 4 * i);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int first = 0; first < items; first += SF_T) {
+        const int item = min(first + (int)threadIdx.x, items - 1);
+        const bool valid = first + (int)threadIdx.x < items;
+        const bool busy = __any_sync(0xffffffffu, valid);
+        const int k = item % nk * KT, r0 = item / nk * RT;
         const float4* x[RT];
 #pragma unroll
         for (int r = 0; r < RT; ++r) x[r] = reinterpret_cast<const float4*>(X + (size_t)min(r0 + r, rows - 1) * ldx);
-        const float* q = Q + k;
-        float2 acc[RT][4];
+        int q[K4];
+#pragma unroll
+        for (int h = 0; h < K4; ++h) q[h] = min(k + 4 * h, ldq - 4);
+        float2 acc[RT][KT];
 #pragma unroll
         for (int r = 0; r < RT; ++r)
 #pragma unroll
-            for (int c = 0; c < 4; ++c) acc[r][c] = make_float2(0.f, 0.f);
-        float4 qn[4];
+            for (int c = 0; c < KT; ++c) acc[r][c] = make_float2(0.f, 0.f);
+        __syncthreads();  // the stages of the round before are free
 #pragma unroll
-        for (int j = 0; j < 4; ++j) qn[j] = __ldg(reinterpret_cast<const float4*>(q + (size_t)j * ldq));
-        for (int j0 = 0; j0 < ldq; j0 += 4) {
-            float4 qc[4];
+        for (int c = 0; c < SF_STAGES - 1; ++c) fill(c);
+        for (int c = 0; c < nc; ++c) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(SF_STAGES - 2) : "memory");
+            __syncthreads();  // chunk c is there, and chunk c - 1 has been read
+            fill(c + SF_STAGES - 1);
+            if (!busy) continue;
+            const float* Qs = stage + (size_t)(c % SF_STAGES) * per_stage;
+            const int jn = min(KC, ldq - c * KC), jx = c * KC / 2;
+#pragma unroll 4
+            for (int j = 0; j < jn; j += 2) {
+                float4 q0[K4], q1[K4];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) qc[j] = qn[j];
-            if (j0 + 4 < ldq) {
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    qn[j] = __ldg(reinterpret_cast<const float4*>(q + (size_t)(j0 + 4 + j) * ldq));
-            }
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const float4 q0 = qc[2 * h], q1 = qc[2 * h + 1];
+                for (int h = 0; h < K4; ++h) {
+                    q0[h] = *reinterpret_cast<const float4*>(Qs + (size_t)j * ldq + q[h]);
+                    q1[h] = *reinterpret_cast<const float4*>(Qs + (size_t)(j + 1) * ldq + q[h]);
+                }
 #pragma unroll
                 for (int r = 0; r < RT; ++r) {
-                    const float4 v = x[r][j0 / 2 + h];
+                    const float4 v = x[r][jx + j / 2];
                     const float2 v0 = make_float2(v.x, v.y), v1 = make_float2(v.z, v.w);
-                    acc[r][0] = __ffma2_rn(make_float2(q0.x, q0.x), v0, acc[r][0]);
-                    acc[r][1] = __ffma2_rn(make_float2(q0.y, q0.y), v0, acc[r][1]);
-                    acc[r][2] = __ffma2_rn(make_float2(q0.z, q0.z), v0, acc[r][2]);
-                    acc[r][3] = __ffma2_rn(make_float2(q0.w, q0.w), v0, acc[r][3]);
-                    acc[r][0] = __ffma2_rn(make_float2(q1.x, q1.x), v1, acc[r][0]);
-                    acc[r][1] = __ffma2_rn(make_float2(q1.y, q1.y), v1, acc[r][1]);
-                    acc[r][2] = __ffma2_rn(make_float2(q1.z, q1.z), v1, acc[r][2]);
-                    acc[r][3] = __ffma2_rn(make_float2(q1.w, q1.w), v1, acc[r][3]);
+#pragma unroll
+                    for (int h = 0; h < K4; ++h) {
+                        float2* a = acc[r] + 4 * h;
+                        a[0] = __ffma2_rn(make_float2(q0[h].x, q0[h].x), v0, a[0]);
+                        a[1] = __ffma2_rn(make_float2(q0[h].y, q0[h].y), v0, a[1]);
+                        a[2] = __ffma2_rn(make_float2(q0[h].z, q0[h].z), v0, a[2]);
+                        a[3] = __ffma2_rn(make_float2(q0[h].w, q0[h].w), v0, a[3]);
+                        a[0] = __ffma2_rn(make_float2(q1[h].x, q1[h].x), v1, a[0]);
+                        a[1] = __ffma2_rn(make_float2(q1[h].y, q1[h].y), v1, a[1]);
+                        a[2] = __ffma2_rn(make_float2(q1[h].z, q1[h].z), v1, a[2]);
+                        a[3] = __ffma2_rn(make_float2(q1[h].w, q1[h].w), v1, a[3]);
+                    }
                 }
             }
         }
+        if (!valid) continue;
 #pragma unroll
-        for (int r = 0; r < RT; ++r)
+        for (int c = 0; c < KT; ++c) {
+            if (k + c >= N) break;
+            const auto col = f.column(k + c);
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
-                if (r0 + r < rows && k + c < N) store(r0 + r, k + c, acc[r][c]);
+            for (int r = 0; r < RT; ++r)
+                if (r0 + r < rows) f.put(col, r0 + r, acc[r][c]);
+        }
     }
 }
 
+// values of line r to the CTA that holds line k of the other axis, at r + at
+struct SendLines {
+    cg::cluster_group& cl;
+    float2* buf;
+    int per, ld, at;  // lines per CTA and length of a line there
+    __device__ __forceinline__ float2* column(int k) const {
+        const int owner = k / per;
+        return cl.map_shared_rank(buf, owner) + (k - owner * per) * ld + at;
+    }
+    __device__ __forceinline__ void put(float2* col, int r, float2 v) const { col[r] = v; }
+};
+
+// v / (Σ_d λ - σb): the denominator formed in FP64 and rounded once
+struct Divide {
+    float2* A;
+    int ld;
+    const double2* lsum;  // at this CTA's first line
+    int N0;
+    double2 sb;
+    __device__ __forceinline__ int column(int k) const { return k; }
+    __device__ __forceinline__ void put(int k, int c, float2 v) const {
+        const float2 d = narrow(csub(__ldg(lsum + (int64_t)k * N0 + c), sb));
+        const float inv = 1.0f / (d.x * d.x + d.y * d.y);
+        A[c * ld + k] = make_float2((v.x * d.x + v.y * d.y) * inv, (v.y * d.x - v.x * d.y) * inv);
+    }
+};
+
+struct Output {
+    double2* out;  // at this CTA's first line
+    const float2* sc;
+    int N0;
+    __device__ __forceinline__ int column(int k) const { return k; }
+    __device__ __forceinline__ void put(int k, int r, float2 v) const {
+        const int g = r * N0 + k;
+        const float2 s = __ldg(sc + g);
+        out[g] = widen(make_float2(v.x * s.x - v.y * s.y, v.x * s.y + v.y * s.x));
+    }
+};
+
 // Rc lines along axis 0 and Cc along axis 1 per CTA (the last CTA may have fewer)
-template <int RT>
+template <int RT, int KT>
 __global__ void __launch_bounds__(SF_T) k_sep_fused(JobSpace js, int in_slot, int out_slot, const double2* sigma,
                                                     double2 b, int N0, int N1, const float* __restrict__ Q0,
                                                     const float* __restrict__ Q1, const float2* __restrict__ sin32,
@@ -104,6 +184,7 @@ __global__ void __launch_bounds__(SF_T) k_sep_fused(JobSpace js, int in_slot, in
     const int size = max(Rc * ld0, Cc * ld1);
     extern __shared__ __align__(16) float2 sf_raw[];
     float2 *A = sf_raw, *Bf = sf_raw + size;  // both hold [Rc][ld0] or [Cc][ld1]
+    float* stage = reinterpret_cast<float*>(Bf + size);
     const int row0 = q * Rc, rows = max(0, min(Rc, N1 - row0));
     const int col0 = q * Cc, cols = max(0, min(Cc, N0 - col0));
     // every CTA of the cluster is running before it is written to, its buffers cleared
@@ -113,16 +194,26 @@ __global__ void __launch_bounds__(SF_T) k_sep_fused(JobSpace js, int in_slot, in
     const double2* in = js.vec + (size_t)job * js.vstride + (size_t)in_slot * js.n;
     double2* out = js.vec + (size_t)job * js.vstride + (size_t)out_slot * js.n;
     const int64_t g0 = (int64_t)row0 * N0;
-#pragma unroll 4
-    for (int i = tid; i < rows * N0; i += SF_T) {
-        const float2 x = from_c128<float2>(in[g0 + i]), s = sin32[g0 + i];
-        A[i / N0 * ld0 + i % N0] = make_float2(x.x * s.x - x.y * s.y, x.x * s.y + x.y * s.x);
+    // four loads in flight before the first conversion
+    for (int i0 = tid; i0 < rows * N0; i0 += 4 * SF_T) {
+        double2 x[4];
+        float2 sc[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + u * SF_T;
+            x[u] = i < rows * N0 ? in[g0 + i] : make_double2(0.0, 0.0);
+            sc[u] = i < rows * N0 ? sin32[g0 + i] : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + u * SF_T;
+            const float2 v = narrow(x[u]);
+            if (i < rows * N0)
+                A[i / N0 * ld0 + i % N0] = make_float2(v.x * sc[u].x - v.y * sc[u].y, v.x * sc[u].y + v.y * sc[u].x);
+        }
     }
     __syncthreads();
-    if (rows > 0)
-        rows_times_q<RT>(A, ld0, rows, N0, Q0, [&](int r, int k, float2 v) {
-            cl.map_shared_rank(Bf, k / Cc)[k % Cc * ld1 + row0 + r] = v;
-        });
+    if (rows > 0) rows_times_q<RT, KT>(A, ld0, rows, N0, Q0, stage, SendLines{cl, Bf, Cc, ld1, row0});
     cl.sync();
     // axis 1, the division, axis 1; A is free and becomes [Cc][ld1]
     if (ld0 != ld1 || Rc != Cc) {
@@ -132,28 +223,14 @@ __global__ void __launch_bounds__(SF_T) k_sep_fused(JobSpace js, int in_slot, in
         for (int i = tid; i < cols * (ld1 - N1); i += SF_T) A[i / (ld1 - N1) * ld1 + N1 + i % (ld1 - N1)] = make_float2(0.f, 0.f);
         __syncthreads();
     }
-    const double2 s = sigma[js.d_jobshift[job]];
-    const double2 sb = cmul(s, b);
-    if (cols > 0)
-        rows_times_q<RT>(Bf, ld1, cols, N1, Q1, [&](int c, int k, float2 v) {
-            const float2 d = from_c128<float2>(csub(lsum[(int64_t)k * N0 + col0 + c], sb));
-            const float inv = 1.0f / (d.x * d.x + d.y * d.y);
-            A[c * ld1 + k] = make_float2((v.x * d.x + v.y * d.y) * inv, (v.y * d.x - v.x * d.y) * inv);
-        });
+    const double2 sb = cmul(sigma[js.d_jobshift[job]], b);
+    if (cols > 0) rows_times_q<RT, KT>(Bf, ld1, cols, N1, Q1, stage, Divide{A, ld1, lsum + col0, N0, sb});
     cl.sync();  // every CTA has read its lines in Bf
     if (rows > 0)  // the padding of the lines that come back
         for (int i = tid; i < Rc * (ld0 - N0); i += SF_T) Bf[i / (ld0 - N0) * ld0 + N0 + i % (ld0 - N0)] = make_float2(0.f, 0.f);
-    if (cols > 0)
-        rows_times_q<RT>(A, ld1, cols, N1, Q1, [&](int c, int k, float2 v) {
-            cl.map_shared_rank(Bf, k / Rc)[k % Rc * ld0 + col0 + c] = v;
-        });
+    if (cols > 0) rows_times_q<RT, KT>(A, ld1, cols, N1, Q1, stage, SendLines{cl, Bf, Rc, ld0, col0});
     cl.sync();
-    if (rows > 0)
-        rows_times_q<RT>(Bf, ld0, rows, N0, Q0, [&](int r, int k, float2 v) {
-            const int64_t g = g0 + (int64_t)r * N0 + k;
-            const float2 sc = sout32[g];
-            out[g] = to_c128(make_float2(v.x * sc.x - v.y * sc.y, v.x * sc.y + v.y * sc.x));
-        });
+    if (rows > 0) rows_times_q<RT, KT>(Bf, ld0, rows, N0, Q0, stage, Output{out + g0, sout32 + g0, N0});
 }
 
 __global__ void k_sep_pad(const float* Q32, int N, int Np, float* Qp) {
@@ -163,14 +240,21 @@ __global__ void k_sep_pad(const float* Q32, int N, int Np, float* Qp) {
     Qp[t] = r < N && c < N ? Q32[(size_t)r * N + c] : 0.f;
 }
 
+// (rows, columns) a thread forms at a time, from few to many
+constexpr int kTiles[3][2] = {{1, 4}, {2, 4}, {4, 4}};
+
 struct FusedShape {
-    int C = 0, Rc = 0, Cc = 0, RT = 4;
+    int C = 0, Rc = 0, Cc = 0, tile = 2;
     size_t smem = 0;
     double cost = 1e300;
 };
 
-// Cluster size by an estimate of the clocks of an apply: the products at half the
-// FP32 rate over the threads that have work, and 2,000 clocks a cluster barrier.
+// Cluster size and tile by an estimate of the clocks of an apply.  A product takes,
+// per two reduction steps and round of 256 threads, 1.5 times its loads' way into
+// the registers (a 16-byte load of a warp takes 4 clocks), at least 200 clocks, and
+// a round's results 100 clocks a value (measured on 30 to 250 points a side: 40,000
+// clocks at 60 points with four CTAs and 1 x 4, 185,000 at 250 with 16 and 4 x 4,
+// where 2 x 4 takes 260,000 and 4 x 8, on half the threads, 220,000).
 FusedShape fused_shape(int N0, int N1, int na) {
     FusedShape best;
     for (int C = 1; C <= 16; ++C) {
@@ -179,20 +263,23 @@ FusedShape fused_shape(int N0, int N1, int na) {
         f.Cc = (N0 + C - 1) / C;
         if (C > 1 && ((C - 1) * f.Rc >= N1 || (C - 1) * f.Cc >= N0)) continue;  // a CTA without lines
         f.C = C;
-        f.smem = 2 * sizeof(float2) * (size_t)std::max(f.Rc * pad4(N0), f.Cc * pad4(N1));
+        f.smem = 2 * sizeof(float2) * (size_t)std::max(f.Rc * pad4(N0), f.Cc * pad4(N1)) +
+                 SF_STAGES * sizeof(float) * std::max(stage_floats(N0), stage_floats(N1));
         if (f.smem > 220 * 1024) continue;
-        for (int RT : {4, 8}) {
+        const double per_sm = std::ceil((double)na * C / 152.0);  // CTAs that share an SM, in turn or at once
+        for (int t = 0; t < 3; ++t) {
+            const int RT = kTiles[t][0], KT = kTiles[t][1];
             auto product = [&](int rows, int N) {
-                const double items = (double)(pad4(N) / 4) * ((rows + RT - 1) / RT);
-                // an item: RT x 4 x N paired FMAs; 256 threads, 64 paired FMAs a clock
-                return std::ceil(items / SF_T) * SF_T * RT * 4.0 * N / 64.0 / (RT == 8 ? 0.6 : 0.45);
+                const int items = (N + KT - 1) / KT * ((rows + RT - 1) / RT);
+                const double rounds = std::ceil((double)items / SF_T);
+                const double warps = std::min<double>(SF_T / 32, std::ceil(items / 32.0));
+                const double lsu = warps * (RT + KT / 2.0) * 4.0;
+                return rounds * (N / 2.0 * std::max(200.0, 1.5 * lsu) + 100.0 * warps * RT * KT / 2.0);
             };
-            const int per_sm = f.smem <= 110 * 1024 ? 2 : 1;
-            const double waves = std::ceil((double)na * C / (152.0 * per_sm)) * (na * C > 152 ? 2.0 / per_sm * per_sm : 1.0);
-            const double cost = waves * (2.0 * product(f.Rc, N0) + 2.0 * product(f.Cc, N1)) + (C > 1 ? 9000.0 : 4000.0);
+            const double cost = per_sm * (2.0 * product(f.Rc, N0) + 2.0 * product(f.Cc, N1)) + (C > 1 ? 9000.0 : 4000.0);
             if (cost < best.cost) {
                 best = f;
-                best.RT = RT;
+                best.tile = t;
                 best.cost = cost;
             }
         }
@@ -200,15 +287,31 @@ FusedShape fused_shape(int N0, int N1, int na) {
     return best;
 }
 
-template <int RT>
+// The same for the separate kernels: a product's CTAs (128 rows of real and
+// imaginary parts each, two to an SM) take 6,000 clocks and 35 per output column for
+// each 32 reduction indices, the elementwise passes 8,000 and their traffic, a
+// launch 2,000.  Many jobs of a few hundred points a side fill the tensor cores and
+// stay there (64 pencils of 219 points: 0.3 ms against 0.5).
+double separate_cost(int N0, int N1, int na) {
+    const double n = (double)N0 * N1;
+    auto product = [&](int N, int rows) {
+        const int NT = std::min(256, (N + 15) / 16 * 16);
+        const double ctas = std::ceil(2.0 * rows / 128.0) * std::ceil((double)N / NT) * na;
+        return std::ceil(ctas / 304.0) * std::ceil(N / 32.0) * (6000.0 + 35.0 * NT);
+    };
+    return 2.0 * product(N0, N1) + 2.0 * product(N1, N0) + 3.0 * (8000.0 + n * na * 48.0 / 3300.0) + 7.0 * 2000.0;
+}
+
+template <int RT, int KT>
 void launch_fused(const Separable& S, const JobSpace& js, int na, int in_slot, int out_slot, const double2* d_sigma,
                   const FusedShape& f, cudaStream_t st) {
     static std::atomic<uint64_t> ready{0};  // devices whose kernel attributes are set
+    auto kern = k_sep_fused<RT, KT>;
     int dev = 0;
     SIM_CUDA(cudaGetDevice(&dev));
     if (dev > 63 || !(ready.load() >> dev & 1)) {
-        SIM_CUDA(cudaFuncSetAttribute(k_sep_fused<RT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-        SIM_CUDA(cudaFuncSetAttribute(k_sep_fused<RT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        SIM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+        SIM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         if (dev <= 63) ready.fetch_or(1ull << dev);
     }
     cudaLaunchConfig_t cfg = {};
@@ -223,9 +326,9 @@ void launch_fused(const Separable& S, const JobSpace& js, int na, int in_slot, i
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    SIM_CUDA(cudaLaunchKernelEx(&cfg, k_sep_fused<RT>, js, in_slot, out_slot, d_sigma, S.b, (int)S.dims[0],
-                                (int)S.dims[1], (const float*)S.Qp[0], (const float*)S.Qp[1],
-                                (const float2*)S.sin32, (const float2*)S.sout32, (const double2*)S.lsum, f.Rc, f.Cc));
+    SIM_CUDA(cudaLaunchKernelEx(&cfg, kern, js, in_slot, out_slot, d_sigma, S.b, (int)S.dims[0], (int)S.dims[1],
+                                (const float*)S.Qp[0], (const float*)S.Qp[1], (const float2*)S.sin32,
+                                (const float2*)S.sout32, (const double2*)S.lsum, f.Rc, f.Cc));
     SIM_LAUNCH_CHECK();
 }
 
@@ -241,9 +344,12 @@ bool sep_fused_2d(const Separable& S, const JobSpace& js, int na, int in_slot, i
                   cudaStream_t st) {
     if (S.ndim != 2 || S.dims[0] > 2048 || S.dims[1] > 2048) return false;
     const FusedShape f = fused_shape((int)S.dims[0], (int)S.dims[1], na);
-    if (f.C == 0) return false;
-    if (f.RT == 8) launch_fused<8>(S, js, na, in_slot, out_slot, d_sigma, f, st);
-    else launch_fused<4>(S, js, na, in_slot, out_slot, d_sigma, f, st);
+    if (f.C == 0 || f.cost > separate_cost((int)S.dims[0], (int)S.dims[1], na)) return false;
+    switch (f.tile) {
+        case 0: launch_fused<1, 4>(S, js, na, in_slot, out_slot, d_sigma, f, st); break;
+        case 1: launch_fused<2, 4>(S, js, na, in_slot, out_slot, d_sigma, f, st); break;
+        default: launch_fused<4, 4>(S, js, na, in_slot, out_slot, d_sigma, f, st); break;
+    }
     return true;
 }
 
