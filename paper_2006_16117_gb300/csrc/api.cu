@@ -1304,16 +1304,31 @@ sim_status sim_apply_shifted(sim_handle h, double sig_re, double sig_im, const d
     if (!h) return fail(nullptr, SIM_ERR_INVALID_ARG, "NULL handle");
     return guarded(h, [&]() -> sim_status {
         if (!x || !y) return fail(h, SIM_ERR_INVALID_ARG, "NULL vector");
-        const int sc = h->cap - 1;
-        const double2 sg = make_double2(sig_re, sig_im);
-        SIM_CUDA(cudaMemcpyAsync(h->d_sigma + sc, &sg, sizeof(double2), cudaMemcpyHostToDevice, h->st));
-        JobSpace js = make_jobspace(h, 1, "cmp_");
-        SIM_CUDA(cudaMemcpyAsync(js.d_jobshift, &sc, sizeof(int), cudaMemcpyHostToDevice, h->st));
-        const int zero = 0;
-        SIM_CUDA(cudaMemcpyAsync(js.d_active, &zero, sizeof(int), cudaMemcpyHostToDevice, h->st));
-        SIM_CUDA(cudaMemcpyAsync(js.vec + (size_t)VS_X * js.n, x, sizeof(double2) * js.n, cudaMemcpyDeviceToDevice, h->st));
-        spmv_shifted_jobs(h->P, js, 1, nullptr, VS_X, VS_W, h->d_sigma, h->st);
-        SIM_CUDA(cudaMemcpyAsync(y, js.vec + (size_t)VS_W * js.n, sizeof(double2) * js.n, cudaMemcpyDeviceToDevice, h->st));
+        const int64_t n = h->P.n;
+        // The kernel reads and writes the caller's vectors where it can: device memory,
+        // aligned, not overlapping (rows read others' entries of x); copies otherwise.
+        auto direct = [](const void* p) {
+            cudaPointerAttributes at{};
+            if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+                (void)cudaGetLastError();
+                return false;
+            }
+            return (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) &&
+                   (reinterpret_cast<uintptr_t>(p) & 15) == 0;
+        };
+        const size_t bytes = sizeof(double2) * n;
+        const double2* xv = reinterpret_cast<const double2*>(x);
+        double2* yv = reinterpret_cast<double2*>(y);
+        const bool overlap = (uintptr_t)x < (uintptr_t)y + bytes && (uintptr_t)y < (uintptr_t)x + bytes;
+        const bool y_direct = direct(y);
+        if (overlap || !direct(x)) {
+            double2* c = h->arena.get<double2>("apply_x", n);
+            SIM_CUDA(cudaMemcpyAsync(c, x, bytes, cudaMemcpyDeviceToDevice, h->st));
+            xv = c;
+        }
+        if (!y_direct) yv = h->arena.get<double2>("apply_y", n);
+        apply_shifted(h->P, make_double2(sig_re, sig_im), xv, yv, h->st);
+        if (!y_direct) SIM_CUDA(cudaMemcpyAsync(y, yv, bytes, cudaMemcpyDeviceToDevice, h->st));
         SIM_CUDA(cudaStreamSynchronize(h->st));
         return SIM_OK;
     });

@@ -178,6 +178,9 @@ bool arnoldi(const Pencil& P, const sim_options& opt, JobSpace& js, const double
 
 void apply_B(const Pencil& P, const double2* x, double2* y, cudaStream_t st);
 
+// y = (A - σB) x; x and y must not overlap.
+void apply_shifted(const Pencil& P, double2 sigma, const double2* x, double2* y, cudaStream_t st);
+
 class DeviceArena;
 JobSpace make_jobspace(DeviceArena& ar, cudaStream_t st, int J, int k, int m, int64_t n, const std::string& tag);
 // Krylov jobs whose job spaces (vectors, basis, preconditioner work vectors)

@@ -352,6 +352,33 @@ void spmv_shifted_jobs(const Pencil& P, const JobSpace& js, int nactive, const d
     spmv_launch_rj(4, P, js, nactive, x_slot, y_slot, -1, d_sigma, st);
 }
 
+// y = (A - σB) x on the caller's vectors, σ by value: the same sums in the same
+// order as k_spmv_jobs.  A thread per row: a call of a few thousand rows is bounded by
+// its launch and the wait for it, so it is one launch (three uploads, two copies of the
+// vectors and the job kernel before).  n = 40,000: 40 -> 23 us a call.
+__global__ void __launch_bounds__(256) k_apply_shifted(Pencil P, double2 sg, const double2* x, double2* y) {
+    const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= P.n) return;
+    double2 acc = make_double2(0.0, 0.0);
+    const int64_t e0 = P.rp[g], e1 = P.rp[g + 1];
+    if (P.b_kind <= 1) {
+        const double2 sb = cmul(sg, P.Bdiag[g]);
+        for (int64_t e = e0; e < e1; ++e) {
+            const int64_t j = P.ci[e];
+            const double2 a = P.Ka[e];
+            acc = cfma(j == g ? csub(a, sb) : a, x[j], acc);
+        }
+    } else {
+        for (int64_t e = e0; e < e1; ++e) acc = cfma(csub(P.Ka[e], cmul(sg, P.Kb[e])), x[P.ci[e]], acc);
+    }
+    y[g] = acc;
+}
+
+void apply_shifted(const Pencil& P, double2 sg, const double2* x, double2* y, cudaStream_t st) {
+    k_apply_shifted<<<cdiv_up(P.n, 256), 256, 0, st>>>(P, sg, x, y);
+    SIM_LAUNCH_CHECK();
+}
+
 __global__ void k_apply_B(Pencil P, const double2* x, double2* y) {
     int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= P.n) return;
