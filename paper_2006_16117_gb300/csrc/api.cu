@@ -280,9 +280,6 @@ void upload_pencil(DeviceArena& ar, cudaStream_t st, Pencil& P, const std::vecto
     P.Lcol = (const int32_t*)up("Lcol", Lcol.data(), sizeof(int32_t) * Lcol.size());
     P.Lidx = (const int32_t*)up("Lidx", Lidx.data(), sizeof(int32_t) * Lidx.size());
     P.nnzL = (int64_t)Lcol.size();
-    std::vector<int32_t> L0col(n);
-    for (int64_t g = 0; g < n; ++g) L0col[g] = Lptr[g + 1] > Lptr[g] ? Lcol[Lptr[g]] : -1;
-    P.L0col = (const int32_t*)up("L0col", L0col.data(), sizeof(int32_t) * L0col.size());
     P.anorm = P.bnorm = 0.0;
     for (int64_t i = 0; i < n; ++i) {
         double ra = 0.0, rb = 0.0;

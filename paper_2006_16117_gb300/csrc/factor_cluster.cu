@@ -291,11 +291,6 @@ __global__ void __launch_bounds__(NT, 1) k_factor_cl(Pencil P, const int* shift_
         const int64_t e_hi = P.Lptr[g_hi];
         for (int64_t e = P.Lptr[g_lo] + tid + (int64_t)q * nt; e < e_hi; e += (int64_t)nt * Cf)
             Lval[e] = from_c128<C>(sval(P, P.Lidx[e], sg));
-        C* L0val = Dinv + factor_l0_offset(P);
-        for (int64_t g = g_lo + tid + (int64_t)q * nt; g < g_hi; g += (int64_t)nt * Cf) {
-            const int e0 = P.Lptr[g];
-            L0val[g] = from_c128<C>(P.Lptr[g + 1] > e0 ? sval(P, P.Lidx[e0], sg) : make_double2(0.0, 0.0));
-        }
     }
     if (Cf > 1) {
         cluster_arrive();

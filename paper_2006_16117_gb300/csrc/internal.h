@@ -51,9 +51,6 @@ struct Pencil {
     const int32_t* Lcol = nullptr;
     const int32_t* Lidx = nullptr;
     int64_t nnzL = 0;
-    // per row g: Lcol of its first coupling, -1 if it has none (a solve can
-    // load it, and the shift's first value L0val[g], without reading Lptr first)
-    const int32_t* L0col = nullptr;
     // host pointer: when set, the inner solver's preconditioner is the
     // fast-diagonalisation inverse of the pencil's separable part instead of
     // the block factorisation (nothing is factored per shift)
@@ -64,16 +61,14 @@ struct Pencil {
 };
 
 // Bytes of one shift's factorisation: Dinv and E (2 nb T² entries; E_mid's place
-// is scratch), Lval and L0val.
+// is scratch) and Lval.
 inline size_t factor_storage_bytes(const Pencil& P, int precision) {
     const size_t cs = precision == SIM_FP64 ? sizeof(double2) : sizeof(float2);
-    return ((size_t)2 * P.nb * (size_t)P.T * P.T + (size_t)P.nnzL + (size_t)P.n + 16) * cs;
+    return ((size_t)2 * P.nb * (size_t)P.T * P.T + (size_t)P.nnzL + 16) * cs;
 }
 
 // Offset (in elements of the factor type) of Lval inside a shift's factor.
 __host__ __device__ inline size_t factor_lval_offset(const Pencil& P) { return (size_t)2 * P.nb * P.T * P.T; }
-// Offset of L0val (n values: the first coupling's shifted value of each row, 0 if none).
-__host__ __device__ inline size_t factor_l0_offset(const Pencil& P) { return factor_lval_offset(P) + (size_t)P.nnzL; }
 
 // Host side of a job space, kept with its buffers: pinned memory (the device
 // writes istat and worst, the host fills act), the list last uploaded and the

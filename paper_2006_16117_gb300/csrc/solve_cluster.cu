@@ -12,21 +12,32 @@
 // backward ones, each cluster computing x_mid for itself first (t_{mid±1} come
 // from a copy in the job's VS_W slot, as side 0 may already have overwritten
 // its own), so that no cluster waits for another.  One right-hand side, T = 200,
-// nb = 200: 696 -> 378 us in complex64.
+// nb = 200, complex64: 696 us as one chain, 378 as two.
 //
 // Only the vectors depend on the previous step, the matrices do not.  So
-// each CTA of a cluster owns a slice of rows of every block, and a producer
-// warp streams the slices, in chain order, through a ring of shared-memory
+// each CTA of a cluster owns a slice of rows of every block, and two producer
+// warps stream the slices, in chain order, through a ring of shared-memory
 // stages (one 1-D bulk copy per row into a padded row, completing on the
 // stage's "full" mbarrier) as far ahead as the ring allows; the consumers
-// release a stage on its "empty" mbarrier.  Per step the eight consumer warps
-// form the right-hand side, then for each chunk of rows run the GEMV with one
-// row per lane (or a row per group of lanes) and a column range per warp, sum
-// the warps' partials through shared memory, and send the new rows of the
-// vector into every CTA's shared memory with st.async, which completes on the
+// release a stage on its "empty" mbarrier.  Per step each of the eight consumer
+// warps forms the right-hand side in its own columns, then for each chunk of rows
+// runs the GEMV over them with one row per lane (or a row per group of lanes); the
+// warps' partial sums are added through shared memory and the new rows of the
+// vector sent into every CTA's shared memory with st.async, which completes on the
 // receiver's per-step mbarrier.  Up to R right-hand sides of the same shift
 // share each pass over the matrices (the k random vectors of the
 // multiplicity step).
+//
+// What bounds a chain step is the number of instructions a warp runs through once:
+// with two or three warps a scheduler and straight-line code that fits no
+// instruction buffer each costs about five clocks.  Hence a kernel per phase and
+// per "one chunk a step" (ONE), the inputs brought by the producers, one barrier a
+// step, the vector stored to memory a step later by warps that wait anyway, and row
+// layouts that are powers of two.  Two sides, T = 200 complex64: 378 -> 268 us
+// (a step 3,800 -> 2,900 clocks forward, 3,100 -> 2,300 backward); T = 102 197 -> 127;
+// eight right-hand sides at T = 102 196 -> 138 us a launch; complex128 T = 30
+// 106 -> 58, T = 98 335 -> 201.  With 56 shifts at T = 200 the matrices bound it:
+// 1,446 -> 1,159 us (5.0 TB/s) in complex64, 12.4 -> 10.2 ms in complex128 (FP64 pipe).
 //
 // Every wait on an mbarrier has an iteration limit; a thread whose wait runs
 // out records an error and the CTA stops computing and issuing copies, keeps
@@ -37,6 +48,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <map>
+#include <type_traits>
 #include <vector>
 
 #include "internal.h"
@@ -117,29 +129,6 @@ __device__ __forceinline__ void st_async_c(uint32_t raddr, double2 v, uint32_t r
 
 constexpr long long WAIT_LIMIT = 1ll << 26;  // try_wait polls before a wait is declared failed
 
-// Sum S values across the warp (S = 8 or 16): at each stage a lane keeps half
-// of its values and trades the other half with its partner, so S-1 shuffles
-// leave one partial per lane; the lanes below the value bits then finish with
-// plain xor shuffles.  Afterwards lane L holds, in v[0], the warp sum of value
-// (L >> (5 - log2 S)) & (S - 1).
-template <class Rt, int S> __device__ __forceinline__ void butterfly(Rt (&v)[S], int lane) {
-#pragma unroll
-    for (int st = 0, width = S; width > 1; ++st, width >>= 1) {
-        const int mask = 16 >> st;
-        const bool upper = (lane & mask) != 0;
-        const int half = width >> 1;
-#pragma unroll
-        for (int i = 0; i < half; ++i) {
-            const Rt send = upper ? v[i] : v[i + half];
-            const Rt keep = upper ? v[i + half] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, mask);
-        }
-    }
-    constexpr int LOGS = S == 16 ? 4 : 3;
-#pragma unroll
-    for (int mask = (1 << (5 - LOGS)) >> 1; mask > 0; mask >>= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], mask);
-}
-
 template <class C> __device__ __forceinline__ C zero_c();
 template <> __device__ __forceinline__ double2 zero_c<double2>() { return make_double2(0.0, 0.0); }
 template <> __device__ __forceinline__ float2 zero_c<float2>() { return make_float2(0.f, 0.f); }
@@ -165,10 +154,14 @@ template <> struct Vec16<double2> {
 // two CTAs per SM for single right-hand sides in complex64 (see choose_shape)
 constexpr bool kTwoPerSm = true;
 
+constexpr int PF_T = 256;                         // largest T whose step inputs are fetched ahead
+constexpr int RW = 9;                             // a row's partial sums, padded off the banks
+constexpr int NE = 2;                             // couplings of a row fetched ahead
 constexpr int CL_WARPS = 8;                       // consumer warps: the GEMVs and the vector work
-constexpr int CL_THREADS = (CL_WARPS + 1) * 32;   // + one producer warp that issues the copies
+constexpr int PROD = 64;                         // threads that issue the copies (two warps)
+constexpr int CL_THREADS = CL_WARPS * 32 + PROD;
 
-// barrier of the consumer warps only (the producer warp never joins it)
+// barrier of the consumer warps only (the producer warps never join it)
 __device__ __forceinline__ void consumer_sync() {
     static_assert(CL_WARPS * 32 == 256, "named barrier thread count");
     asm volatile("bar.sync 1, 256;" ::: "memory");
@@ -178,15 +171,30 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
+// BYTES of src to shared memory, or zeros
+template <int BYTES> __device__ __forceinline__ void copy_async(void* dst, const void* src, bool there = true) {
+    const uint32_t n = there ? BYTES : 0;
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(n) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(smem_u32(dst)), "l"(src), "n"(BYTES), "r"(n)
+                     : "memory");
+}
+// an arrival on the barrier once this thread's copies so far are done
+__device__ __forceinline__ void arrive_after_copies(uint64_t* bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 __device__ __forceinline__ bool failed_flag(const int* f) { return *(const volatile int*)f != 0; }
 
 // MINB: CTAs per SM the launch is built for (2 caps the registers at 112 so
 // that two CTAs of at most ~112 KB of shared memory share an SM)
-template <class C, int R, int MINB>
+template <class C, int R, int MINB, bool ONE, int phase>
 __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, JobSpace js, int in_slot,
                                                                   int out_slot, void* const* fptrs,
-                                                                  const int* grp_jobs, int SR, int NS, int TP,
-                                                                  int* err, int phase) {
+                                                                  const int* grp_jobs, int SR, int NS, int TP, int pf_ok,
+                                                                  int* err) {
     cg::cluster_group cl = cg::this_cluster();
     const int Ccl = (int)cl.num_blocks();
     const int q = (int)cl.block_rank();
@@ -208,9 +216,9 @@ __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, J
     __shared__ const double2* s_in[R];
     __shared__ double2* s_out[R];
     __shared__ int s_fail;
-    int nr = 0;
+    int nr = 1;
 #pragma unroll
-    for (int j = 0; j < R; ++j)
+    for (int j = 1; j < R; ++j)
         if (grp_jobs[grp * R + j] >= 0) nr = j + 1;
     const int job0 = grp_jobs[grp * R];
     if (tid < R) {
@@ -223,28 +231,33 @@ __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, J
     const C* Dinv = reinterpret_cast<const C*>(fptrs[s]);
     const C* E = Dinv + (size_t)nb * T * T;
     const C* Lval = Dinv + factor_lval_offset(P);
-    const C* L0val = Dinv + factor_l0_offset(P);
 
     const int Tc = (T + Ccl - 1) / Ccl;
     const int r0 = min(T, q * Tc), r1 = min(T, r0 + Tc);
     const int myrows = r1 - r0;
-    const int nsub = (myrows + SR - 1) / SR;
-    const int total = nsteps * nsub;
+    const int Cact = (T + Tc - 1) / Tc;  // CTAs that have rows: the others take no part
 
     extern __shared__ __align__(128) unsigned char raw[];
     C* stage = reinterpret_cast<C*>(raw);                  // [NS][SR][TP]: rows padded to TP
     C* vbuf = stage + (size_t)NS * SR * TP;                // [3][R][T]: the chain's vectors
-    C* sbuf = vbuf + (size_t)3 * R * T;                    // [R][T]
-    C* tbuf = sbuf + (size_t)R * T;                        // [R][T]: t_k rows of this CTA (backward)
-    C* red = tbuf + (size_t)R * T;                         // [2][warps][R][SR]: per-warp partial sums
-    uint64_t* full = reinterpret_cast<uint64_t*>(red + (size_t)2 * CL_WARPS * R * SR);  // [NS] stage filled
+    C* sbuf = vbuf + (size_t)3 * R * T;                    // [R][T]: r_k - L_k t_outer
+    C* red = sbuf + (size_t)R * T;                         // [2][R][SR][RW]: per-warp partial sums
+    double2* tpf = reinterpret_cast<double2*>(red + (size_t)2 * RW * R * SR);
+    // (tpf [3][R][SR]: t_k of this and the next two steps' rows)
+    // fetched ahead if pf_ok: r_k [2][R][T], the first couplings' values and columns
+    // [2][NE][T], the bounds of the rows' couplings [4][2][T]
+    double2* rpf = tpf + (size_t)3 * R * SR;
+    C* apf = reinterpret_cast<C*>(rpf + (pf_ok ? (size_t)2 * R * T : 0));
+    int* cpf = reinterpret_cast<int*>(apf + (pf_ok ? (size_t)2 * NE * T : 0));
+    int* bpf = cpf + (pf_ok ? (size_t)2 * NE * T : 0);
+    uint64_t* full = reinterpret_cast<uint64_t*>(bpf + (pf_ok ? (size_t)8 * T : 0));     // [NS] stage filled
     uint64_t* empty = full + NS;                                                         // [NS] stage consumed
     uint64_t* vbar = empty + NS;                                                         // [3] vector received
 
     if (tid == 0) {
         s_fail = 0;
         for (int i = 0; i < NS; ++i) {
-            mbar_init(&full[i], 1);
+            mbar_init(&full[i], 1 + PROD);  // the bulk copies' expected bytes, and the producers
             mbar_init(&empty[i], 1);
         }
         for (int i = 0; i < 3; ++i) mbar_init(&vbar[i], 1);
@@ -256,129 +269,300 @@ __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, J
         for (int i = 0; i < 3 && i <= nsteps - 2; ++i) mbar_expect_tx(&vbar[i], vec_bytes);  // steps 0, 1, 2
     cl.sync();  // every CTA of the cluster is running, barriers initialised and armed, before any remote store
 
-    if (warp == CL_WARPS) {
-        // ---- producer: chunk c = up to SR rows of one block, one 1-D bulk copy
-        // per row into its padded row of stage c % NS, once that stage is consumed
-        int c = 0;
-        for (; c < total; ++c) {
-            const int slot = c % NS;
-            int ok = 1;
-            if (lane == 0) {
-                if (c >= NS) {
-                    const uint32_t par = (uint32_t)(((c / NS) - 1) & 1);
-                    long long it = 0;
-                    while (!mbar_try_wait(&empty[slot], par)) {
-                        if (failed_flag(&s_fail)) {
-                            ok = 0;
-                            break;
-                        }
-                        if (++it > WAIT_LIMIT) {
-                            s_fail = 1;
-                            atomicExch(err, 4);
-                            ok = 0;
-                            break;
-                        }
-                    }
-                }
-                if (failed_flag(&s_fail)) ok = 0;
+    // A wait that gives up once the CTA has failed, or after WAIT_LIMIT polls.
+    auto bounded = [&](auto&& done, int code) {
+        if (__builtin_expect(done(), 1)) return true;
+        for (long long it = 0; !failed_flag(&s_fail); ++it) {
+            if (done()) return true;
+            if (it > WAIT_LIMIT) {
+                s_fail = 1;
+                atomicExch(err, code);
             }
-            ok = __shfl_sync(0xffffffffu, ok, 0);
-            if (!ok) break;
-            const int b = c / nsub, sub = c % nsub;
-            const int rs = r0 + sub * SR;
-            const int rows = min(SR, r1 - rs);
-            const C* M = (phase == 0 || b == 0 ? Dinv : E) + (size_t)block_of(b) * T * T + (size_t)rs * T;
-            C* dst = stage + (size_t)slot * SR * TP;
-            if (lane == 0) mbar_expect_tx(&full[slot], (uint32_t)((size_t)rows * T * sizeof(C)));
-            __syncwarp();
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            for (int i = lane; i < rows; i += 32)
-                tma_load_1d(dst + (size_t)i * TP, M + (size_t)i * T, (uint32_t)(T * sizeof(C)), &full[slot]);
         }
+        return false;
+    };
+
+    if (myrows == 0) {
+    } else if (warp >= CL_WARPS) {
+        // ---- producers: chunk c = up to SR rows of one block, one 1-D bulk copy
+        // per row into its padded row of stage c % NS, once that stage is consumed.
+        //
+        // With the chunks come, through asynchronous copies by their lanes that count
+        // on the same "full" barriers, the inputs of the right-hand sides (a load to a
+        // consumer's register would be waited for wherever the compiler moves that
+        // register): forward, of every column, r_k and the first NE couplings of the
+        // row, whose bounds came a step earlier; backward (ONE) t_k of this CTA's rows.
+        // They share two buffers, so with one chunk a step they come one chunk after
+        // their own: the stage of chunk c is free when chunk c - 3 is consumed, the
+        // inputs' buffer of chunk c - 1 as well.
+        constexpr int LAG = ONE ? 1 : 0;
+        const int pt = tid - CL_WARPS * 32;
+        auto fetch_bounds = [&](int bb) {
+            if (phase != 0 || !pf_ok || bb >= nsteps) return;
+            const int64_t g = (int64_t)block_of(bb) * T;
+            int* d = bpf + (bb & 3) * 2 * T;
+            for (int i = pt; i < T; i += PROD) {
+                const bool in = g + i < P.n;
+                const int* src = P.Lptr + (in ? g + i : 0);
+                copy_async<4>(d + i, src, in);
+                copy_async<4>(d + T + i, src + 1, in);
+            }
+        };
+        auto fetch_inputs = [&](int bb) {
+            if (bb < 0) return;
+            const int64_t g = (int64_t)block_of(bb) * T;
+            if (phase == 0 && pf_ok) {
+                const int* d = bpf + (bb & 3) * 2 * T;
+                const int at = (bb & 1) * NE * T;
+                double2* rd = rpf + (bb & 1) * R * T;
+                for (int i = pt; i < T; i += PROD) {
+                    const int lo = d[i], cnt = d[T + i] - lo;
+#pragma unroll
+                    for (int e = 0; e < NE; ++e)
+                        if (e < cnt) {
+                            copy_async<4>(cpf + at + e * T + i, P.Lcol + lo + e);
+                            copy_async<sizeof(C)>(apf + at + e * T + i, Lval + lo + e);
+                        }
+                    const bool in = g + i < P.n;
+                    for (int j = 0; j < nr; ++j) copy_async<16>(rd + j * T + i, s_in[j] + (in ? g + i : 0), in);
+                }
+            } else if (phase == 1 && ONE && bb > 0) {
+                for (int i = pt; i < myrows; i += PROD) {
+                    const bool in = g + r0 + i < P.n;
+                    for (int j = 0; j < nr; ++j)
+                        copy_async<16>(tpf + ((bb % 3) * R + j) * SR + i, s_out[j] + (in ? g + r0 + i : 0), in);
+                }
+            }
+        };
+        int slot = 0, round = 0, issued = 0;  // c = round * NS + slot
+        bool ok = true;
+        fetch_bounds(0);
+        for (int b = 0; b < nsteps && ok; ++b) {
+            const C* M = (phase == 0 || b == 0 ? Dinv : E) + (size_t)block_of(b) * T * T;
+            for (int rs = r0; rs < r1; rs += SR) {
+                if (lane == 0) {
+                    if (round > 0)
+                        ok = bounded([&] { return mbar_try_wait(&empty[slot], (uint32_t)((round - 1) & 1)); }, 4);
+                    if (failed_flag(&s_fail)) ok = false;
+                }
+                ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+                if (!ok) break;
+                const int rows = min(SR, r1 - rs);
+                C* dst = stage + (size_t)slot * SR * TP;
+                if (pt == 0) mbar_expect_tx(&full[slot], (uint32_t)((size_t)rows * T * sizeof(C)));
+                __syncwarp();
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                for (int i = pt; i < rows; i += PROD)
+                    tma_load_1d(dst + (size_t)i * TP, M + (size_t)(rs + i) * T, (uint32_t)(T * sizeof(C)),
+                                &full[slot]);
+                if (!ONE && myrows <= SR && b >= 2) {
+                    // one chunk a step in this CTA: the inputs' buffer, as above
+                    if (lane == 0)
+                        ok = bounded([&] { return mbar_try_wait(&empty[(b - 2) % NS], (uint32_t)(((b - 2) / NS) & 1)); }, 4);
+                    __syncwarp();
+                }
+                if (rs == r0) {
+                    copies_done();  // the bounds asked for a step ago
+                    __syncwarp();
+                    fetch_inputs(b - LAG);
+                    fetch_bounds(b + 1);
+                }
+                if constexpr (ONE) {
+                    if (b > 0) arrive_after_copies(&full[slot == 0 ? NS - 1 : slot - 1]);
+                } else {
+                    arrive_after_copies(&full[slot]);
+                }
+                ++issued;
+                if (++slot == NS) {
+                    slot = 0;
+                    ++round;
+                }
+            }
+        }
+        if constexpr (ONE) {
+            // the last chunk's inputs: their buffer is free when the chunk two before is
+            const int c = nsteps - 1;
+            if (ok && c >= 0) {
+                if (lane == 0 && c >= 2)
+                    ok = bounded([&] { return mbar_try_wait(&empty[(c - 2) % NS], (uint32_t)(((c - 2) / NS) & 1)); }, 4);
+                ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+                copies_done();
+                __syncwarp();
+                if (ok) fetch_inputs(c);
+                arrive_after_copies(&full[c % NS]);
+            } else if (issued > 0) {
+                arrive_after_copies(&full[(issued - 1) % NS]);
+            }
+        }
+        copies_done();
         // stopped early (a failure): the last issued copies may still be in flight,
         // and this CTA's shared memory must outlive them
-        if (lane == 0 && c < total) {
-            for (int d = max(0, c - NS); d < c; ++d) {
+        if (pt == 0 && !ok) {
+            for (int d = max(0, issued - NS); d < issued; ++d) {
                 long long it = 0;
                 while (!mbar_try_wait(&full[d % NS], (uint32_t)((d / NS) & 1)) && ++it < WAIT_LIMIT) {
                 }
             }
         }
     } else {
-        // ---- consumers
-        // Prefetch of the next step's chain-independent inputs, one row per
-        // thread, kept as loaded (no arithmetic on them until they are used):
-        // r_k and the row's couplings (forward), t_k of this CTA's rows (backward).
-        const bool pf_ok = T <= CL_WARPS * 32;
-        double2 pf_v[R];
-        int pf_lo = 0, pf_hi = 0, pf_c = 0;
-        C pf_a = zero_c<C>();
-        auto prefetch_fwd = [&](int kk) {
-            const int64_t g = (int64_t)kk * T + tid;
-            if (tid < T) {
-                const bool in = g < P.n;
-#pragma unroll
-                for (int j = 0; j < R; ++j)
-                    if (j < nr) pf_v[j] = in ? s_in[j][g] : make_double2(0.0, 0.0);
-                if (in) {
-                    pf_lo = P.Lptr[g];
-                    pf_hi = P.Lptr[g + 1];
-                    pf_c = P.L0col[g];
-                    pf_a = L0val[g];
-                } else {
-                    pf_lo = pf_hi = 0;
-                }
-            }
-        };
-        auto prefetch_bwd = [&](int kk) {
-            const int64_t g = (int64_t)kk * T + r0 + tid;
-            if (tid < myrows) {
-#pragma unroll
-                for (int j = 0; j < R; ++j)
-                    if (j < nr) pf_v[j] = g < P.n ? s_out[j][g] : make_double2(0.0, 0.0);
-            }
-        };
-        if (pf_ok && phase == 0) prefetch_fwd(block_of(0));
-
-        // this warp's 16-byte column units of every row
+        // ---- consumers.  A step is a chain of short phases, and with two or three
+        // warps a scheduler an instruction of such a chain costs about five clocks
+        // whatever it does: everything that does not depend on the vector (indices,
+        // inputs, the stage's wait, remote addresses) is done ahead of its arrival.
+        //
+        // A complex128 value is dealt to two lanes, one a component: an FP64 instruction
+        // holds its scheduler's pipe 64 clocks however few lanes are active.
+        constexpr int NC = sizeof(C) == 16 ? 2 : 1;
+        constexpr int V = 2 / NC;  // real values a lane holds of one complex value
+        // this warp's 16-byte column units of every row, and its columns
         const int U = T / VN;
         const int u0 = (warp * U) / CL_WARPS, u1 = ((warp + 1) * U) / CL_WARPS;
+        const int c0 = u0 * VN, nc = (u1 - u0) * VN;
+        const int dir = (phase == 0) != (side != 0) ? 1 : -1;  // block_of(b + 1) - block_of(b)
 
-        int chunk = 0;
+        // The rows of a chunk and their lanes: lane = row r (of 2^lg >= rows), then the
+        // column phase cp of CP = 2^lgc, no more phases than the warp has units.  ONE: a
+        // CTA's rows are one chunk, and all of this is loop-invariant.
+        struct Lay {
+            int rows, lg, lgc, r, cp;
+            bool on;
+        };
+        auto layout = [&](int rows) {
+            Lay y;
+            y.rows = rows;
+            y.lg = rows > 1 ? 32 - __clz(rows - 1) : 0;
+            y.lgc = min(5 - y.lg, u1 - u0 > 1 ? 32 - __clz(u1 - u0 - 1) : 0);
+            y.r = lane & ((1 << y.lg) - 1);
+            y.cp = lane >> y.lg;
+            y.on = y.r < rows && y.cp < (1 << y.lgc);
+            return y;
+        };
+        Lay L = layout(min(SR, myrows));
+
+        // t_k of a chunk's rows, several chunks a step: warp w takes those of job j = w out
+        // of its partial sums
+        auto fetch_t = [&](int64_t gr, int rows) {
+            if (lane < rows && warp < nr)
+                copy_async<16>(tpf + warp * SR + lane, s_out[warp] + (gr + lane < P.n ? gr + lane : 0), gr + lane < P.n);
+        };
+        // How the rows of a chunk are finished.  EVERY (up to two jobs in complex64):
+        // every warp adds up all rows' partial sums for itself and sends them to its own
+        // CTAs, a store to one CTA at a time whose lanes' addresses are contiguous.
+        // Otherwise LPE lanes share a (row, job), each adding up its share of the partial
+        // sums (complex128: of one component) and sending to its share of the CTAs.
+        constexpr bool EVERY = NC == 1 && R <= 2;
+        constexpr int LPE = R <= 2 ? 8 : (R == 4 || NC == 2 ? 4 : 2);
+        constexpr int DSTEP = EVERY ? CL_WARPS : LPE;
+        const int dst = EVERY ? warp : tid % LPE;  // first CTA this thread sends to
+        uint32_t rvec[2], rbar[2];
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            rvec[x] = mapa_u32(vbuf, min(dst + x * DSTEP, Ccl - 1));
+            rbar[x] = mapa_u32(vbar, min(dst + x * DSTEP, Ccl - 1));
+        }
+
+        int slot = 0, chunk = 0;
+        uint32_t spar = 0, vpar = 0;     // parities of the stages' round and of the vectors' round
+        int cur = 0, prv = 2;            // b % 3, (b - 1) % 3
         for (int b = 0; b < nsteps; ++b) {
             const bool fwd = phase == 0 || b == 0;
-            const int k = block_of(b);
-            const int64_t g0 = (int64_t)k * T;
-            const int cur = b % 3, prv = (b + 2) % 3;
-            const C* vprev = vbuf + (size_t)prv * R * T;  // t_outer (fwd) or x_inner (bwd)
-            const bool last = b == nsteps - 1;            // nobody reads the last vector: not sent
-            if (b > 0 && !failed_flag(&s_fail)) {
-                // the previous step's vector: every CTA's rows, delivered by st.async
-                const uint32_t par = (uint32_t)(((b - 1) / 3) & 1);
-                long long it = 0;
-                while (!mbar_try_wait_cluster(&vbar[prv], par)) {
-                    if (failed_flag(&s_fail)) break;
-                    if (++it > WAIT_LIMIT) {
-                        s_fail = 1;
-                        atomicExch(err, 3);
-                        break;
+            const int64_t g0 = (int64_t)block_of(b) * T;
+            const C* vprev = vbuf + prv * R * T;   // t_outer (fwd) or x_inner (bwd)
+            const bool last = b == nsteps - 1;     // nobody reads the last vector: not sent
+            // the step's inputs, off the chain
+            constexpr bool EARLY = R <= 2;  // more jobs: too many registers
+            constexpr int PF = NC;          // entries a lane
+            int in_n[PF], in_c[PF][NE];
+            C in_a[PF][NE];
+            Rt in_r[PF][EARLY ? R : 1][V];
+            C in_t = zero_c<C>();
+            auto read_part = [&](const double2* p, int cm, Rt (&v)[V]) {
+                const double* d = reinterpret_cast<const double*>(p);
+                if constexpr (NC == 2) {
+                    v[0] = d[cm];
+                } else {
+                    v[0] = (Rt)d[0];
+                    v[1] = (Rt)d[1];
+                }
+            };
+            // the stage and the inputs: there long before the vector
+            bounded([&] { return mbar_try_wait(&full[slot], spar); }, 2);
+            const double2* rin = rpf + (b & 1) * R * T + c0;
+            const int* bin = bpf + (b & 3) * 2 * T + c0;
+            if (phase == 0 && pf_ok) {
+#pragma unroll
+                for (int x = 0; x < PF; ++x) {
+                    const int id = lane + 32 * x, i = id / NC;
+                    in_n[x] = 0;
+                    if (id < nc * NC) {
+                        in_n[x] = bin[T + i] - bin[i];
+                        const int at = (b & 1) * NE * T + c0 + i;
+#pragma unroll
+                        for (int e = 0; e < NE; ++e)
+                            if (e < in_n[x]) {
+                                in_c[x][e] = cpf[at + e * T];
+                                in_a[x][e] = apf[at + e * T];
+                            }
+                        if constexpr (EARLY) {
+#pragma unroll
+                            for (int j = 0; j < R; ++j)
+                                if (j < nr) read_part(rin + j * T + i, id % NC, in_r[x][j]);
+                        }
                     }
                 }
             }
-            consumer_sync();  // also: the previous step's reads of sbuf and tbuf are done
-            // re-arm that barrier for step b+2 now: no CTA can send step b+2's rows
-            // before it has ours of step b+1, so the expected bytes are always
-            // registered before the first of them arrives
-            if (tid == 0 && b > 0 && !failed_flag(&s_fail) && b + 2 <= nsteps - 2)
-                mbar_expect_tx(&vbar[prv], vec_bytes);
-            const bool failed = failed_flag(&s_fail);
+            if constexpr (ONE && R == 1)
+                if (!fwd && warp == 0 && L.on) in_t = from_c128<C>(tpf[cur * SR + L.r]);
+            if (b > 0) {
+                // the previous step's vector: every CTA's rows, delivered by st.async
+                bounded([&] { return mbar_try_wait_cluster(&vbar[prv], vpar); }, 3);
+                // re-arm that barrier for step b+2 now: no CTA can send step b+2's rows
+                // before it has ours of step b+1, so the expected bytes are always
+                // registered before the first of them arrives
+                if (tid == 0 && b + 2 <= nsteps - 2) mbar_expect_tx(&vbar[prv], vec_bytes);
+            }
             if (fwd) {
-                // s_k = r_k - L_k t_outer: every CTA forms the whole block
-                if (failed) {
-                } else if (phase == 1) {
-                    // x_mid's: the couplings to both neighbours, their t from the copies
-                    for (int idx = tid; idx < T * nr; idx += CL_WARPS * 32) {
-                        const int i = idx % T, j = idx / T;
+                // s_k = r_k - L_k t_outer in this warp's columns
+                if (phase == 0 && pf_ok) {
+#pragma unroll
+                    for (int x = 0; x < PF; ++x) {
+                        const int id = lane + 32 * x, i = id / NC, cm = id % NC;
+                        if (id < nc * NC) {
+#pragma unroll
+                            for (int j = 0; j < R; ++j) {
+                                if (j >= nr) break;
+                                Rt v[V];
+                                if constexpr (EARLY) {
+#pragma unroll
+                                    for (int c = 0; c < V; ++c) v[c] = in_r[x][j][c];
+                                } else {
+                                    read_part(rin + j * T + i, cm, v);
+                                }
+                                const C* tj = vprev + j * T;
+                                auto entry = [&](const C a, const C t) {
+                                    if constexpr (NC == 2) {
+                                        v[0] = fma(-a.x, cm ? t.y : t.x, v[0]);
+                                        v[0] = fma(cm ? -a.y : a.y, cm ? t.x : t.y, v[0]);
+                                    } else {
+                                        v[0] -= a.x * t.x - a.y * t.y;
+                                        v[1] -= a.x * t.y + a.y * t.x;
+                                    }
+                                };
+#pragma unroll
+                                for (int e = 0; e < NE; ++e)
+                                    if (e < in_n[x]) entry(in_a[x][e], tj[in_c[x][e]]);
+                                for (int e = bin[i] + NE; e < bin[i] + in_n[x]; ++e) entry(Lval[e], tj[P.Lcol[e]]);
+                                C* d = sbuf + j * T + c0 + i;
+                                if constexpr (NC == 2) reinterpret_cast<double*>(d)[cm] = v[0];
+                                else *d = C{v[0], v[1]};
+                            }
+                        }
+                    }
+                } else {
+                    // without the fetched inputs; x_mid's (phase 1) takes the couplings to both
+                    // neighbours, their t from the copies
+                    for (int id = lane; id < nc * nr; id += 32) {
+                        const int i = c0 + id % nc, j = id / nc;
                         const int64_t g = g0 + i;
                         C v = zero_c<C>();
                         if (g < P.n) {
@@ -387,229 +571,242 @@ __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, J
                             for (int e = P.Lptr[g]; e < P.Lptr[g + 1]; ++e) {
                                 const C a = Lval[e];
                                 const int c = P.Lcol[e];
-                                const C t = from_c128<C>(tw[c < T ? g0 - T + c : g0 + c]);
+                                const C t = phase ? from_c128<C>(tw[c < T ? g0 - T + c : g0 + c]) : vprev[j * T + c];
                                 v.x -= a.x * t.x - a.y * t.y;
                                 v.y -= a.x * t.y + a.y * t.x;
                             }
                         }
-                        sbuf[(size_t)j * T + i] = v;
-                    }
-                    if (pf_ok && nsteps > 1) prefetch_bwd(block_of(1));
-                } else if (pf_ok) {
-                    if (tid < T) {
-                        const int i = tid;
-#pragma unroll
-                        for (int j = 0; j < R; ++j) {
-                            if (j >= nr) break;
-                            C v = from_c128<C>(pf_v[j]);
-                            if (pf_hi > pf_lo) {
-                                const C tt = vprev[(size_t)j * T + pf_c];
-                                v.x -= pf_a.x * tt.x - pf_a.y * tt.y;
-                                v.y -= pf_a.x * tt.y + pf_a.y * tt.x;
-                                for (int e = pf_lo + 1; e < pf_hi; ++e) {
-                                    const C a = Lval[e];
-                                    const C t2 = vprev[(size_t)j * T + P.Lcol[e]];
-                                    v.x -= a.x * t2.x - a.y * t2.y;
-                                    v.y -= a.x * t2.y + a.y * t2.x;
-                                }
-                            }
-                            sbuf[(size_t)j * T + i] = v;
-                        }
-                    }
-                    if (!last) prefetch_fwd(block_of(b + 1));
-                } else {
-                    for (int idx = tid; idx < T * nr; idx += CL_WARPS * 32) {
-                        const int i = idx % T, j = idx / T;
-                        const int64_t g = g0 + i;
-                        C v = zero_c<C>();
-                        if (g < P.n) {
-                            v = from_c128<C>(s_in[j][g]);
-                            const int e0 = P.Lptr[g], e1 = P.Lptr[g + 1];
-                            for (int e = e0; e < e1; ++e) {
-                                const C a = Lval[e];
-                                const C t = vprev[(size_t)j * T + P.Lcol[e]];
-                                v.x -= a.x * t.x - a.y * t.y;
-                                v.y -= a.x * t.y + a.y * t.x;
-                            }
-                        }
-                        sbuf[(size_t)j * T + i] = v;
+                        sbuf[j * T + i] = v;
                     }
                 }
-                consumer_sync();
+                __syncwarp();
             }
             const C* rhs = fwd ? sbuf : vprev;
-            if (!fwd && !failed) {
-                // t_k of this CTA's rows, for x_k = t_k - E_k x_inner (read after the next barrier)
-                if (pf_ok) {
-                    if (tid < myrows) {
-#pragma unroll
-                        for (int j = 0; j < R; ++j)
-                            if (j < nr) tbuf[(size_t)j * T + tid] = from_c128<C>(pf_v[j]);
-                    }
-                    if (!last) prefetch_bwd(block_of(b + 1));
-                } else {
-                    for (int idx = tid; idx < myrows * nr; idx += CL_WARPS * 32) {
-                        const int i = idx % myrows, j = idx / myrows;
-                        const int64_t g = g0 + r0 + i;
-                        tbuf[(size_t)j * T + i] = g < P.n ? from_c128<C>(s_out[j][g]) : zero_c<C>();
-                    }
+            for (int rs = r0; ONE ? rs == r0 : rs < r1; rs += SR, ++chunk) {
+                C* rbuf = red + (chunk & 1) * RW * R * SR;
+                if constexpr (!ONE) {
+                    if (rs > r0) bounded([&] { return mbar_try_wait(&full[slot], spar); }, 2);
+                    L = layout(min(SR, r1 - rs));
+                    // many rows a CTA: the matrices bound the step, not its chain
+                    if (!fwd) fetch_t(g0 + rs, L.rows);
                 }
-            }
-            for (int sub = 0; sub < nsub; ++sub, ++chunk) {
-                const int slot = chunk % NS;
-                C* rbuf = red + (size_t)(chunk & 1) * CL_WARPS * R * SR;
-                if (!failed_flag(&s_fail)) {
-                    const uint32_t par = (uint32_t)((chunk / NS) & 1);
-                    long long it = 0;
-                    while (!mbar_try_wait(&full[slot], par)) {
-                        if (failed_flag(&s_fail)) break;
-                        if (++it > WAIT_LIMIT) {
-                            s_fail = 1;
-                            atomicExch(err, 2);
-                            break;
-                        }
-                    }
-                }
-                const int rs = r0 + sub * SR;
-                const int rows = min(SR, r1 - rs);
-                // warp-uniform test: the GEMV's shuffles need every lane, and the
-                // flag can change under a warp's feet (the producer sets it too)
-                if (__all_sync(0xffffffffu, !failed_flag(&s_fail))) {
-                    // lane = row r (of SRp, the power of two >= rows) + SRp * column phase cp
-                    int lg = 0;
-                    while ((1 << lg) < rows) ++lg;
-                    const int SRp = 1 << lg;
-                    const int CP = 32 >> lg;
-                    const int r = lane & (SRp - 1), cp = lane >> lg;
-                    Rt acc[2 * R];
+                const int CP = 1 << L.lgc;
+                Rt acc[R][2];
 #pragma unroll
-                    for (int v = 0; v < 2 * R; ++v) acc[v] = Rt(0);
-                    auto mac = [&](const VT& mv, const VT (&xv)[R]) {
-#pragma unroll
-                        for (int j = 0; j < R; ++j) {
-#pragma unroll
-                            for (int e = 0; e < VN; ++e) {
-                                const C m = Vec16<C>::get(mv, e), x = Vec16<C>::get(xv[j], e);
-                                acc[2 * j] = fma(m.x, x.x, acc[2 * j]);
-                                acc[2 * j] = fma(-m.y, x.y, acc[2 * j]);
-                                acc[2 * j + 1] = fma(m.x, x.y, acc[2 * j + 1]);
-                                acc[2 * j + 1] = fma(m.y, x.x, acc[2 * j + 1]);
-                            }
-                        }
-                    };
-                    if (r < rows) {
-                        const VT* Mrow = reinterpret_cast<const VT*>(stage + ((size_t)slot * SR + r) * TP);
+                for (int j = 0; j < R; ++j) acc[j][0] = acc[j][1] = Rt(0);
+                if (L.on) {
+                    const VT* Mrow = reinterpret_cast<const VT*>(stage + (slot * SR + L.r) * TP);
+                    int u = u0 + L.cp;
+                    if constexpr (NC == 1) {
                         const VT* X = reinterpret_cast<const VT*>(rhs);  // unit u of job j at X[j * U + u]
-                        int u = u0 + cp;
-                        if constexpr (sizeof(C) == 8) {
-                            // complex64: the next unit's operands load while this one's FMAs run.
-                            // Packed FP32 pairs: pa_j += (m.x, m.x) * (x.x, x.y) and
-                            // pb_j += (m.y, m.y) * (x.x, x.y), so that m x = (pa.x - pb.y, pa.y + pb.x):
-                            // two paired FMAs per complex product instead of four scalar ones
-                            float2 pa[R], pb[R];
+                        // packed FP32 pairs, pa_j += (m.x, m.x) * (x.x, x.y) and
+                        // pb_j += (m.y, m.y) * (x.x, x.y), so that m x = (pa.x - pb.y, pa.y + pb.x):
+                        // two paired FMAs per complex product instead of four scalar ones
+                        float2 pa[R], pb[R];
 #pragma unroll
-                            for (int j = 0; j < R; ++j) pa[j] = pb[j] = make_float2(0.f, 0.f);
-                            auto mac2 = [&](const VT& mv, const VT (&xv)[R]) {
+                        for (int j = 0; j < R; ++j) pa[j] = pb[j] = make_float2(0.f, 0.f);
+                        auto units = [&](auto un) {
+                            constexpr int N = decltype(un)::value;
+                            VT mv[N], xv[N][R];
+#pragma unroll
+                            for (int i = 0; i < N; ++i) {
+                                mv[i] = Mrow[u + i * CP];
+#pragma unroll
+                                for (int j = 0; j < R; ++j) xv[i][j] = X[j * U + u + i * CP];
+                            }
+#pragma unroll
+                            for (int i = 0; i < N; ++i)
 #pragma unroll
                                 for (int e = 0; e < VN; ++e) {
-                                    const C m = Vec16<C>::get(mv, e);
+                                    const C m = Vec16<C>::get(mv[i], e);
                                     const float2 mr = make_float2(m.x, m.x), mi = make_float2(m.y, m.y);
 #pragma unroll
                                     for (int j = 0; j < R; ++j) {
-                                        const C x = Vec16<C>::get(xv[j], e);
+                                        const C x = Vec16<C>::get(xv[i][j], e);
                                         const float2 xx = make_float2(x.x, x.y);
                                         pa[j] = __ffma2_rn(mr, xx, pa[j]);
                                         pb[j] = __ffma2_rn(mi, xx, pb[j]);
                                     }
                                 }
-                            };
-                            if (u < u1) {
-                                VT mv = Mrow[u];
-                                VT xv[R];
+                            u += N * CP;
+                        };
+                        if constexpr (R == 1)
+                            while (u + 3 * CP < u1) units(std::integral_constant<int, 4>{});
+                        if constexpr (R <= 2)
+                            while (u + CP < u1) units(std::integral_constant<int, 2>{});
+                        while (u < u1) units(std::integral_constant<int, 1>{});
 #pragma unroll
-                                for (int j = 0; j < R; ++j) xv[j] = X[(size_t)j * U + u];
-                                while (true) {
-                                    const int un = u + CP;
-                                    const bool more = un < u1;
-                                    VT mn = mv;
-                                    VT xn[R];
-#pragma unroll
-                                    for (int j = 0; j < R; ++j) xn[j] = xv[j];
-                                    if (more) {
-                                        mn = Mrow[un];
-#pragma unroll
-                                        for (int j = 0; j < R; ++j) xn[j] = X[(size_t)j * U + un];
-                                    }
-                                    mac2(mv, xv);
-                                    if (!more) break;
-                                    mv = mn;
-#pragma unroll
-                                    for (int j = 0; j < R; ++j) xv[j] = xn[j];
-                                    u = un;
-                                }
-                            }
+                        for (int j = 0; j < R; ++j) {
+                            acc[j][0] = pa[j].x - pb[j].y;
+                            acc[j][1] = pa[j].y + pb[j].x;
+                        }
+                    } else {
+                        for (; u < u1; u += CP) {
+                            const C m = Mrow[u];
 #pragma unroll
                             for (int j = 0; j < R; ++j) {
-                                acc[2 * j] = pa[j].x - pb[j].y;
-                                acc[2 * j + 1] = pa[j].y + pb[j].x;
-                            }
-                        } else {
-                            for (; u < u1; u += CP) {
-                                const VT mv = Mrow[u];
-                                VT xv[R];
-#pragma unroll
-                                for (int j = 0; j < R; ++j) xv[j] = X[(size_t)j * U + u];
-                                mac(mv, xv);
+                                const C x = rhs[j * T + u];
+                                acc[j][0] = fma(m.x, x.x, acc[j][0]);
+                                acc[j][1] = fma(m.x, x.y, acc[j][1]);
+                                acc[j][0] = fma(-m.y, x.y, acc[j][0]);
+                                acc[j][1] = fma(m.y, x.x, acc[j][1]);
                             }
                         }
                     }
-                    // sum the column phases of each row
-                    for (int mask = 16; mask >= SRp; mask >>= 1) {
+                }
+                // Sum the column phases of each row: while a lane holds several jobs it keeps
+                // half of them and trades the other half with its partner, so that the
+                // stages cost R/2 + R/4 + ... sums instead of R each.
+                int jb = 0, width = R, dup = 0;
+                int cpart = -1;  // the component a lane has kept
 #pragma unroll
-                        for (int v = 0; v < 2 * R; ++v) acc[v] += __shfl_xor_sync(0xffffffffu, acc[v], mask);
-                    }
-                    if (cp == 0 && r < rows) {
+                for (int st = 0; st < 5; ++st) {
+                    if (st >= L.lgc) break;
+                    const int mask = 1 << (L.lg + L.lgc - 1 - st);
+                    const int w = R >> st;  // constant after unrolling
+                    if (w > 1) {
+                        const bool upper = (lane & mask) != 0;
 #pragma unroll
-                        for (int j = 0; j < R; ++j) {
-                            if (j < nr) {
-                                C v;
-                                v.x = acc[2 * j];
-                                v.y = acc[2 * j + 1];
-                                rbuf[((size_t)warp * R + j) * SR + r] = v;
+                        for (int j = 0; j < R / 2; ++j)
+                            if (j < w / 2) {
+#pragma unroll
+                                for (int v = 0; v < 2; ++v) {
+                                    const Rt give = upper ? acc[j][v] : acc[j + w / 2][v];
+                                    const Rt keep = upper ? acc[j + w / 2][v] : acc[j][v];
+                                    acc[j][v] = keep + __shfl_xor_sync(0xffffffffu, give, mask);
+                                }
                             }
+                        if (upper) jb += w / 2;
+                        width = w / 2;
+                    } else if (NC == 2 && (st == 0 || (R >> (st - 1)) > 1)) {
+                        // complex128: then a component, an FP64 addition less a stage
+                        const bool upper = (lane & mask) != 0;
+                        const Rt give = upper ? acc[0][0] : acc[0][1];
+                        const Rt keep = upper ? acc[0][1] : acc[0][0];
+                        acc[0][0] = keep + __shfl_xor_sync(0xffffffffu, give, mask);
+                        cpart = upper ? 1 : 0;
+                    } else {
+#pragma unroll
+                        for (int v = 0; v < V; ++v) acc[0][v] += __shfl_xor_sync(0xffffffffu, acc[0][v], mask);
+                        dup |= mask;
+                    }
+                }
+                if constexpr (!ONE) {
+                    if (!fwd) {
+                        copies_done();
+                        __syncwarp();
+                    }
+                }
+                if (L.on && (lane & dup) == 0) {
+                    const double2* tch = tpf + (ONE ? cur * R * SR : 0) + L.r;
+#pragma unroll
+                    for (int j = 0; j < R; ++j) {
+                        if (j < width && jb + j < nr) {
+                            if (!fwd && jb + j == warp) {  // R <= 8 jobs: one a warp
+                                if constexpr (!(ONE && R == 1)) in_t = from_c128<C>(tch[(jb + j) * SR]);
+                                acc[j][0] -= NC == 2 && cpart == 1 ? in_t.y : in_t.x;
+                                if (NC == 1 || cpart < 0) acc[j][1] -= in_t.y;
+                            }
+                            C* d = rbuf + ((jb + j) * SR + L.r) * RW + warp;
+                            if (NC == 1 || cpart < 0) *d = C{acc[j][0], acc[j][1]};
+                            else reinterpret_cast<Rt*>(d)[cpart] = acc[j][0];
                         }
                     }
                 }
                 consumer_sync();  // partial sums written; the stage is consumed
                 if (tid == 0) mbar_arrive(&empty[slot]);
-                if (!failed_flag(&s_fail)) {
-                    // one thread per (row, job): sum the warps' partials, store, broadcast
-                    for (int t = tid; t < rows * nr; t += CL_WARPS * 32) {
-                        const int r = t % rows, j = t / rows;
-                        C v = rbuf[(size_t)j * SR + r];
-#pragma unroll
-                        for (int w = 1; w < CL_WARPS; ++w) {
-                            const C p = rbuf[((size_t)w * R + j) * SR + r];
-                            v.x += p.x;
-                            v.y += p.y;
-                        }
-                        const int rr = rs + r;
-                        const int64_t g = g0 + rr;
-                        if (!fwd) v = csub(tbuf[(size_t)j * T + (rr - r0)], v);
-                        // send first: the peers wait for these rows, nobody here waits for the store
-                        if (!last) {
-                            C* loc = vbuf + (size_t)cur * R * T + (size_t)j * T + rr;
-                            for (int qq = 0; qq < Ccl; ++qq)
-                                st_async_c(mapa_u32(loc, qq), v, mapa_u32(&vbar[cur], qq));
-                        }
-                        // x_mid is every side's; side 0 stores it
-                        if (g < P.n && (phase == 0 || b > 0 || side == 0)) s_out[j][g] = to_c128(v);
+                const bool failed = failed_flag(&s_fail);
+                const int nel = nr << L.lg;  // (row, job) pairs, rows padded to a power of two
+                const Rt sgn = fwd ? Rt(1) : Rt(-1);
+                auto finished = [&](const C v, int r, int j) {
+                    if (failed) return;
+                    if (!last) {
+                        const uint32_t off = (uint32_t)(((cur * R + j) * T + rs + r) * (int)sizeof(C));
+                        const uint32_t boff = (uint32_t)(cur * (int)sizeof(uint64_t));
+                        if (dst < Cact) st_async_c(rvec[0] + off, v, rbar[0] + boff);
+                        if (dst + DSTEP < Cact) st_async_c(rvec[1] + off, v, rbar[1] + boff);
+                        if constexpr (DSTEP < 8)
+                            for (int qq = dst + 2 * DSTEP; qq < Cact; qq += DSTEP)
+                                st_async_c(mapa_u32(vbuf, qq) + off, v, mapa_u32(vbar, qq) + boff);
+                    } else if (dst == 0 && g0 + rs + r < P.n) {
+                        // the last vector; x_mid is every side's, side 0 stores it
+                        const int64_t g = g0 + rs + r;
+                        if (phase == 0 || b > 0 || side == 0) s_out[j][g] = to_c128(v);
                         // t_{mid±1}: the copy that launch 1 reads
-                        if (g < P.n && phase == 0 && last)
-                            s_out[j][g + ((int64_t)VS_W - out_slot) * js.n] = to_c128(v);
+                        if (phase == 0) s_out[j][g + ((int64_t)VS_W - out_slot) * js.n] = to_c128(v);
+                    }
+                };
+                if constexpr (EVERY) {
+                    for (int e = lane; e < nel; e += 32) {
+                        const int r = R == 1 ? e : e & ((1 << L.lg) - 1), j = R == 1 ? 0 : e >> L.lg;
+                        if (r >= L.rows) continue;
+                        const C* pr = rbuf + (j * SR + r) * RW;
+                        C p[CL_WARPS];
+#pragma unroll
+                        for (int w = 0; w < CL_WARPS; ++w) p[w] = pr[w];
+#pragma unroll
+                        for (int h = CL_WARPS / 2; h > 0; h /= 2)
+#pragma unroll
+                            for (int w = 0; w < h; ++w) {
+                                p[w].x += p[w + h].x;
+                                p[w].y += p[w + h].y;
+                            }
+                        finished(C{sgn * p[0].x, sgn * p[0].y}, r, j);
+                    }
+                } else {
+                    constexpr int PARTS = LPE / NC;
+                    const int comp = NC == 2 ? tid % 2 : 0, part = (tid % LPE) / NC;
+                    for (int e = tid / LPE; (e & ~(32 / LPE - 1)) < nel; e += CL_WARPS * 32 / LPE) {
+                        const int r = e & ((1 << L.lg) - 1), j = e >> L.lg;
+                        const bool in = r < L.rows && j < nr;
+                        const int at = (in ? j * SR + r : 0) * RW + part;
+                        C v;
+                        if constexpr (NC == 2) {
+                            const double* pr = reinterpret_cast<const double*>(rbuf + at) + comp;
+                            double a = pr[0];
+#pragma unroll
+                            for (int w = PARTS; w < CL_WARPS; w += PARTS) a += pr[2 * w];
+#pragma unroll
+                            for (int m = NC; m < LPE; m *= 2) a += __shfl_xor_sync(0xffffffffu, a, m);
+                            if (!fwd) a = -a;
+                            const double o = __shfl_xor_sync(0xffffffffu, a, 1);
+                            v.x = comp ? o : a;
+                            v.y = comp ? a : o;
+                        } else {
+                            const C* pr = rbuf + at;
+                            v = pr[0];
+#pragma unroll
+                            for (int w = PARTS; w < CL_WARPS; w += PARTS) {
+                                v.x += pr[w].x;
+                                v.y += pr[w].y;
+                            }
+#pragma unroll
+                            for (int m = 1; m < LPE; m *= 2) {
+                                v.x += __shfl_xor_sync(0xffffffffu, v.x, m);
+                                v.y += __shfl_xor_sync(0xffffffffu, v.y, m);
+                            }
+                            v = C{sgn * v.x, sgn * v.y};
+                        }
+                        if (in) finished(v, r, j);
                     }
                 }
+                if (++slot == NS) {
+                    slot = 0;
+                    spar ^= 1;
+                }
+                if (rs != r0) continue;
+                // Once a step, while its rows are on their way: the previous vector's rows of
+                // this CTA go to memory.  (That vector stays until the peers have our next rows.)
+                if (b > 0 && !failed && (phase == 0 || b > 1 || side == 0)) {
+                    const int64_t gp = g0 - (int64_t)dir * T + r0;
+                    for (int i = (CL_WARPS - 1 - warp) * 32 + lane; i < myrows; i += CL_WARPS * 32)
+                        if (gp + i < P.n)
+                            for (int j = 0; j < nr; ++j) s_out[j][gp + i] = to_c128(vprev[j * T + r0 + i]);
+                }
             }
+            if (b > 0 && prv == 2) vpar ^= 1;
+            prv = cur;
+            cur = cur == 2 ? 0 : cur + 1;
         }
     }
     // the cluster barrier keeps every CTA's shared memory alive until all peers
@@ -622,6 +819,7 @@ namespace {
 
 struct Plan {
     int R = 1, SR = 1, NS = 3, TP = 1;
+    int pf = 0;  // the right-hand sides' inputs are fetched ahead
     size_t smem = 0;
 };
 
@@ -634,42 +832,33 @@ int padded_row(int T, size_t cs) {
     return TP;
 }
 
-size_t plan_smem(const Plan& p, int T, size_t cs) {
-    return (size_t)p.NS * p.SR * p.TP * cs + (size_t)5 * p.R * T * cs + (size_t)2 * CL_WARPS * p.R * p.SR * cs +
-           (2 * p.NS + 3) * sizeof(uint64_t) + 16;
+// the chain's vectors and the inputs fetched ahead
+size_t vec_smem(int R, int T, size_t cs, bool pf) {
+    return (size_t)4 * R * T * cs +
+           (pf ? (size_t)T * (2 * R * sizeof(double2) + 2 * NE * (cs + sizeof(int)) + 8 * sizeof(int)) : 0);
 }
 
-// Largest R (right-hand sides per pass) and stage height SR that fit in
-// `budget` bytes of shared memory.
-bool make_plan(int T, size_t cs, int want_R, Plan& p, size_t budget = 220 * 1024) {
-    const int TP = padded_row(T, cs);
-    for (int R : {8, 4, 2, 1}) {
-        if (R > want_R && R != 1) continue;
-        const size_t vec = (size_t)5 * R * T * cs;
-        if (vec + 96 >= budget) continue;
-        const int NS = 3;
-        const size_t per_row = (size_t)NS * TP * cs + (size_t)2 * CL_WARPS * R * cs;
-        const int SR = (int)std::min<size_t>(32, (budget - vec - 96) / per_row);
-        if (SR < 1) continue;
-        p.R = R;
-        p.SR = SR;
-        p.NS = NS;
-        p.TP = TP;
-        p.smem = plan_smem(p, T, cs);
-        return true;
-    }
-    return false;
+// a stage row of R right-hand sides: partial sums, fetched t
+size_t row_smem(int R, size_t cs) { return (size_t)2 * RW * R * cs + 3 * R * sizeof(double2); }
+
+size_t plan_smem(const Plan& p, int T, size_t cs) {
+    return (size_t)p.NS * p.SR * p.TP * cs + vec_smem(p.R, T, cs, p.pf) + p.SR * row_smem(p.R, cs) +
+           (2 * p.NS + 3) * sizeof(uint64_t) + 32;
 }
 
 // Stage height for a CTA of Tc rows: each chunk of `rows` rows occupies the
 // lanes as rows x column phases with rows padded to a power of two, so the
-// estimate charges the padded rows' multiply-adds (FP32: 4 warp-instructions a clock per SM,
-// FP64: one per 16 clocks) plus a fixed cost per chunk (its waits, barrier and
-// epilogue, about 2 us).
+// estimate charges the padded rows' multiply-adds plus a fixed cost per chunk: its
+// waits, barrier and sums.  Clocks: complex128 64 an FP64 instruction on each
+// scheduler; complex64 measured at T = 200 on CTAs of 100 and 200 rows (16 and 25 rows
+// a chunk with eight right-hand sides: 1,790 and 3,110; 16 and 20 with one: 880 and
+// 1,100).
 int choose_rows(int Tc, int SRmax, int T, size_t cs, int R) {
     const int VN = (int)(16 / cs);
-    const int Uw = (T / VN + CL_WARPS - 1) / CL_WARPS;
-    const double per_fma = cs == 16 ? 16.0 : 0.25;
+    const bool dbl = cs == 16;
+    const int Uw = cdiv_up(T / VN, CL_WARPS);
+    const double per_unit = dbl ? R * 4 * 2 * 64.0 : R * VN * 14.0;
+    const double per_chunk = dbl ? 4000.0 : (R <= 2 ? 700.0 : 250.0);
     int best = SRmax;
     double best_c = 1e300;
     for (int SR = 1; SR <= SRmax; ++SR) {
@@ -679,7 +868,7 @@ int choose_rows(int Tc, int SRmax, int T, size_t cs, int R) {
             int SRp = 1;
             while (SRp < rows) SRp <<= 1;
             const int CP = 32 / SRp;
-            c += (double)((Uw + CP - 1) / CP) * R * VN * 4 * CL_WARPS * per_fma + 4000.0;
+            c += (double)((Uw + CP - 1) / CP) * per_unit + per_chunk;
         }
         if (c < best_c) {
             best_c = c;
@@ -689,20 +878,57 @@ int choose_rows(int Tc, int SRmax, int T, size_t cs, int R) {
     return best;
 }
 
+// The plan of R right-hand sides for CTAs of Tc rows in `budget` bytes of shared
+// memory: stage height, and whether inputs are fetched ahead.  That shortens the
+// chain; where its shared memory would cut a CTA's rows into more chunks, the
+// multiply-adds bound the step, not the chain (complex128, T = 200, eight
+// right-hand sides on a cluster of 16: stages of 3 rows instead of 9).
+bool make_plan(int T, size_t cs, int R, int Tc, Plan& p, size_t budget = 220 * 1024) {
+    p.R = R;
+    p.NS = 3;
+    p.TP = padded_row(T, cs);
+    auto height = [&](bool pf) {
+        const size_t vec = vec_smem(R, T, cs, pf) + 112;
+        if (vec >= budget) return 0;
+        const int most = (int)std::min<size_t>(32, (budget - vec) / ((size_t)p.NS * p.TP * cs + row_smem(R, cs)));
+        return most < 1 ? 0 : choose_rows(Tc, most, T, cs, R);
+    };
+    p.SR = height(false);
+    p.pf = T <= PF_T && p.SR >= 1 && height(true) == p.SR;
+    p.smem = plan_smem(p, T, cs);
+    return p.SR >= 1;
+}
+
+// Largest R (right-hand sides per pass), at most want_R, whose stages fit.
+int choose_R(int T, size_t cs, int want_R) {
+    Plan p;
+    for (int R : {8, 4, 2, 1})
+        if ((R <= want_R || R == 1) && make_plan(T, cs, R, T, p)) return R;
+    return 0;
+}
+
 template <class C, int R, int MINB> void set_smem_attr(size_t smem) {
     static size_t attr_set = 0;  // per instantiation
     static bool nonportable = false;
+    auto both = [](auto&& f) {
+        f(k_block_solve_cl<C, R, MINB, true, 0>);
+        f(k_block_solve_cl<C, R, MINB, true, 1>);
+        f(k_block_solve_cl<C, R, MINB, false, 0>);
+        f(k_block_solve_cl<C, R, MINB, false, 1>);
+    };
     if (!nonportable) {
         // clusters of up to 16 CTAs (beyond the portable 8) for launches of few groups
         // (where that is refused, the occupancy query reports no room for them)
-        if (cudaFuncSetAttribute(k_block_solve_cl<C, R, MINB>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-            cudaSuccess)
-            (void)cudaGetLastError();
+        both([](auto* k) {
+            if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+                (void)cudaGetLastError();
+        });
         nonportable = true;
     }
     if (smem > attr_set) {
-        SIM_CUDA(cudaFuncSetAttribute(k_block_solve_cl<C, R, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
+        both([&](auto* k) {
+            SIM_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        });
         attr_set = smem;
     }
 }
@@ -734,7 +960,7 @@ template <class C, int R, int MINB> int max_active_clusters(int Ccl, size_t smem
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = cluster_config(1, Ccl, smem, nullptr, attr);
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_block_solve_cl<C, R, MINB>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, k_block_solve_cl<C, R, MINB, true, 0>, &cfg) != cudaSuccess) {
         (void)cudaGetLastError();
         n = 0;
     }
@@ -748,10 +974,16 @@ void launch_cl(const Pencil& P, const JobSpace& js, int in_slot, int out_slot, v
     set_smem_attr<C, R, MINB>(pl.smem);
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = cluster_config(ngroups * (P.mid + 1 < P.nb ? 2 : 1), Ccl, pl.smem, st, attr);
-    for (int phase = P.mid > 0 ? 0 : 1; phase < 2; ++phase) {
-        SIM_CUDA(cudaLaunchKernelEx(&cfg, k_block_solve_cl<C, R, MINB>, P, js, in_slot, out_slot, fptrs, d_grp, pl.SR,
-                                    pl.NS, pl.TP, d_err, phase));
+    auto launch = [&](auto* kernel) {
+        SIM_CUDA(cudaLaunchKernelEx(&cfg, kernel, P, js, in_slot, out_slot, fptrs, d_grp, pl.SR, pl.NS, pl.TP, pl.pf, d_err));
         SIM_LAUNCH_CHECK();
+    };
+    if (cdiv_up(P.T, Ccl) <= pl.SR) {  // every CTA's rows in one chunk
+        if (P.mid > 0) launch(k_block_solve_cl<C, R, MINB, true, 0>);
+        launch(k_block_solve_cl<C, R, MINB, true, 1>);
+    } else {
+        if (P.mid > 0) launch(k_block_solve_cl<C, R, MINB, false, 0>);
+        launch(k_block_solve_cl<C, R, MINB, false, 1>);
     }
 }
 
@@ -767,18 +999,15 @@ struct Shape {
 // of two.  Two CTAs per SM are considered for single right-hand sides in
 // complex64, whose plan then fits in half of an SM's shared memory.
 template <class C, int R>
-Shape choose_shape(const Pencil& P, size_t cs, const Plan& base, int ng) {
+Shape choose_shape(const Pencil& P, size_t cs, int ng) {
     Shape best;
     double best_cost = 1e300;
     const int cmax = std::min(16, P.T);
     for (int minb = 1; minb <= 2; ++minb) {
         if (minb == 2 && !(kTwoPerSm && R == 1 && sizeof(C) == 8)) continue;
-        Plan pl = base;
-        if (minb == 2 && !make_plan(P.T, cs, R, pl, 110 * 1024)) continue;
         for (int c = 1; c <= cmax; ++c) {
-            Plan q = pl;
-            q.SR = choose_rows((P.T + c - 1) / c, pl.SR, P.T, cs, pl.R);
-            q.smem = plan_smem(q, P.T, cs);
+            Plan q;
+            if (!make_plan(P.T, cs, R, cdiv_up(P.T, c), q, minb == 2 ? 110 * 1024 : 220 * 1024)) continue;
             int maxc = 0;
             if constexpr (R == 1 && sizeof(C) == 8)
                 maxc = minb == 1 ? max_active_clusters<C, R, 1>(c, q.smem) : max_active_clusters<C, R, 2>(c, q.smem);
@@ -799,9 +1028,7 @@ Shape choose_shape(const Pencil& P, size_t cs, const Plan& base, int ng) {
     if (best_cost == 1e300) {  // no occupancy answer: one CTA per group
         best.Ccl = 1;
         best.minb = 1;
-        best.pl = base;
-        best.pl.SR = choose_rows(P.T, base.SR, P.T, cs, base.R);
-        best.pl.smem = plan_smem(best.pl, P.T, cs);
+        make_plan(P.T, cs, R, P.T, best.pl);
     }
     return best;
 }
@@ -834,17 +1061,17 @@ bool block_solve_cluster(const Pencil& P, int precision, const JobSpace& js, con
             groups.push_back({j});
         maxr = std::max<int>(maxr, (int)groups.back().size());
     }
-    Plan pl;
-    if (!make_plan(P.T, cs, maxr, pl)) return false;
+    const int R = choose_R(P.T, cs, maxr);
+    if (R == 0) return false;
     // split groups larger than the plan's R
     std::vector<std::vector<int>> gs;
     for (auto& g : groups)
-        for (size_t a = 0; a < g.size(); a += pl.R) gs.emplace_back(g.begin() + a, g.begin() + std::min(g.size(), a + pl.R));
+        for (size_t a = 0; a < g.size(); a += R) gs.emplace_back(g.begin() + a, g.begin() + std::min(g.size(), a + R));
     const int ng = (int)gs.size();
     const int nclusters = ng * (P.mid + 1 < P.nb ? 2 : 1);  // a cluster per side
-    std::vector<int> flat((size_t)ng * pl.R, -1);
+    std::vector<int> flat((size_t)ng * R, -1);
     for (int g = 0; g < ng; ++g)
-        for (size_t j = 0; j < gs[g].size(); ++j) flat[(size_t)g * pl.R + j] = gs[g][j];
+        for (size_t j = 0; j < gs[g].size(); ++j) flat[(size_t)g * R + j] = gs[g][j];
     if (!g_err) {
         SIM_CUDA(cudaMalloc(&g_err, sizeof(int)));
         SIM_CUDA(cudaMemset(g_err, 0, sizeof(int)));
@@ -875,18 +1102,18 @@ bool block_solve_cluster(const Pencil& P, int precision, const JobSpace& js, con
     SIM_CUDA(cudaEventRecord(g_grp_ev[fb], st));
     Shape sh;
     if (precision == SIM_FP64) {
-        if (pl.R == 8) sh = choose_shape<double2, 8>(P, cs, pl, nclusters);
-        else if (pl.R == 4) sh = choose_shape<double2, 4>(P, cs, pl, nclusters);
-        else if (pl.R == 2) sh = choose_shape<double2, 2>(P, cs, pl, nclusters);
-        else sh = choose_shape<double2, 1>(P, cs, pl, nclusters);
+        if (R == 8) sh = choose_shape<double2, 8>(P, cs, nclusters);
+        else if (R == 4) sh = choose_shape<double2, 4>(P, cs, nclusters);
+        else if (R == 2) sh = choose_shape<double2, 2>(P, cs, nclusters);
+        else sh = choose_shape<double2, 1>(P, cs, nclusters);
     } else {
-        if (pl.R == 8) sh = choose_shape<float2, 8>(P, cs, pl, nclusters);
-        else if (pl.R == 4) sh = choose_shape<float2, 4>(P, cs, pl, nclusters);
-        else if (pl.R == 2) sh = choose_shape<float2, 2>(P, cs, pl, nclusters);
-        else sh = choose_shape<float2, 1>(P, cs, pl, nclusters);
+        if (R == 8) sh = choose_shape<float2, 8>(P, cs, nclusters);
+        else if (R == 4) sh = choose_shape<float2, 4>(P, cs, nclusters);
+        else if (R == 2) sh = choose_shape<float2, 2>(P, cs, nclusters);
+        else sh = choose_shape<float2, 1>(P, cs, nclusters);
     }
     const int Ccl = sh.Ccl;
-    pl = sh.pl;
+    const Plan& pl = sh.pl;
     const double TT = (double)P.T * P.T, blocks = 2.0 * P.nb - 1.0;
     // instrumentation also files each launch under its shape (right-hand sides
     // per pass, CTAs per group), e.g. "block_solve_r8_c2"
