@@ -15,8 +15,9 @@
 //   panel   the owner's threads hold one row of the panel each, in registers;
 //           a pivot (the largest |re|+|im| of the rows not used yet, ties to the
 //           lower row) costs one warp reduction per 32 rows and one barrier of
-//           the panel's warps (two in FP64, where only the winner's warp divides:
-//           an FP64 warp instruction holds the SM's pipe for 16 clocks).  The
+//           the panel's warps (none with one warp; two in FP64 with more than four,
+//           where only the winner's warp divides: an FP64 warp instruction holds its
+//           scheduler's pipe for 64 clocks).  The
 //           panel becomes G: column j is what the panel's pivots make of unit
 //           vector e_{r_j}, r_j the row of pivot j.
 //   update  every CTA, its other columns: R = the pivot rows' old values,
@@ -108,7 +109,16 @@ template <int B> __device__ __forceinline__ void store_row(double2* p, const dou
     for (int j = 0; j < B; ++j) p[j] = v[j];
 }
 __device__ __forceinline__ float2 neg(float2 a) { return make_float2(-a.x, -a.y); }
-__device__ __forceinline__ double2 neg(double2 a) { return make_double2(-a.x, -a.y); }
+// in complex128 by integer operations: negations and comparisons go through the FP64 pipe
+__device__ __forceinline__ double neg(double a) {
+    return __hiloint2double(__double2hiint(a) ^ (int)0x80000000, __double2loint(a));
+}
+__device__ __forceinline__ double2 neg(double2 a) { return make_double2(neg(a.x), neg(a.y)); }
+__device__ __forceinline__ bool is_zero(float2 a) { return a.x == 0.f && a.y == 0.f; }
+__device__ __forceinline__ bool is_zero(double2 a) {
+    return (((uint32_t)(__double2hiint(a.x) | __double2hiint(a.y)) << 1) | (uint32_t)__double2loint(a.x) |
+            (uint32_t)__double2loint(a.y)) == 0u;
+}
 
 constexpr int FC_MAXW = 16;  // panel warps: T <= 512 rows
 
@@ -331,29 +341,35 @@ __global__ void __launch_bounds__(NT, 1) k_factor_cl(Pencil P, const int* shift_
         for (int jj = 0; jj < bw; ++jj) {
             const int bo = (jj & 1) * FC_MAXW;
             const uint32_t ball = __ballot_sync(0xffffffffu, win);
-            if (ball == 0u ? lane == 0 : lane == __ffs(ball) - 1) {
-                ckey[bo + warp] = make_uint4(ball ? mh : 0u, ml, (uint32_t)r, 0u);
+            const int wl = ball == 0u ? 0 : __ffs(ball) - 1;
+            if (lane == wl) {
+                if (PW > 1) ckey[bo + warp] = make_uint4(ball ? mh : 0u, ml, (uint32_t)r, 0u);
                 store_row<B>(cand + (size_t)(bo + warp) * B, a);
             }
-            bar_panel(PW * 32);
-            // the winner among the warps' candidates: largest key, lowest warp (lowest row)
-            const uint4 ck = ckey[bo + (lane < PW ? lane : 0)];
-            const uint32_t wh = __reduce_max_sync(0xffffffffu, ck.x);
-            bool wm = ck.x == wh;
-            if constexpr (sizeof(C) == 16) {
-                const uint32_t wl = __reduce_max_sync(0xffffffffu, wm ? ck.y : 0u);
-                wm = wm && ck.y == wl;
+            int ws = 0, row = wl;
+            if (PW == 1) {
+                __syncwarp();
+            } else {
+                bar_panel(PW * 32);
+                // the winner among the warps' candidates: largest key, lowest warp (lowest row)
+                const uint4 ck = ckey[bo + (lane < PW ? lane : 0)];
+                const uint32_t wh = __reduce_max_sync(0xffffffffu, ck.x);
+                bool wm = ck.x == wh;
+                if constexpr (sizeof(C) == 16) {
+                    const uint32_t wl = __reduce_max_sync(0xffffffffu, wm ? ck.y : 0u);
+                    wm = wm && ck.y == wl;
+                }
+                ws = __ffs(__ballot_sync(0xffffffffu, wm)) - 1;
+                row = (int)__shfl_sync(0xffffffffu, ck.z, ws);
             }
-            const int ws = __ffs(__ballot_sync(0xffffffffu, wm)) - 1;
-            const int row = (int)__shfl_sync(0xffffffffu, ck.z, ws);
             C pr[B];
             load_row<B>(cand + (size_t)(bo + ws) * B, pr);
-            if (pr[0].x == 0 && pr[0].y == 0) {  // singular Schur complement
+            if (is_zero(pr[0])) {  // singular Schur complement
                 pr[0].x = (decltype(pr[0].x))1e-30;
                 if (tid == 0) atomicExch(err, 1);
             }
             C inv;
-            if constexpr (sizeof(C) == 8) {
+            if (sizeof(C) == 8 || PW <= 4) {  // (four: a warp per scheduler)
                 inv = crecip(pr[0]);
             } else {
                 if (warp == ws) {

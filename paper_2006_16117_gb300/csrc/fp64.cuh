@@ -52,7 +52,7 @@ __device__ __forceinline__ double scale2(double v, int k) {
 }
 
 // 1 / a (seven FP64 operations): 1/d, d = |a 2^k|^2 in [1, 8), is r + r (e + e^2) with
-// e = 1 - d r from an FP32 reciprocal r (e^3 < 2^-66).
+// e = 1 - d r from an FP32 reciprocal r (2 ulp: e^3 < 2^-60).
 __device__ __forceinline__ double2 crecip(double2 a) {
     const int e = max((__double2hiint(a.x) >> 20) & 2047, (__double2hiint(a.y) >> 20) & 2047);
     if (e < 64 || e > 1983) {  // far out: by division
@@ -65,7 +65,7 @@ __device__ __forceinline__ double2 crecip(double2 a) {
     const double d = fma(x, x, y * y);  // [1, 8)
     const uint32_t hd = (uint32_t)__double2hiint(d), ld = (uint32_t)__double2loint(d);
     const float f = __uint_as_float(((((hd >> 20) & 2047u) - 1023u + 127u) << 23) | ((hd & 0xFFFFFu) << 3) | (ld >> 29));
-    const uint32_t g = __float_as_uint(1.0f / f);
+    const uint32_t g = __float_as_uint(__fdividef(1.0f, f));
     const double r0 = __hiloint2double((int)((((g >> 23) - 127u + 1023u) << 20) | ((g & 0x7FFFFFu) >> 3)), (int)(g << 29));
     const double t = fma(-d, r0, 1.0);
     const double r = fma(r0, fma(t, t, t), r0);
