@@ -38,9 +38,9 @@
 //
 // Measured for one shift, T = 200, nb = 200 complex64: 138 ms with rows over the
 // cluster and two cluster barriers a pivot, 39.7 with the panels (2,050 clocks a
-// pivot, about 1,000 of them the pivot itself), 20.1 from both ends; T = 98, nb =
-// 97 complex128: 106, 31.6, 16.0 ms; T = 30, nb = 30 complex128: 5.6, 2.2, 1.2 ms.
-// 55 shifts of T = 200 complex64 in two calls: 372 -> 80 ms.
+// pivot, about 1,000 of them the pivot itself), 20.1 from both ends, 16.3 on 13 CTAs
+// a side; T = 98, nb = 97 complex128: 106, 31.6, 16.0, 12.7 ms; T = 30, nb = 30
+// complex128: 5.6, 2.2, 1.2, 0.97 ms.  56 shifts of T = 200 complex64: 372 -> 53 ms.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -670,10 +670,13 @@ int active_clusters(size_t cs, const FactorShape& f) {
 
 // Launch shape by an estimate of the clocks of one block: T pivots in panels of
 // B, each panel's chain (its pivots, the next panel's columns, and with more than
-// one CTA the cluster barrier and G's way through L2: 3,000 clocks measured, 600
-// for one CTA) or its share of the update (68% of the FP32 rate measured, all of
-// FP64's), whichever is longer, times the waves the shifts need.  So one CTA takes
-// T up to about 140 in complex64, four T = 200, and every shift runs in one wave if the GPU holds it.
+// one CTA the cluster barrier and G's way through L2: 1,500 clocks) plus a part of
+// the CTA's own columns' work (the update, which shares the FP64 pipe or the issue
+// slots with the panel, and the forming and storing of the block's columns) or that
+// work plus a part of the chain, times the waves the shifts need.  Why the sum and
+// not the larger: T = 200 complex64 on 4, 7, 13 CTAs 20.0, 17.4, 16.3 ms in panels of 8 (20.1, 18.2,
+// 17.5 of 16); T = 102 on 1, 3, 7 CTAs 5.5, 4.6, 4.1 ms; T = 98 complex128 on 5, 7,
+// 13 CTAs 16.7, 15.3, 12.7 ms; T = 30 on 1, 2, 4 CTAs 1.09, 1.02, 0.97 ms.
 FactorShape choose_factor_shape(int T, size_t cs, int count) {
     FactorShape best;
     double best_cost = 1e300;
@@ -693,11 +696,12 @@ FactorShape choose_factor_shape(int T, size_t cs, int count) {
             const int active = active_clusters(cs, f);
             if (active <= 0) continue;
             const int np = (T + B - 1) / B;
-            const double pivot = f64 ? 64.0 * B * PW + 1300.0 : 350.0 + 8.0 * B;
+            const double pivot = f64 ? 64.0 * B * PW + 1300.0 : 500.0 + 30.0 * B + 40.0 * PW;
             const double look = f64 ? 2.2 * T * B * B : 0.07 * T * B * B + 500.0;
-            const double chain = B * pivot + look + (C > 1 ? 3000.0 : 600.0);
-            const double upd = (f64 ? 2.2 : 0.06) * (double)T * T * f.Tc / np + (C > 1 ? 2000.0 : 600.0);
-            const double cost = (double)((count + active - 1) / active) * np * std::max(chain, upd);
+            const double chain = B * pivot + look + (C > 1 ? 1500.0 : 300.0);
+            const double own = (f64 ? 2.2 : 0.06) * (double)T * T * f.Tc / np;
+            const double panel = std::max(chain + (f64 ? 0.65 : 0.8) * own, own + 0.5 * chain);
+            const double cost = (double)((count + active - 1) / active) * np * panel;
             if (cost < best_cost) {
                 best_cost = cost;
                 best = f;
