@@ -120,7 +120,9 @@ typedef struct {
                                  with partial pivoting of I + (σ - z) H_m at every node */
     int32_t separable_tensor_cores; /* mixed precision with sim_set_separable: 1 (default) the mode
                                  products on the tensor cores (tcgen05, TF32 with hi/lo splitting to
-                                 FP32 accuracy); 0: FP32 CUDA-core GEMMs */
+                                 FP32 accuracy), or for 2-D grids that a thread-block cluster
+                                 holds the whole apply in one kernel of FP32 FMAs where that is
+                                 estimated to be faster; 0: FP32 CUDA-core GEMMs */
 } sim_options;
 
 /* Counters of the last set_region .. multiplicity sequence. */
