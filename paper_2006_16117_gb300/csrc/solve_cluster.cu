@@ -188,12 +188,22 @@ __device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;
 
 __device__ __forceinline__ bool failed_flag(const int* f) { return *(const volatile int*)f != 0; }
 
+// The launch's groups: R jobs each, -1 past a group's last.  As a parameter up to
+// MAX jobs (a copy between the kernels of a stream costs about 5 us of its time), in
+// device memory (`far`) beyond.
+struct Groups {
+    static constexpr int MAX = 512;
+    const int* far;
+    short near[MAX];
+    __device__ __forceinline__ int job(int i) const { return far ? far[i] : near[i]; }
+};
+
 // MINB: CTAs per SM the launch is built for (2 caps the registers at 112 so
 // that two CTAs of at most ~112 KB of shared memory share an SM)
 template <class C, int R, int MINB, bool ONE, int phase>
 __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, JobSpace js, int in_slot,
                                                                   int out_slot, void* const* fptrs,
-                                                                  const int* grp_jobs, int SR, int NS, int TP, int pf_ok,
+                                                                  const __grid_constant__ Groups groups, int SR, int NS, int TP, int pf_ok,
                                                                   int* err) {
     cg::cluster_group cl = cg::this_cluster();
     const int Ccl = (int)cl.num_blocks();
@@ -219,10 +229,10 @@ __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, J
     int nr = 1;
 #pragma unroll
     for (int j = 1; j < R; ++j)
-        if (grp_jobs[grp * R + j] >= 0) nr = j + 1;
-    const int job0 = grp_jobs[grp * R];
+        if (groups.job(grp * R + j) >= 0) nr = j + 1;
+    const int job0 = groups.job(grp * R);
     if (tid < R) {
-        const int jb = grp_jobs[grp * R + tid];
+        const int jb = groups.job(grp * R + tid);
         const int jj = jb >= 0 ? jb : job0;
         s_in[tid] = js.vec + (size_t)jj * js.vstride + (size_t)in_slot * js.n;
         s_out[tid] = js.vec + (size_t)jj * js.vstride + (size_t)out_slot * js.n;
@@ -969,13 +979,13 @@ template <class C, int R, int MINB> int max_active_clusters(int Ccl, size_t smem
 }
 
 template <class C, int R, int MINB>
-void launch_cl(const Pencil& P, const JobSpace& js, int in_slot, int out_slot, void* const* fptrs, const int* d_grp,
+void launch_cl(const Pencil& P, const JobSpace& js, int in_slot, int out_slot, void* const* fptrs, const Groups& groups,
                int ngroups, int Ccl, const Plan& pl, int* d_err, cudaStream_t st) {
     set_smem_attr<C, R, MINB>(pl.smem);
     cudaLaunchAttribute attr[1];
     const cudaLaunchConfig_t cfg = cluster_config(ngroups * (P.mid + 1 < P.nb ? 2 : 1), Ccl, pl.smem, st, attr);
     auto launch = [&](auto* kernel) {
-        SIM_CUDA(cudaLaunchKernelEx(&cfg, kernel, P, js, in_slot, out_slot, fptrs, d_grp, pl.SR, pl.NS, pl.TP, pl.pf, d_err));
+        SIM_CUDA(cudaLaunchKernelEx(&cfg, kernel, P, js, in_slot, out_slot, fptrs, groups, pl.SR, pl.NS, pl.TP, pl.pf, d_err));
         SIM_LAUNCH_CHECK();
     };
     if (cdiv_up(P.T, Ccl) <= pl.SR) {  // every CTA's rows in one chunk
@@ -1076,30 +1086,36 @@ bool block_solve_cluster(const Pencil& P, int precision, const JobSpace& js, con
         SIM_CUDA(cudaMalloc(&g_err, sizeof(int)));
         SIM_CUDA(cudaMemset(g_err, 0, sizeof(int)));
     }
-    if ((int)flat.size() > g_grp_cap) {
-        if (g_grp) {
-            SIM_CUDA(cudaStreamSynchronize(st));
-            cudaFree(g_grp);
+    Groups table;
+    table.far = nullptr;
+    if ((int)flat.size() <= Groups::MAX && js.J <= 32767) {
+        std::copy(flat.begin(), flat.end(), table.near);
+    } else {
+        if ((int)flat.size() > g_grp_cap) {
+            if (g_grp) {
+                SIM_CUDA(cudaStreamSynchronize(st));
+                cudaFree(g_grp);
+            }
+            g_grp_cap = (int)flat.size() * 2;
+            SIM_CUDA(cudaMalloc(&g_grp, sizeof(int) * g_grp_cap * 2));
         }
-        g_grp_cap = (int)flat.size() * 2;
-        SIM_CUDA(cudaMalloc(&g_grp, sizeof(int) * g_grp_cap * 2));
-    }
-    if ((int)flat.size() > g_grp_h_cap) {
-        for (int b = 0; b < 2; ++b) {
-            if (g_grp_ev[b]) SIM_CUDA(cudaEventSynchronize(g_grp_ev[b]));
-            if (g_grp_h[b]) cudaFreeHost(g_grp_h[b]);
-            SIM_CUDA(cudaMallocHost(&g_grp_h[b], sizeof(int) * flat.size() * 2));
-            if (!g_grp_ev[b]) SIM_CUDA(cudaEventCreateWithFlags(&g_grp_ev[b], cudaEventDisableTiming));
+        if ((int)flat.size() > g_grp_h_cap) {
+            for (int b = 0; b < 2; ++b) {
+                if (g_grp_ev[b]) SIM_CUDA(cudaEventSynchronize(g_grp_ev[b]));
+                if (g_grp_h[b]) cudaFreeHost(g_grp_h[b]);
+                SIM_CUDA(cudaMallocHost(&g_grp_h[b], sizeof(int) * flat.size() * 2));
+                if (!g_grp_ev[b]) SIM_CUDA(cudaEventCreateWithFlags(&g_grp_ev[b], cudaEventDisableTiming));
+            }
+            g_grp_h_cap = (int)flat.size() * 2;
         }
-        g_grp_h_cap = (int)flat.size() * 2;
+        const int fb = g_grp_flip;
+        g_grp_flip ^= 1;
+        SIM_CUDA(cudaEventSynchronize(g_grp_ev[fb]));  // the copy that last used this buffer is done
+        std::copy(flat.begin(), flat.end(), g_grp_h[fb]);
+        table.far = g_grp + (size_t)fb * g_grp_cap;
+        SIM_CUDA(cudaMemcpyAsync(const_cast<int*>(table.far), g_grp_h[fb], sizeof(int) * flat.size(), cudaMemcpyHostToDevice, st));
+        SIM_CUDA(cudaEventRecord(g_grp_ev[fb], st));
     }
-    const int fb = g_grp_flip;
-    g_grp_flip ^= 1;
-    SIM_CUDA(cudaEventSynchronize(g_grp_ev[fb]));  // the copy that last used this buffer is done
-    std::copy(flat.begin(), flat.end(), g_grp_h[fb]);
-    int* d_grp = g_grp + (size_t)fb * g_grp_cap;
-    SIM_CUDA(cudaMemcpyAsync(d_grp, g_grp_h[fb], sizeof(int) * flat.size(), cudaMemcpyHostToDevice, st));
-    SIM_CUDA(cudaEventRecord(g_grp_ev[fb], st));
     Shape sh;
     if (precision == SIM_FP64) {
         if (R == 8) sh = choose_shape<double2, 8>(P, cs, nclusters);
@@ -1122,7 +1138,7 @@ bool block_solve_cluster(const Pencil& P, int precision, const JobSpace& js, con
     kprof_begin("block_solve", st);
     kprof_begin(shape, st);
 #define SIM_LAUNCH_R(CT, RR, MB) \
-    launch_cl<CT, RR, MB>(P, js, in_slot, out_slot, d_factor_ptrs, d_grp, ng, Ccl, pl, g_err, st)
+    launch_cl<CT, RR, MB>(P, js, in_slot, out_slot, d_factor_ptrs, table, ng, Ccl, pl, g_err, st)
     if (precision == SIM_FP64) {
         if (pl.R == 8) SIM_LAUNCH_R(double2, 8, 1);
         else if (pl.R == 4) SIM_LAUNCH_R(double2, 4, 1);

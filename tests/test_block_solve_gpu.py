@@ -65,3 +65,19 @@ def test_right_hand_sides_of_a_shift(simlib, precision, grid, k):
     assert np.max(np.min(np.abs(lam[None, :] - eig[:, None]), axis=1)) <= 1e-6
     assert np.array_equal(mult, np.ones(eig.size, dtype=int)) and eig.size >= 1
     assert st["max_gmres_iterations"] <= 8
+
+
+def test_more_groups_than_a_launch_carries(simlib):
+    """Many shifts with 64 vectors each: the table of groups goes through device
+    memory instead of the launch's parameters."""
+    from test_levels_small_gpu import _locate
+    from workloads import cd2d_csr, cd2d_eigenvalues, complex_gaussian
+    from workloads.configs import window_region
+
+    A = cd2d_csr(12, (1.0, 0.5))
+    lam = np.sort(cd2d_eigenvalues(12, (1.0, 0.5)).real)
+    region = window_region(lam, 20, 90)
+    _, eig, mult, st = _locate(simlib, A, region, complex_gaussian(A.n, 0), precision="mixed", mult_k=64)
+    assert st["num_shifts"] * 64 > 512
+    assert np.max(np.min(np.abs(lam[None, :] - eig[:, None]), axis=1)) <= 1e-6
+    assert np.array_equal(mult, np.ones(eig.size, dtype=int)) and eig.size >= 80
