@@ -33,10 +33,10 @@
 // instruction buffer each costs about five clocks.  Hence a kernel per phase and
 // per "one chunk a step" (ONE), the inputs brought by the producers, one barrier a
 // step, the vector stored to memory a step later by warps that wait anyway, and row
-// layouts that are powers of two.  Two sides, T = 200 complex64: 378 -> 268 us
-// (a step 3,800 -> 2,900 clocks forward, 3,100 -> 2,300 backward); T = 102 197 -> 127;
-// eight right-hand sides at T = 102 196 -> 138 us a launch; complex128 T = 30
-// 106 -> 58, T = 98 335 -> 201.  With 56 shifts at T = 200 the matrices bound it:
+// layouts that are powers of two.  Launch 1 starts under launch 0 and fills its stages
+// (5 us a solve).  Two sides, T = 200 complex64: 378 -> 263 us (a step 3,800 -> 2,900
+// clocks forward, 3,100 -> 2,300 backward); T = 102 197 -> 123; eight right-hand sides at
+// T = 102 196 -> 138 us a launch; complex128 T = 30 106 -> 53, T = 98 335 -> 195.  With 56 shifts at T = 200 the matrices bound it:
 // 1,446 -> 1,159 us (5.0 TB/s) in complex64, 12.4 -> 10.2 ms in complex128 (FP64 pipe).
 //
 // Every wait on an mbarrier has an iteration limit; a thread whose wait runs
@@ -278,6 +278,13 @@ __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, J
     if (tid == 0)
         for (int i = 0; i < 3 && i <= nsteps - 2; ++i) mbar_expect_tx(&vbar[i], vec_bytes);  // steps 0, 1, 2
     cl.sync();  // every CTA of the cluster is running, barriers initialised and armed, before any remote store
+    // Launch 1 starts while launch 0 runs (where SMs are free) and fills its stages; it
+    // waits for launch 0's end before it reads or writes a vector.  The factors are older
+    // than launch 0, which starts after everything before it has ended.
+    if (phase == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    auto vectors_ready = [&] {
+        if (phase == 1) asm volatile("griddepcontrol.wait;" ::: "memory");
+    };
 
     // A wait that gives up once the CTA has failed, or after WAIT_LIMIT polls.
     auto bounded = [&](auto&& done, int code) {
@@ -365,6 +372,7 @@ __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, J
                 for (int i = pt; i < rows; i += PROD)
                     tma_load_1d(dst + (size_t)i * TP, M + (size_t)(rs + i) * T, (uint32_t)(T * sizeof(C)),
                                 &full[slot]);
+                if (b == 0 && rs == r0) vectors_ready();
                 if (!ONE && myrows <= SR && b >= 2) {
                     // one chunk a step in this CTA: the inputs' buffer, as above
                     if (lane == 0)
@@ -471,6 +479,7 @@ __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, J
             rbar[x] = mapa_u32(vbar, min(dst + x * DSTEP, Ccl - 1));
         }
 
+        vectors_ready();
         int slot = 0, chunk = 0;
         uint32_t spar = 0, vpar = 0;     // parities of the stages' round and of the vectors' round
         int cur = 0, prv = 2;            // b % 3, (b - 1) % 3
@@ -982,18 +991,22 @@ template <class C, int R, int MINB>
 void launch_cl(const Pencil& P, const JobSpace& js, int in_slot, int out_slot, void* const* fptrs, const Groups& groups,
                int ngroups, int Ccl, const Plan& pl, int* d_err, cudaStream_t st) {
     set_smem_attr<C, R, MINB>(pl.smem);
-    cudaLaunchAttribute attr[1];
-    const cudaLaunchConfig_t cfg = cluster_config(ngroups * (P.mid + 1 < P.nb ? 2 : 1), Ccl, pl.smem, st, attr);
-    auto launch = [&](auto* kernel) {
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = cluster_config(ngroups * (P.mid + 1 < P.nb ? 2 : 1), Ccl, pl.smem, st, attr);
+    // launch 1 may start before launch 0 has ended (griddepcontrol in the kernel)
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    auto launch = [&](auto* kernel, bool after) {
+        cfg.numAttrs = after ? 2 : 1;
         SIM_CUDA(cudaLaunchKernelEx(&cfg, kernel, P, js, in_slot, out_slot, fptrs, groups, pl.SR, pl.NS, pl.TP, pl.pf, d_err));
         SIM_LAUNCH_CHECK();
     };
     if (cdiv_up(P.T, Ccl) <= pl.SR) {  // every CTA's rows in one chunk
-        if (P.mid > 0) launch(k_block_solve_cl<C, R, MINB, true, 0>);
-        launch(k_block_solve_cl<C, R, MINB, true, 1>);
+        if (P.mid > 0) launch(k_block_solve_cl<C, R, MINB, true, 0>, false);
+        launch(k_block_solve_cl<C, R, MINB, true, 1>, P.mid > 0);
     } else {
-        if (P.mid > 0) launch(k_block_solve_cl<C, R, MINB, false, 0>);
-        launch(k_block_solve_cl<C, R, MINB, false, 1>);
+        if (P.mid > 0) launch(k_block_solve_cl<C, R, MINB, false, 0>, false);
+        launch(k_block_solve_cl<C, R, MINB, false, 1>, P.mid > 0);
     }
 }
 
