@@ -1,0 +1,29 @@
+"""The block solve's waits that one lane makes for its warp: all lanes have to get
+the outcome, or those of a failed wait would wait in the next warp-wide
+instruction for a lane that has gone on (read from the source: a wait that runs
+out is not provoked on a GPU)."""
+import os
+import re
+
+SRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                   "paper_2006_16117_gb300", "csrc", "solve_cluster.cu")
+
+
+def _producers():
+    s = open(SRC).read()
+    return s[s.index("// ---- producers"): s.index("// ---- consumers")]
+
+
+def test_every_wait_of_one_lane_is_broadcast_to_its_warp():
+    text = _producers()
+    waits = [m.start() for m in re.finditer(r"\bbounded\(", text)]
+    assert waits
+    for at in waits:
+        # the outcome's variable, and what follows the statement that waits: the next
+        # warp-wide instruction has to hand that variable to all lanes
+        name = re.search(r"(\w+) = $", text[:at]).group(1)
+        nxt = re.search(r"__(shfl|syncwarp|any|all|ballot|reduce)\w*", text[at:])
+        assert nxt is not None and nxt.group(0).startswith("__shfl"), text[at: at + 200]
+        args = text[at + nxt.end(): at + nxt.end() + 60]
+        assert re.match(r"\(0xffffffffu, \(int\)%s, 0\)" % name, args), args
+        assert "break" not in text[at: at + nxt.start()] and "continue" not in text[at: at + nxt.start()]
