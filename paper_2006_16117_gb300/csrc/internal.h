@@ -71,13 +71,14 @@ inline size_t factor_storage_bytes(const Pencil& P, int precision) {
 __host__ __device__ inline size_t factor_lval_offset(const Pencil& P) { return (size_t)2 * P.nb * P.T * P.T; }
 
 // Host side of a job space, kept with its buffers: pinned memory (the device
-// writes istat and worst, the host fills act), the list last uploaded and the
+// writes istat, worst and err, the host fills act), the list last uploaded and the
 // iterations every job of the last solve took.
 struct JobHost {
     int J = 0;
     int* istat = nullptr;
     double* worst = nullptr;
     int* act = nullptr;
+    int* err = nullptr;            // code of a block solve's wait that ran out, else 0
     cudaEvent_t act_ev = nullptr;  // the last upload from `act`
     std::vector<int> uploaded;
     int usual_steps = 0;
@@ -88,6 +89,7 @@ struct JobHost {
         if (istat) cudaFreeHost(istat);
         if (worst) cudaFreeHost(worst);
         if (act) cudaFreeHost(act);
+        if (err) cudaFreeHost(err);
         if (act_ev) cudaEventDestroy(act_ev);
     }
 };

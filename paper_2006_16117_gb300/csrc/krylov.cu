@@ -586,6 +586,7 @@ bool inner_solve(const Pencil& P, const sim_options& opt, JobSpace& js, const st
             gram_schmidt(a, na, st);
             if (first && i + 1 < usual) continue;
             SIM_CUDA(cudaStreamSynchronize(st));
+            block_solve_check(*js.host);
             std::vector<int> next;
             for (int j : act)
                 if (!ist[j * IS_N + IS_CYCLE_DONE]) next.push_back(j);
@@ -599,6 +600,7 @@ bool inner_solve(const Pencil& P, const sim_options& opt, JobSpace& js, const st
         k_gm_check<<<ni, 256, 0, st>>>(js, opt.inner_tol, opt.inner_max_iter, d_sigma, P.anorm, P.bnorm);
         SIM_LAUNCH_CHECK();
         SIM_CUDA(cudaStreamSynchronize(st));
+        block_solve_check(*js.host);
         if (first) {
             usual = k;
             for (int j : cyc) usual = std::min(usual, ist[j * IS_N + IS_STEPS]);

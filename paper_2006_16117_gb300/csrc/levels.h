@@ -90,6 +90,8 @@ public:
             SIM_CUDA(cudaMallocHost(&h.act, sizeof(int) * J));
             h.J = J;
         }
+        if (!h.err) SIM_CUDA(cudaMallocHost(&h.err, sizeof(int)));
+        *h.err = 0;
         if (!h.act_ev) SIM_CUDA(cudaEventCreateWithFlags(&h.act_ev, cudaEventDisableTiming));
         h.uploaded.clear();
         h.usual_steps = 0;

@@ -40,7 +40,8 @@
 // 1,446 -> 1,159 us (5.0 TB/s) in complex64, 12.4 -> 10.2 ms in complex128 (FP64 pipe).
 //
 // Every wait on an mbarrier has an iteration limit; a thread whose wait runs
-// out records an error and the CTA stops computing and issuing copies, keeps
+// out records an error, which the inner solver throws when it has waited for the
+// stream (block_solve_check), and the CTA stops computing and issuing copies, keeps
 // taking part in its barriers (so no thread waits forever), and waits (again
 // bounded) for its own copies in flight before it exits.
 #include <cooperative_groups.h>
@@ -293,7 +294,7 @@ __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, J
             if (done()) return true;
             if (it > WAIT_LIMIT) {
                 s_fail = 1;
-                atomicExch(err, code);
+                *(volatile int*)err = code;  // pinned host memory
             }
         }
         return false;
@@ -1057,7 +1058,6 @@ Shape choose_shape(const Pencil& P, size_t cs, int ng) {
     return best;
 }
 
-int* g_err = nullptr;
 int* g_grp = nullptr;
 int g_grp_cap = 0;
 // pinned staging for the group table: a pageable upload would synchronise the stream
@@ -1096,10 +1096,6 @@ bool block_solve_cluster(const Pencil& P, int precision, const JobSpace& js, con
     std::vector<int> flat((size_t)ng * R, -1);
     for (int g = 0; g < ng; ++g)
         for (size_t j = 0; j < gs[g].size(); ++j) flat[(size_t)g * R + j] = gs[g][j];
-    if (!g_err) {
-        SIM_CUDA(cudaMalloc(&g_err, sizeof(int)));
-        SIM_CUDA(cudaMemset(g_err, 0, sizeof(int)));
-    }
     Groups table;
     table.far = nullptr;
     if ((int)flat.size() <= Groups::MAX && js.J <= 32767) {
@@ -1152,7 +1148,7 @@ bool block_solve_cluster(const Pencil& P, int precision, const JobSpace& js, con
     kprof_begin("block_solve", st);
     kprof_begin(shape, st);
 #define SIM_LAUNCH_R(CT, RR, MB) \
-    launch_cl<CT, RR, MB>(P, js, in_slot, out_slot, d_factor_ptrs, table, ng, Ccl, pl, g_err, st)
+    launch_cl<CT, RR, MB>(P, js, in_slot, out_slot, d_factor_ptrs, table, ng, Ccl, pl, js.host->err, st)
     if (precision == SIM_FP64) {
         if (pl.R == 8) SIM_LAUNCH_R(double2, 8, 1);
         else if (pl.R == 4) SIM_LAUNCH_R(double2, 4, 1);
@@ -1174,11 +1170,11 @@ bool block_solve_cluster(const Pencil& P, int precision, const JobSpace& js, con
     return true;
 }
 
-int block_solve_error() {
-    if (!g_err) return 0;
-    int e = 0;
-    cudaMemcpy(&e, g_err, sizeof(int), cudaMemcpyDeviceToHost);
-    return e;
+void block_solve_check(JobHost& host) {
+    const int code = host.err ? *(volatile int*)host.err : 0;
+    if (code == 0) return;
+    *host.err = 0;
+    throw CudaError{cudaErrorLaunchTimeout, "block solve: a wait on an mbarrier ran out (code " + std::to_string(code) + ")"};
 }
 
 }  // namespace sim

@@ -15,7 +15,9 @@ bool block_solve_cluster(const Pencil& P, int precision, const JobSpace& js, con
                          int in_slot, int out_slot, const double2* d_sigma, void* const* d_factor_ptrs,
                          cudaStream_t st);
 
-// Nonzero if a cluster solve recorded a failed wait (an mbarrier poll limit).
-int block_solve_error();
+// Throws if a block solve on this job space has recorded a failed wait (an mbarrier
+// poll limit) in host.err, and clears it.  For the host to call once it has waited
+// for the stream: what such a solve left behind is no solution.
+void block_solve_check(JobHost& host);
 
 }  // namespace sim

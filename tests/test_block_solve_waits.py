@@ -27,3 +27,33 @@ def test_every_wait_of_one_lane_is_broadcast_to_its_warp():
         args = text[at + nxt.end(): at + nxt.end() + 60]
         assert re.match(r"\(0xffffffffu, \(int\)%s, 0\)" % name, args), args
         assert "break" not in text[at: at + nxt.start()] and "continue" not in text[at: at + nxt.start()]
+
+
+def test_recorded_wait_error_is_thrown_once(tmp_path):
+    import native_program
+
+    out = native_program.run(tmp_path, r'''
+#include <cstdio>
+#include "solve_cluster.h"
+int main() {
+    int code = 3, thrown = 0;
+    sim::JobHost h;
+    h.err = &code;
+    for (int i = 0; i < 2; ++i) try {
+        sim::block_solve_check(h);
+    } catch (const sim::CudaError& e) {
+        ++thrown;
+        printf("%s\n", e.what.c_str());
+    }
+    h.err = nullptr;
+    printf("%d %d\n", thrown, code);
+}
+''').splitlines()
+    assert out[-1] == "1 0" and "code 3" in out[0], out
+
+
+def test_inner_solve_reads_the_error_wherever_it_waits():
+    s = open(os.path.join(os.path.dirname(SRC), "krylov.cu")).read()
+    body = s[s.index("bool inner_solve(const Pencil& P"): s.index("// Arnoldi with CGS2 for all jobs")]
+    waits = re.findall(r"cudaStreamSynchronize\(st\)\);\s*(\w+)", body)
+    assert waits and set(waits) == {"block_solve_check"}, waits
