@@ -12,6 +12,7 @@
 #include <string>
 #include <vector>
 
+#include "in_place.h"
 #include "internal.h"
 #include "factor_cluster.h"
 #include "levels.h"
@@ -1302,16 +1303,17 @@ sim_status sim_apply_shifted(sim_handle h, double sig_re, double sig_im, const d
     return guarded(h, [&]() -> sim_status {
         if (!x || !y) return fail(h, SIM_ERR_INVALID_ARG, "NULL vector");
         const int64_t n = h->P.n;
-        // The kernel reads and writes the caller's vectors where it can: device memory,
-        // aligned, not overlapping (rows read others' entries of x); copies otherwise.
-        auto direct = [](const void* p) {
+        // The kernel reads and writes the caller's vectors where it can (in_place.h) and
+        // they do not overlap (rows read others' entries of x); copies otherwise.
+        int dev = 0;
+        SIM_CUDA(cudaGetDevice(&dev));
+        auto direct = [dev](const void* p) {
             cudaPointerAttributes at{};
             if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
                 (void)cudaGetLastError();
                 return false;
             }
-            return (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged) &&
-                   (reinterpret_cast<uintptr_t>(p) & 15) == 0;
+            return usable_in_place(at, dev, p);
         };
         const size_t bytes = sizeof(double2) * n;
         const double2* xv = reinterpret_cast<const double2*>(x);
