@@ -52,40 +52,36 @@ __device__ __forceinline__ double2 sub_product(double2 v, double2 a, double2 b) 
 // scratch of m(m+1)/2 entries.  Returns |y_{m-1}| and ||y||^2 (warp-uniform).
 //
 // An FP64 instruction costs a warp 64 clocks however many lanes it serves, so
-// what counts is their number, about 1,500 a solve at m = 50 (5,500 with
-// divisions, alpha's products and the right-hand side on every lane: 4,096
-// squares of 8 nodes took 9.65 ms, now 4.1):
-//  * the system is divided by alpha, (H + τI) y = β τ e1 with τ = 1/alpha, so that
-//    rows are loaded as they stand;
+// what counts is their number, about 1,850 a solve at m = 50 (5,500 with divisions
+// and the right-hand side on every lane):
 //  * the right-hand side is column m of the rows;
 //  * a pivot's reciprocal (crecip) serves the elimination and, kept by the pivot's
 //    lane, the back substitution;
 //  * columns below 32 are done with from row 32 on.
+// The system is not divided by alpha, although H's rows would then serve as they
+// stand (330 instructions fewer): the rounding of 1 / alpha goes into every diagonal
+// entry alike, and the median error of |y_{m-1}| / ||y|| grows 2 to 3 times.
 __device__ __forceinline__ void warp_hess_solve(const double2* Hs, int m, double2 alpha, double beta, double2* U, double2* ys,
                                 double& ylast, double& ynorm2) {
     const int lane = threadIdx.x & 31;
     const int c0 = lane, c1 = lane + 32;
     const double2 zero = make_double2(0.0, 0.0);
-    if (alpha.x == 0.0 && alpha.y == 0.0) {  // the identity
-        for (int c = lane; c < m; c += 32) ys[c] = c == 0 ? make_double2(beta, 0.0) : zero;
-        __syncwarp();
-        ylast = m == 1 ? fabs(beta) : 0.0;
-        ynorm2 = beta * beta;
-        return;
-    }
-    const double2 tau = crecip(alpha);
-    // the diagonal entries of this lane's columns
-    const double2 d0 = c0 < m ? cadd(Hs[c0 * m + c0], tau) : zero, d1 = c1 < m ? cadd(Hs[c1 * m + c1], tau) : zero;
-    auto entry = [&](int r, int c, double2 d) -> double2 { return c == r ? d : (c < m ? Hs[r * m + c] : zero); };
-    double2 a0 = entry(0, c0, d0), a1 = entry(0, c1, d1);
-    if (c0 == m) a0 = cscale(tau, beta);
-    if (c1 == m) a1 = cscale(tau, beta);
+    // entry (r, c) of I + alpha H
+    auto entry = [&](int r, int c) -> double2 {
+        if (c >= m) return zero;
+        const double2 h = Hs[r * m + c];
+        const double one = c == r ? 1.0 : 0.0;
+        return make_double2(fma(alpha.x, h.x, fma(-alpha.y, h.y, one)), fma(alpha.x, h.y, alpha.y * h.x));
+    };
+    double2 a0 = entry(0, c0), a1 = entry(0, c1);
+    if (c0 == m) a0 = make_double2(beta, 0.0);
+    if (c1 == m) a1 = make_double2(beta, 0.0);
     double2 iv0 = zero, iv1 = zero;  // reciprocals of U's diagonal in this lane's columns
     for (int k = 0; k < m; ++k) {
         const bool low = k < 32;  // columns 0..31 still in work
         const bool more = k + 1 < m;
-        double2 b0 = low && more ? entry(k + 1, c0, d0) : zero;
-        double2 b1 = more ? entry(k + 1, c1, d1) : zero;
+        double2 b0 = low && more ? entry(k + 1, c0) : zero;
+        double2 b1 = more ? entry(k + 1, c1) : zero;
         const int src = k & 31;
         double2 ak, bk;
         ak.x = __shfl_sync(0xffffffffu, low ? a0.x : a1.x, src);
