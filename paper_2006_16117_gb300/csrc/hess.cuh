@@ -66,12 +66,13 @@ __device__ __forceinline__ void warp_hess_solve(const double2* Hs, int m, double
     const int lane = threadIdx.x & 31;
     const int c0 = lane, c1 = lane + 32;
     const double2 zero = make_double2(0.0, 0.0);
-    // entry (r, c) of I + alpha H
+    // entry (r, c) of I + alpha H: alpha h rounded before 1 is added, as an FMA onto the
+    // 1 would round its first product to the 1's last place (a fifth more error)
     auto entry = [&](int r, int c) -> double2 {
         if (c >= m) return zero;
-        const double2 h = Hs[r * m + c];
-        const double one = c == r ? 1.0 : 0.0;
-        return make_double2(fma(alpha.x, h.x, fma(-alpha.y, h.y, one)), fma(alpha.x, h.y, alpha.y * h.x));
+        double2 v = cmul(alpha, Hs[r * m + c]);
+        if (c == r) v.x += 1.0;
+        return v;
     };
     double2 a0 = entry(0, c0), a1 = entry(0, c1);
     if (c0 == m) a0 = make_double2(beta, 0.0);
