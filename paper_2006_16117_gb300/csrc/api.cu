@@ -498,7 +498,7 @@ void ensure_adjoint(sim_ctx* h) {
         }
         sa->S.b = make_double2(h->sep->S.b.x, -h->sep->S.b.y);
         sa->ar = &h->arena;
-        separable_setup(sa->S, h->arena, h->st, "sepadj_");
+        separable_setup(sa->S, h->opt.precision, h->arena, h->st, "sepadj_");
         h->sep_adj = std::move(sa);
         h->Padj.sep = h->sep_adj.get();
     }
@@ -1392,7 +1392,7 @@ sim_status sim_set_separable(sim_handle h, int32_t ndim, const int64_t* dims, co
         }
         sep->S.tc = h->opt.separable_tensor_cores != 0;
         sep->ar = &h->arena;
-        separable_setup(sep->S, h->arena, h->st);
+        separable_setup(sep->S, h->opt.precision, h->arena, h->st);
         // the factorisations of an earlier region are no longer used
         for (int s = 0; s < h->cap; ++s) {
             if (h->factors[s]) {

@@ -331,7 +331,8 @@ void apply_t(const Separable& S, const JobSpace& js, int na, int in_slot, int ou
 
 }  // namespace
 
-void separable_setup(Separable& S, DeviceArena& ar, cudaStream_t st, const std::string& prefix) {
+void separable_setup(Separable& S, int precision, DeviceArena& ar, cudaStream_t st, const std::string& prefix) {
+    const bool fused = sep_fused_applies(S, precision);
     for (int d = 0; d < S.ndim; ++d) {
         const int64_t N = S.dims[d];
         const std::string tag = prefix + "ax" + std::to_string(d) + "_";
@@ -346,9 +347,12 @@ void separable_setup(Separable& S, DeviceArena& ar, cudaStream_t st, const std::
                                                          S.Q32[d], S.rho[d], S.irho[d], S.lam[d]);
         SIM_LAUNCH_CHECK();
         sep_split_tables(S.Q64[d], (int)N, S.Qh[d], S.Ql[d], st);
-        const int64_t Np = (N + 3) / 4 * 4;
-        S.Qp[d] = ar.get<float>(tag + "Qp", Np * Np);
-        sep_pad_table(S.Q32[d], (int)N, S.Qp[d], st);
+        S.Qp[d] = nullptr;
+        if (fused) {
+            const int64_t Np = (N + 3) / 4 * 4;
+            S.Qp[d] = ar.get<float>(tag + "Qp", Np * Np);
+            sep_pad_table(S.Q32[d], (int)N, S.Qp[d], st);
+        }
     }
     int64_t n = 1;
     for (int d = 0; d < S.ndim; ++d) n *= S.dims[d];
@@ -359,6 +363,8 @@ void separable_setup(Separable& S, DeviceArena& ar, cudaStream_t st, const std::
                                                       S.sin32, S.sout32, S.lsum);
     SIM_LAUNCH_CHECK();
     SIM_CUDA(cudaStreamSynchronize(st));
+    if (!fused)  // an earlier separable part's
+        for (int d = 0; d < 3; ++d) ar.release(prefix + "ax" + std::to_string(d) + "_Qp");
 }
 
 void separable_apply(const Separable& S, int precision, const JobSpace& js, const std::vector<int>& active,
@@ -367,9 +373,10 @@ void separable_apply(const Separable& S, int precision, const JobSpace& js, cons
     if (na <= 0) return;
     // the active list is already on the device (js.d_active) in this order
     kprof_begin("separable", st);
-    if (precision != SIM_FP64 && S.tc && sep_fused_2d(S, js, na, in_slot, out_slot, d_sigma, st)) {
-    } else if (precision == SIM_FP64) apply_t<double, double>(S, js, na, in_slot, out_slot, d_sigma, ar, st);
-    else apply_t<float, float>(S, js, na, in_slot, out_slot, d_sigma, ar, st);
+    if (precision == SIM_FP64)
+        apply_t<double, double>(S, js, na, in_slot, out_slot, d_sigma, ar, st);
+    else if (!S.Qp[0] || !sep_fused_2d(S, js, na, in_slot, out_slot, d_sigma, st))
+        apply_t<float, float>(S, js, na, in_slot, out_slot, d_sigma, ar, st);
     double flops = 0.0;
     for (int d = 0; d < S.ndim; ++d) flops += 2.0 * 4.0 * (double)js.n * (double)S.dims[d];  // 2 passes, 2 FMA
     const double cw = precision == SIM_FP64 ? 16.0 : 8.0;

@@ -35,7 +35,7 @@ struct Separable {
     float* Qh[3] = {nullptr, nullptr, nullptr};
     float* Ql[3] = {nullptr, nullptr, nullptr};
     // Q in FP32 for the fused kernel: rows and columns padded with zeros to a
-    // multiple of 4 (separable_fused.cu)
+    // multiple of 4 (separable_fused.cu); only where sep_fused_applies
     float* Qp[3] = {nullptr, nullptr, nullptr};
     bool tc = false;  // complex64 mode products on the tensor cores (separable_tc.cu)
     // per element, for the complex64 path: Π_d ρ_d^{-j_d} and Π_d ρ_d^{j_d} rounded
@@ -52,7 +52,7 @@ struct SepCtx {
 };
 
 // Builds the per-axis tables on the device (arena buffers tag + "ax*").
-void separable_setup(Separable& S, DeviceArena& ar, cudaStream_t st, const std::string& tag = "sep_");
+void separable_setup(Separable& S, int precision, DeviceArena& ar, cudaStream_t st, const std::string& tag = "sep_");
 
 // One mode product of na complex64 vectors on the tensor cores (3xTF32),
 // Y = X ×_axis Q for an axis of length N with inner stride P (separable_tc.cu).
@@ -60,7 +60,9 @@ bool sep_mode_tc(const float2* cur, float2* nxt, const float* Qhi, const float* 
                  int64_t n, int na, cudaStream_t st);
 // The whole apply of a two-dimensional separable part in one kernel, a cluster per
 // job with its vector in shared memory (separable_fused.cu); false (nothing
-// launched) where the vector does not fit or the separate kernels are faster.
+// launched) where the separate kernels are faster.  Only where sep_fused_applies:
+// complex64, two axes, a vector that some cluster holds.
+bool sep_fused_applies(const Separable& S, int precision);
 bool sep_fused_2d(const Separable& S, const JobSpace& js, int na, int in_slot, int out_slot, const double2* d_sigma,
                   cudaStream_t st);
 void sep_pad_table(const float* Q32, int N, float* Qp, cudaStream_t st);

@@ -340,9 +340,13 @@ void sep_pad_table(const float* Q32, int N, float* Qp, cudaStream_t st) {
     SIM_LAUNCH_CHECK();
 }
 
+bool sep_fused_applies(const Separable& S, int precision) {
+    return precision != SIM_FP64 && S.tc && S.ndim == 2 && S.dims[0] <= 2048 && S.dims[1] <= 2048 &&
+           fused_shape((int)S.dims[0], (int)S.dims[1], 1).C > 0;
+}
+
 bool sep_fused_2d(const Separable& S, const JobSpace& js, int na, int in_slot, int out_slot, const double2* d_sigma,
                   cudaStream_t st) {
-    if (S.ndim != 2 || S.dims[0] > 2048 || S.dims[1] > 2048) return false;
     const FusedShape f = fused_shape((int)S.dims[0], (int)S.dims[1], na);
     if (f.C == 0 || f.cost > separate_cost((int)S.dims[0], (int)S.dims[1], na)) return false;
     switch (f.tile) {
