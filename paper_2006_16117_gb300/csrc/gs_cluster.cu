@@ -22,13 +22,10 @@
 // step's own kernel (7 us) and a copy of w included.
 #include <cooperative_groups.h>
 
-#include <algorithm>
-#include <atomic>
-#include <cmath>
-#include <limits>
-
+#include "cluster_fit.h"
 #include "gs.h"
 #include "gs_finish.cuh"
+#include "gs_shape.h"
 
 namespace cg = cooperative_groups;
 
@@ -38,8 +35,6 @@ namespace {
 
 constexpr int GC_MAXT = 256;
 constexpr int GC_WARPS = GC_MAXT / 32;
-constexpr int GC_MAXV = 64;   // basis vectors per call (cnt)
-constexpr int GC_MAXE = 20;   // rows per thread: two CTAs' pieces of w fit an SM
 
 struct GcShared {
     double red[GC_WARPS][2 * GC_MAXV + 4];  // per-warp sums, (re, im) per value
@@ -187,28 +182,11 @@ __global__ void __launch_bounds__(GC_MAXT, 2) k_gs_cluster(GSArgs a, int E) {
     cl.sync();  // no CTA leaves while a peer reads its sums
 }
 
-struct ClusterShape {
-    int Cg = 0, E = 0, NT = 256;
-    double cost = std::numeric_limits<double>::infinity();
-};
-
-// Cluster size and rows per thread: as many CTAs a job as the GPU holds at two per
-// SM, at most 16 (the hardware's limit) and no more than there are rows for.  The
-// estimate charges each SM's FP64 instructions 64 clocks a warp on its four
-// schedulers and 2,500 clocks a pass for the sums across the cluster.
-ClusterShape cluster_shape(int64_t n, int cnt, int passes, int nactive) {
-    ClusterShape s;
-    s.NT = n <= 128 * 16 ? 128 : 256;
-    const int need = cdiv_up(n, (int64_t)s.NT * GC_MAXE);
-    if (need > 16 || cnt > GC_MAXV) return s;
-    const int room = std::max(1, 2 * 152 / std::max(1, nactive));
-    s.Cg = std::max(need, std::min(std::min(16, room), cdiv_up(n, s.NT)));
-    s.E = cdiv_up(n, (int64_t)s.NT * s.Cg);
-    s.Cg = cdiv_up(n, (int64_t)s.NT * s.E);
-    const double per_warp = s.E * (4.0 * cnt * passes + 6.0) + 1.2 * cnt * passes + 20.0;
-    const double per_sm = std::ceil((double)nactive * s.Cg / 152.0);
-    s.cost = per_warp * 64.0 * (s.NT / 128) * per_sm + (passes + 1.0) * 2500.0;
-    return s;
+// The shape of a launch that this device can place (E = 0: none).
+GsShape cluster_shape(int64_t n, int cnt, int passes, int nactive) {
+    return gs_cluster_shape(n, cnt, passes, nactive, sm_count(), [](int C, int threads, size_t smem) {
+        return clusters_that_fit((const void*)k_gs_cluster, C, threads, smem) > 0;
+    });
 }
 
 }  // namespace
@@ -219,11 +197,11 @@ double gs_cluster_cost(int64_t n, int cnt, int passes, int nactive) {
 
 void gs_cluster(const GSArgs& a, int nactive, cudaStream_t st) {
     const int passes = a.cnt == 0 ? 0 : (a.dgks || a.single ? 2 : 4);
-    const ClusterShape s = cluster_shape(a.n, a.cnt, passes, nactive);
+    const GsShape s = cluster_shape(a.n, a.cnt, passes, nactive);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nactive * s.Cg);
     cfg.blockDim = dim3(s.NT);
-    cfg.dynamicSmemBytes = (size_t)s.E * s.NT * sizeof(double2);
+    cfg.dynamicSmemBytes = s.smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -232,15 +210,6 @@ void gs_cluster(const GSArgs& a, int nactive, cudaStream_t st) {
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    static std::atomic<uint64_t> ready{0};  // devices whose kernel attributes are set
-    int dev = 0;
-    SIM_CUDA(cudaGetDevice(&dev));
-    if (dev > 63 || !(ready.load() >> dev & 1)) {
-        SIM_CUDA(cudaFuncSetAttribute(k_gs_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      GC_MAXE * GC_MAXT * (int)sizeof(double2)));
-        SIM_CUDA(cudaFuncSetAttribute(k_gs_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        if (dev <= 63) ready.fetch_or(1ull << dev);
-    }
     SIM_CUDA(cudaLaunchKernelEx(&cfg, k_gs_cluster, a, s.E));
     SIM_LAUNCH_CHECK();
 }

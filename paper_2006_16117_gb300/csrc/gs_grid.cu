@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "cluster_fit.h"
 #include "gs.h"
 #include "gs_finish.cuh"
 
@@ -226,7 +227,7 @@ __global__ void __launch_bounds__(GG_T) k_gsg_scale(GSArgs a, int from_src) {
 // an SM, 16 rows a thread at most.
 int rows_per_thread(int64_t n, int nactive) {
     int per = 1;
-    while (per < 16 && (int64_t)nactive * cdiv_up(n, (int64_t)GG_T * per) > 2 * 152) per *= 2;
+    while (per < 16 && (int64_t)nactive * cdiv_up(n, (int64_t)GG_T * per) > 2 * sm_count()) per *= 2;
     return per;
 }
 
@@ -270,7 +271,7 @@ double gs_grid_cost(int64_t n, int cnt, int passes, int nactive) {
     const double ctas = (double)nactive * cdiv_up(n, (int64_t)GG_T * per);
     const double per_warp = per * (4.0 * cnt * passes + 6.0) + 1.2 * cnt * passes + 20.0;
     const double launches = cnt == 0 ? 2.0 : (passes == 4 ? 4.0 : 3.5);
-    return per_warp * 64.0 * 2.0 * std::ceil(ctas / 152.0) + launches * 6000.0;
+    return per_warp * 64.0 * 2.0 * std::ceil(ctas / sm_count()) + launches * 6000.0;
 }
 
 int64_t gs_grid_partials(int64_t n, int J, int pw) {

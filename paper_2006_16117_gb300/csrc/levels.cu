@@ -15,6 +15,7 @@
 // indicator's two quadrature sums are reduced inside the CTA.
 #include <cmath>
 
+#include "cluster_fit.h"
 #include "internal.h"
 #include "levels.h"
 #include "hess.cuh"
@@ -254,7 +255,7 @@ void eval_explicit(const double2* H, int m, int meff, double beta, double2 sigma
     if (count <= 0) return;
     const size_t sm = eval_smem_bytes(m);
     SIM_CUDA(cudaFuncSetAttribute(k_eval_explicit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-    int grid = (int)std::min<int64_t>(count, 152);  // one CTA fits an SM: H staged once for all its squares
+    int grid = (int)std::min<int64_t>(count, sm_count());  // one CTA an SM (at m = 50 no more fit): H staged once
     k_eval_explicit<<<grid, 256, sm, stream>>>(H, m, meff, beta, sigma, centers, sides, count, scale, ind, rho);
     SIM_LAUNCH_CHECK();
 }

@@ -18,13 +18,14 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 
+#include "cluster_fit.h"
 #include "fp64.cuh"
 #include "internal.h"
 #include "levels.h"
 #include "separable.h"
+#include "separable_fused_shape.h"
 
 namespace cg = cooperative_groups;
 
@@ -32,19 +33,12 @@ namespace sim {
 
 namespace {
 
-constexpr int SF_T = 256;
-
-__host__ __device__ constexpr int pad4(int n) { return (n + 3) / 4 * 4; }
+__device__ __forceinline__ int pad4(int n) { return sf_pad4(n); }
 
 __device__ __forceinline__ void copy_async_16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
                  : "memory");
 }
-
-constexpr int SF_STAGES = 3;
-// rows of Q per stage: three stages within 48 KB
-__host__ __device__ constexpr int stage_rows(int ldq) { return ldq <= 256 ? 16 : (ldq <= 512 ? 8 : 4); }
-__host__ __device__ constexpr size_t stage_floats(int N) { return (size_t)stage_rows(pad4(N)) * pad4(N); }
 
 // f.put(f.column(k), r, Σ_j X[r][j] Q[j][k]) for r < rows, k < N.  X: [rows][ldx] in
 // shared memory, zero from column N to ldx = pad4(N); Q: pad4(N) x pad4(N), zero
@@ -56,7 +50,7 @@ __device__ __forceinline__ void rows_times_q(const float2* X, int ldx, int rows,
                                              float* stage, const F& f) {
     constexpr int K4 = KT / 4;
     const int ldq = pad4(N), nk = (ldq + KT - 1) / KT, nr = (rows + RT - 1) / RT, items = nk * nr;
-    const int KC = stage_rows(ldq), nc = (ldq + KC - 1) / KC, per_stage = KC * ldq;
+    const int KC = sf_stage_rows(ldq), nc = (ldq + KC - 1) / KC, per_stage = KC * ldq;
     auto fill = [&](int c) {
         if (c < nc) {
             float* dst = stage + (size_t)(c % SF_STAGES) * per_stage;
@@ -240,53 +234,6 @@ __global__ void k_sep_pad(const float* Q32, int N, int Np, float* Qp) {
     Qp[t] = r < N && c < N ? Q32[(size_t)r * N + c] : 0.f;
 }
 
-// (rows, columns) a thread forms at a time, from few to many
-constexpr int kTiles[3][2] = {{1, 4}, {2, 4}, {4, 4}};
-
-struct FusedShape {
-    int C = 0, Rc = 0, Cc = 0, tile = 2;
-    size_t smem = 0;
-    double cost = 1e300;
-};
-
-// Cluster size and tile by an estimate of the clocks of an apply.  A product takes,
-// per two reduction steps and round of 256 threads, 1.5 times its loads' way into
-// the registers (a 16-byte load of a warp takes 4 clocks), at least 200 clocks, and
-// a round's results 100 clocks a value (measured on 30 to 250 points a side: 40,000
-// clocks at 60 points with four CTAs and 1 x 4, 185,000 at 250 with 16 and 4 x 4,
-// where 2 x 4 takes 260,000 and 4 x 8, on half the threads, 220,000).
-FusedShape fused_shape(int N0, int N1, int na) {
-    FusedShape best;
-    for (int C = 1; C <= 16; ++C) {
-        FusedShape f;
-        f.Rc = (N1 + C - 1) / C;
-        f.Cc = (N0 + C - 1) / C;
-        if (C > 1 && ((C - 1) * f.Rc >= N1 || (C - 1) * f.Cc >= N0)) continue;  // a CTA without lines
-        f.C = C;
-        f.smem = 2 * sizeof(float2) * (size_t)std::max(f.Rc * pad4(N0), f.Cc * pad4(N1)) +
-                 SF_STAGES * sizeof(float) * std::max(stage_floats(N0), stage_floats(N1));
-        if (f.smem > 220 * 1024) continue;
-        const double per_sm = std::ceil((double)na * C / 152.0);  // CTAs that share an SM, in turn or at once
-        for (int t = 0; t < 3; ++t) {
-            const int RT = kTiles[t][0], KT = kTiles[t][1];
-            auto product = [&](int rows, int N) {
-                const int items = (N + KT - 1) / KT * ((rows + RT - 1) / RT);
-                const double rounds = std::ceil((double)items / SF_T);
-                const double warps = std::min<double>(SF_T / 32, std::ceil(items / 32.0));
-                const double lsu = warps * (RT + KT / 2.0) * 4.0;
-                return rounds * (N / 2.0 * std::max(200.0, 1.5 * lsu) + 100.0 * warps * RT * KT / 2.0);
-            };
-            const double cost = per_sm * (2.0 * product(f.Rc, N0) + 2.0 * product(f.Cc, N1)) + (C > 1 ? 9000.0 : 4000.0);
-            if (cost < best.cost) {
-                best = f;
-                best.tile = t;
-                best.cost = cost;
-            }
-        }
-    }
-    return best;
-}
-
 // The same for the separate kernels: a product's CTAs (128 rows of real and
 // imaginary parts each, two to an SM) take 6,000 clocks and 35 per output column for
 // each 32 reduction indices, the elementwise passes 8,000 and their traffic, a
@@ -297,7 +244,7 @@ double separate_cost(int N0, int N1, int na) {
     auto product = [&](int N, int rows) {
         const int NT = std::min(256, (N + 15) / 16 * 16);
         const double ctas = std::ceil(2.0 * rows / 128.0) * std::ceil((double)N / NT) * na;
-        return std::ceil(ctas / 304.0) * std::ceil(N / 32.0) * (6000.0 + 35.0 * NT);
+        return std::ceil(ctas / (2.0 * sm_count())) * std::ceil(N / 32.0) * (6000.0 + 35.0 * NT);
     };
     return 2.0 * product(N0, N1) + 2.0 * product(N1, N0) + 3.0 * (8000.0 + n * na * 48.0 / 3300.0) + 7.0 * 2000.0;
 }
@@ -305,15 +252,7 @@ double separate_cost(int N0, int N1, int na) {
 template <int RT, int KT>
 void launch_fused(const Separable& S, const JobSpace& js, int na, int in_slot, int out_slot, const double2* d_sigma,
                   const FusedShape& f, cudaStream_t st) {
-    static std::atomic<uint64_t> ready{0};  // devices whose kernel attributes are set
     auto kern = k_sep_fused<RT, KT>;
-    int dev = 0;
-    SIM_CUDA(cudaGetDevice(&dev));
-    if (dev > 63 || !(ready.load() >> dev & 1)) {
-        SIM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-        SIM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-        if (dev <= 63) ready.fetch_or(1ull << dev);
-    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(na * f.C);
     cfg.blockDim = dim3(SF_T);
@@ -332,22 +271,30 @@ void launch_fused(const Separable& S, const JobSpace& js, int na, int in_slot, i
     SIM_LAUNCH_CHECK();
 }
 
+FusedShape shape_on_device(const Separable& S, int na) {
+    return fused_shape_that_fits((int)S.dims[0], (int)S.dims[1], na, sm_count(), [](const FusedShape& f) {
+        const void* kern = f.tile == 0 ? (const void*)k_sep_fused<1, 4>
+                                       : (f.tile == 1 ? (const void*)k_sep_fused<2, 4> : (const void*)k_sep_fused<4, 4>);
+        return clusters_that_fit(kern, f.C, SF_T, f.smem) > 0;
+    });
+}
+
 }  // namespace
 
 void sep_pad_table(const float* Q32, int N, float* Qp, cudaStream_t st) {
-    const int Np = pad4(N);
+    const int Np = sf_pad4(N);
     k_sep_pad<<<cdiv_up((int64_t)Np * Np, 256), 256, 0, st>>>(Q32, N, Np, Qp);
     SIM_LAUNCH_CHECK();
 }
 
 bool sep_fused_applies(const Separable& S, int precision) {
     return precision != SIM_FP64 && S.tc && S.ndim == 2 && S.dims[0] <= 2048 && S.dims[1] <= 2048 &&
-           fused_shape((int)S.dims[0], (int)S.dims[1], 1).C > 0;
+           shape_on_device(S, 1).C > 0;
 }
 
 bool sep_fused_2d(const Separable& S, const JobSpace& js, int na, int in_slot, int out_slot, const double2* d_sigma,
                   cudaStream_t st) {
-    const FusedShape f = fused_shape((int)S.dims[0], (int)S.dims[1], na);
+    const FusedShape f = shape_on_device(S, na);
     if (f.C == 0 || f.cost > separate_cost((int)S.dims[0], (int)S.dims[1], na)) return false;
     switch (f.tile) {
         case 0: launch_fused<1, 4>(S, js, na, in_slot, out_slot, d_sigma, f, st); break;
