@@ -52,8 +52,7 @@ struct GSArgs {
     int single = 0;
     GmArgs gm;
     // scratch of the grid kernels (gs_grid.cu)
-    double2* part = nullptr;  // partial sums: part_cap per half
-    int64_t part_cap = 0;
+    double2* part = nullptr;  // partial sums: gs_grid_partials()
     int pw = 0;               // values per chunk
     double2* hsum = nullptr;  // [2][J][pw] totals of the two passes
     double* fin = nullptr;    // [J] scale of the result

@@ -214,8 +214,10 @@ void gs_cluster(const GSArgs& a, int nactive, cudaStream_t st) {
     SIM_LAUNCH_CHECK();
 }
 
-void gram_schmidt(const GSArgs& a, int nactive, cudaStream_t st) {
+void gram_schmidt(const GSArgs& args, int nactive, cudaStream_t st) {
     if (nactive <= 0) return;
+    GSArgs a = args;
+    if (a.single) a.dgks = 0;  // for either form
     const int passes = a.cnt == 0 ? 0 : (a.dgks || a.single ? 2 : 4);
     // algorithmic bytes: w read and written once; the basis streamed once per
     // pass (two passes with the selective test in its usual outcome, four for CGS2)
