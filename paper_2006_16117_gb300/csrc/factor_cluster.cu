@@ -70,17 +70,6 @@ __device__ __forceinline__ double2 sval(const Pencil& P, int64_t e, double2 sg) 
 // pivot magnitude |re| + |im| in the factor's own precision
 template <class C> __device__ __forceinline__ auto m1(C a) -> decltype(a.x) { return fabs(a.x) + fabs(a.y); }
 
-// 1 / a, scaled by a power of two so that |a|^2 neither overflows nor underflows
-__device__ __forceinline__ float2 crecip(float2 a) {
-    const float m = fmaxf(fabsf(a.x), fabsf(a.y));
-    const int e = (int)((__float_as_uint(m) >> 23) & 255u);
-    const float s = __uint_as_float((uint32_t)min(max(254 - e, 1), 253) << 23);  // about 1/m
-    const float x = a.x * s, y = a.y * s;  // the larger in [1, 2) but for the ends of the range
-    const float d = fmaf(x, x, y * y);
-    float r = __fdividef(1.0f, d);
-    r = fmaf(r, fmaf(-d, r, 1.0f), r) * s;  // one Newton step
-    return make_float2(x * r, -y * r);
-}
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 __device__ __forceinline__ void bar_panel(int threads) {

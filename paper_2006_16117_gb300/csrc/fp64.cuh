@@ -1,7 +1,9 @@
-// FP64 scalar helpers with few FP64 operations: a warp's FP64 instruction takes 64
+// Scalar helpers with few FP64 operations: a warp's FP64 instruction takes 64
 // clocks of its scheduler on this GPU however few lanes are active, so scalings by
-// powers of two are exponent arithmetic and roots and reciprocals are one
-// third-order Newton step from an FP32 seed.
+// powers of two are exponent arithmetic, and roots and reciprocals are one step of
+// Householder's third-order iteration (A. S. Householder, The Numerical Treatment of
+// a Single Nonlinear Equation, 1970) from an FP32 seed: with the seed's residual t,
+// the series of (1 - t)^(-1/2) or (1 - t)^(-1) through t^2.
 #pragma once
 
 #include "common.cuh"
@@ -56,6 +58,7 @@ __device__ __forceinline__ double scale2(double v, int k) {
 __device__ __forceinline__ double2 crecip(double2 a) {
     const int e = max((__double2hiint(a.x) >> 20) & 2047, (__double2hiint(a.y) >> 20) & 2047);
     if (e < 64 || e > 1983) {  // far out: by division
+        if (isinf(a.x) || isinf(a.y)) return make_double2(0.0, 0.0);
         const double s = e < 64 ? 0x1p+960 : 0x1p-960;
         const double x = a.x * s, y = a.y * s, d = x * x + y * y;
         return make_double2(x / d * s, -(y / d) * s);
@@ -70,6 +73,19 @@ __device__ __forceinline__ double2 crecip(double2 a) {
     const double t = fma(-d, r0, 1.0);
     const double r = fma(r0, fma(t, t, t), r0);
     return make_double2(scale2(x * r, k), scale2(-(y * r), k));
+}
+
+// The same in FP32: a division's seed and one Newton step.  The power of two goes
+// onto the products, not onto the reciprocal, which it could overflow.
+__device__ __forceinline__ float2 crecip(float2 a) {
+    const float m = fmaxf(fabsf(a.x), fabsf(a.y));
+    const int e = (int)((__float_as_uint(m) >> 23) & 255u);
+    const float s = __uint_as_float((uint32_t)min(max(254 - e, 1), 253) << 23);  // about 1/m
+    const float x = a.x * s, y = a.y * s;  // the larger in [1, 2) but for the ends of the range
+    const float d = fmaf(x, x, y * y);
+    float r = __fdividef(1.0f, d);
+    r = fmaf(r, fmaf(-d, r, 1.0f), r);  // one Newton step
+    return make_float2(x * r * s, -(y * r) * s);
 }
 
 }  // namespace sim
