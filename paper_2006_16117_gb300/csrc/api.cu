@@ -43,6 +43,7 @@ std::string g_create_error;
 
 struct sim_ctx {
     cudaStream_t st = nullptr;
+    int device = 0;  // the device the handle was created on
     sim_options opt{};
     std::string err;
     int state = ST_CREATED;
@@ -797,6 +798,7 @@ sim_status sim_create(const sim_csr* A, const sim_csr* B, const sim_options* opt
             }
             rp[i + 1] = (int32_t)ci.size();
         }
+        SIM_CUDA(cudaGetDevice(&h->device));
         Pencil& P = h->P;
         upload_pencil(h->arena, h->st, P, rp, ci, Ka, Kb, hasB ? (bdiag ? 1 : 2) : 0, bd, "P_");
         const int T = P.T, nb = P.nb;
@@ -1305,9 +1307,7 @@ sim_status sim_apply_shifted(sim_handle h, double sig_re, double sig_im, const d
         const int64_t n = h->P.n;
         // The kernel reads and writes the caller's vectors where it can (in_place.h) and
         // they do not overlap (rows read others' entries of x); copies otherwise.
-        int dev = 0;
-        SIM_CUDA(cudaGetDevice(&dev));
-        auto direct = [dev](const void* p) {
+        auto direct = [dev = h->device](const void* p) {
             cudaPointerAttributes at{};
             if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
                 (void)cudaGetLastError();
