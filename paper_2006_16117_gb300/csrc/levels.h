@@ -132,7 +132,7 @@ struct MergeResult {
     int* rank = nullptr;  // output position, -1 if outside R
 };
 
-// Schur forms of shifts s0 .. s0+count-1 (one warp each).
+// Schur forms of shifts s0 .. s0+count-1 (a CTA each).
 void schur_shifts(const double2* H, int m, const int* meff, const double* beta, int s0, int count, double2* T,
                   double2* C, double2* Q, int* ok, cudaStream_t st);
 // Mode-0 evaluation of every square against its own shift through the Schur

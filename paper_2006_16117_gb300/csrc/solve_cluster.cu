@@ -33,8 +33,8 @@
 // instruction buffer each costs about five clocks.  Hence a kernel per phase and
 // per "one chunk a step" (ONE), the inputs brought by the producers, one barrier a
 // step, the vector stored to memory a step later by warps that wait anyway, and row
-// layouts that are powers of two.  Launch 1 starts under launch 0 and fills its stages
-// (5 us a solve).  Two sides, T = 200 complex64: 378 -> 263 us (a step 3,800 -> 2,900
+// layouts that are powers of two.  Launch 1 starts under launch 0 and fills its first
+// stage (5 us a solve).  Two sides, T = 200 complex64: 378 -> 263 us (a step 3,800 -> 2,900
 // clocks forward, 3,100 -> 2,300 backward); T = 102 197 -> 123; eight right-hand sides at
 // T = 102 196 -> 138 us a launch; complex128 T = 30 106 -> 53, T = 98 335 -> 195.  With 56 shifts at T = 200 the matrices bound it:
 // 1,446 -> 1,159 us (5.0 TB/s) in complex64, 12.4 -> 10.2 ms in complex128 (FP64 pipe).
@@ -151,9 +151,6 @@ template <> struct Vec16<double2> {
     static constexpr int N = 1;
     __device__ static __forceinline__ double2 get(const double2& v, int) { return v; }
 };
-
-// two CTAs per SM for single right-hand sides in complex64 (see choose_shape)
-constexpr bool kTwoPerSm = true;
 
 constexpr int PF_T = 256;                         // largest T whose step inputs are fetched ahead
 constexpr int RW = 9;                             // a row's partial sums, padded off the banks
@@ -279,7 +276,7 @@ __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, J
     if (tid == 0)
         for (int i = 0; i < 3 && i <= nsteps - 2; ++i) mbar_expect_tx(&vbar[i], vec_bytes);  // steps 0, 1, 2
     cl.sync();  // every CTA of the cluster is running, barriers initialised and armed, before any remote store
-    // Launch 1 starts while launch 0 runs (where SMs are free) and fills its stages; it
+    // Launch 1 starts while launch 0 runs (where SMs are free) and fills its first stage; it
     // waits for launch 0's end before it reads or writes a vector.  The factors are older
     // than launch 0, which starts after everything before it has ended.
     if (phase == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -1029,7 +1026,7 @@ Shape choose_shape(const Pencil& P, size_t cs, int ng) {
     double best_cost = 1e300;
     const int cmax = std::min(16, P.T);
     for (int minb = 1; minb <= 2; ++minb) {
-        if (minb == 2 && !(kTwoPerSm && R == 1 && sizeof(C) == 8)) continue;
+        if (minb == 2 && !(R == 1 && sizeof(C) == 8)) continue;
         for (int c = 1; c <= cmax; ++c) {
             Plan q;
             if (!make_plan(P.T, cs, R, cdiv_up(P.T, c), q, minb == 2 ? 110 * 1024 : 220 * 1024)) continue;
