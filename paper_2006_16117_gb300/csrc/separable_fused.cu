@@ -296,11 +296,14 @@ bool sep_fused_2d(const Separable& S, const JobSpace& js, int na, int in_slot, i
                   cudaStream_t st) {
     const FusedShape f = shape_on_device(S, na);
     if (f.C == 0 || f.cost > separate_cost((int)S.dims[0], (int)S.dims[1], na)) return false;
+    kprof_begin("sep_fused", st);  // instrumentation: a part of "separable"
     switch (f.tile) {
         case 0: launch_fused<1, 4>(S, js, na, in_slot, out_slot, d_sigma, f, st); break;
         case 1: launch_fused<2, 4>(S, js, na, in_slot, out_slot, d_sigma, f, st); break;
         default: launch_fused<4, 4>(S, js, na, in_slot, out_slot, d_sigma, f, st); break;
     }
+    kprof_end("sep_fused", st, na * 32.0 * (double)js.n,
+              na * 8.0 * (double)js.n * (double)(S.dims[0] + S.dims[1]));
     return true;
 }
 
