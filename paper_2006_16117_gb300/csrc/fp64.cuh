@@ -53,16 +53,20 @@ __device__ __forceinline__ double scale2(double v, int k) {
     return e > 0 && e + k > 0 ? __hiloint2double((int)(h + ((uint32_t)k << 20)), __double2loint(v)) : 0.0;
 }
 
+// 1 / a far out of the middle of the range, e its exponent: by division.  A function of
+// its own, so that its rare code does not lie in the pivot chains' loops.
+static __device__ __noinline__ double2 crecip_far(double2 a, int e) {
+    if (isinf(a.x) || isinf(a.y)) return make_double2(0.0, 0.0);
+    const double s = e < 64 ? 0x1p+960 : 0x1p-960;
+    const double x = a.x * s, y = a.y * s, d = x * x + y * y;
+    return make_double2(x / d * s, -(y / d) * s);
+}
+
 // 1 / a (seven FP64 operations): 1/d, d = |a 2^k|^2 in [1, 8), is r + r (e + e^2) with
 // e = 1 - d r from an FP32 reciprocal r (2 ulp: e^3 < 2^-60).
 __device__ __forceinline__ double2 crecip(double2 a) {
     const int e = max((__double2hiint(a.x) >> 20) & 2047, (__double2hiint(a.y) >> 20) & 2047);
-    if (e < 64 || e > 1983) {  // far out: by division
-        if (isinf(a.x) || isinf(a.y)) return make_double2(0.0, 0.0);
-        const double s = e < 64 ? 0x1p+960 : 0x1p-960;
-        const double x = a.x * s, y = a.y * s, d = x * x + y * y;
-        return make_double2(x / d * s, -(y / d) * s);
-    }
+    if (e < 64 || e > 1983) return crecip_far(a, e);
     const int k = 1023 - e;  // a 2^k has its larger part in [1, 2)
     const double x = scale2(a.x, k), y = scale2(a.y, k);
     const double d = fma(x, x, y * y);  // [1, 8)
@@ -76,7 +80,7 @@ __device__ __forceinline__ double2 crecip(double2 a) {
 }
 
 // The same in FP32: a division's seed and one Newton step.  The power of two goes
-// onto the products, not onto the reciprocal, which it could overflow.
+// onto the components, not onto the real reciprocal, which it could overflow.
 __device__ __forceinline__ float2 crecip(float2 a) {
     const float m = fmaxf(fabsf(a.x), fabsf(a.y));
     const int e = (int)((__float_as_uint(m) >> 23) & 255u);
@@ -85,7 +89,7 @@ __device__ __forceinline__ float2 crecip(float2 a) {
     const float d = fmaf(x, x, y * y);
     float r = __fdividef(1.0f, d);
     r = fmaf(r, fmaf(-d, r, 1.0f), r);  // one Newton step
-    return make_float2(x * r * s, -(y * r) * s);
+    return make_float2((x * s) * r, -((y * s) * r));
 }
 
 }  // namespace sim
