@@ -65,10 +65,9 @@ struct GSArgs {
 // breakdown test, normalisation, FGMRES step.  Picks one of the two forms below.
 void gram_schmidt(const GSArgs& a, int nactive, cudaStream_t st);
 
-// Estimated clocks of the two forms, and their launches.
+// Estimated clocks of the two forms, and the second one's launches.
 double gs_cluster_cost(int64_t n, int cnt, int passes, int nactive);  // infinite: out of its range
 double gs_grid_cost(int64_t n, int cnt, int passes, int nactive);
-void gs_cluster(const GSArgs& a, int nactive, cudaStream_t st);
 void gs_grid(const GSArgs& a, int nactive, cudaStream_t st);
 // Rows per CTA of the grid form and the partial sums it needs for any number of
 // active jobs up to J.

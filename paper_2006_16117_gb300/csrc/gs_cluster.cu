@@ -189,15 +189,7 @@ GsShape cluster_shape(int64_t n, int cnt, int passes, int nactive) {
     });
 }
 
-}  // namespace
-
-double gs_cluster_cost(int64_t n, int cnt, int passes, int nactive) {
-    return cluster_shape(n, cnt, passes, nactive).cost;
-}
-
-void gs_cluster(const GSArgs& a, int nactive, cudaStream_t st) {
-    const int passes = a.cnt == 0 ? 0 : (a.dgks || a.single ? 2 : 4);
-    const GsShape s = cluster_shape(a.n, a.cnt, passes, nactive);
+void launch_cluster(const GSArgs& a, int nactive, const GsShape& s, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nactive * s.Cg);
     cfg.blockDim = dim3(s.NT);
@@ -214,6 +206,12 @@ void gs_cluster(const GSArgs& a, int nactive, cudaStream_t st) {
     SIM_LAUNCH_CHECK();
 }
 
+}  // namespace
+
+double gs_cluster_cost(int64_t n, int cnt, int passes, int nactive) {
+    return cluster_shape(n, cnt, passes, nactive).cost;
+}
+
 void gram_schmidt(const GSArgs& args, int nactive, cudaStream_t st) {
     if (nactive <= 0) return;
     GSArgs a = args;
@@ -222,8 +220,9 @@ void gram_schmidt(const GSArgs& args, int nactive, cudaStream_t st) {
     // algorithmic bytes: w read and written once; the basis streamed once per
     // pass (two passes with the selective test in its usual outcome, four for CGS2)
     kprof_begin("gram_schmidt", st);
-    if (gs_cluster_cost(a.n, a.cnt, passes, nactive) <= gs_grid_cost(a.n, a.cnt, passes, nactive))
-        gs_cluster(a, nactive, st);
+    const GsShape s = cluster_shape(a.n, a.cnt, passes, nactive);
+    if (s.cost <= gs_grid_cost(a.n, a.cnt, passes, nactive))
+        launch_cluster(a, nactive, s, st);
     else
         gs_grid(a, nactive, st);
     kprof_end("gram_schmidt", st, nactive * ((double)passes * a.cnt + 2.0) * a.n * sizeof(double2),
