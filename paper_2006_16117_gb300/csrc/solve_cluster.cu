@@ -349,24 +349,18 @@ __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, J
                 }
             }
         };
-        // A wait for a stage to be consumed, made by lane 0 for its whole warp: every lane
-        // gets the outcome, and false once the CTA has failed.  (A lane that went on
-        // alone would leave the others waiting in the next warp-wide instruction.)
-        auto stage_free = [&](int st, int rnd) {
-            bool free = true;
-            if (lane == 0) {
-                if (rnd >= 0) free = bounded([&] { return mbar_try_wait(&empty[st], (uint32_t)(rnd & 1)); }, 4);
-                if (failed_flag(&s_fail)) free = false;
-            }
-            return __shfl_sync(0xffffffffu, (int)free, 0) != 0;
-        };
         int slot = 0, round = 0, issued = 0;  // c = round * NS + slot
         bool ok = true;
         fetch_bounds(0);
         for (int b = 0; b < nsteps && ok; ++b) {
             const C* M = (phase == 0 || b == 0 ? Dinv : E) + (size_t)block_of(b) * T * T;
             for (int rs = r0; rs < r1; rs += SR) {
-                ok = stage_free(slot, round - 1);
+                if (lane == 0) {
+                    if (round > 0)
+                        ok = bounded([&] { return mbar_try_wait(&empty[slot], (uint32_t)((round - 1) & 1)); }, 4);
+                    if (failed_flag(&s_fail)) ok = false;
+                }
+                ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
                 if (!ok) break;
                 const int rows = min(SR, r1 - rs);
                 C* dst = stage + (size_t)slot * SR * TP;
@@ -377,10 +371,16 @@ __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, J
                     tma_load_1d(dst + (size_t)i * TP, M + (size_t)(rs + i) * T, (uint32_t)(T * sizeof(C)),
                                 &full[slot]);
                 if (b == 0 && rs == r0) vectors_ready();
-                // one chunk a step in this CTA: the inputs' buffer, as above (a wait that has
-                // failed ends the loop, after the arrivals of the chunk that is under way)
-                if (!ONE && myrows <= SR && b >= 2) ok = stage_free((b - 2) % NS, (b - 2) / NS);
-                if (ok && rs == r0) {
+                if (!ONE && myrows <= SR && b >= 2) {
+                    // one chunk a step in this CTA: the inputs' buffer, as above.  The outcome
+                    // is not kept in lane 0 alone (it would leave the loop by itself, and the
+                    // others wait for it in the next shuffle): a wait that ran out has set
+                    // s_fail, which the next chunk's check hands to the whole warp.
+                    if (lane == 0)
+                        bounded([&] { return mbar_try_wait(&empty[(b - 2) % NS], (uint32_t)(((b - 2) / NS) & 1)); }, 4);
+                    __syncwarp();
+                }
+                if (rs == r0) {
                     copies_done();  // the bounds asked for a step ago
                     __syncwarp();
                     fetch_inputs(b - LAG);
@@ -402,7 +402,9 @@ __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, J
             // the last chunk's inputs: their buffer is free when the chunk two before is
             const int c = nsteps - 1;
             if (ok && c >= 0) {
-                if (c >= 2) ok = stage_free((c - 2) % NS, (c - 2) / NS);
+                if (lane == 0 && c >= 2)
+                    ok = bounded([&] { return mbar_try_wait(&empty[(c - 2) % NS], (uint32_t)(((c - 2) / NS) & 1)); }, 4);
+                ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
                 copies_done();
                 __syncwarp();
                 if (ok) fetch_inputs(c);
@@ -412,9 +414,9 @@ __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, J
             }
         }
         copies_done();
-        // stopped early (a failure): the last issued copies may still be in flight,
+        // stopped by a failure: the last issued copies may still be in flight,
         // and this CTA's shared memory must outlive them
-        if (pt == 0 && !ok) {
+        if (pt == 0 && (!ok || failed_flag(&s_fail))) {
             for (int d = max(0, issued - NS); d < issued; ++d) {
                 long long it = 0;
                 while (!mbar_try_wait(&full[d % NS], (uint32_t)((d / NS) & 1)) && ++it < WAIT_LIMIT) {

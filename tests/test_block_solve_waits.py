@@ -1,7 +1,7 @@
-"""The block solve's waits that one lane makes for its warp: all lanes have to get
-the outcome, or those of a failed wait would wait in the next warp-wide
-instruction for a lane that has gone on (read from the source: a wait that runs
-out is not provoked on a GPU)."""
+"""The block solve's waits that one lane makes for its warp: a failed one must not
+send that lane on alone, or the others would wait for it in the next warp-wide
+instruction (read from the source: a wait that runs out is not provoked on a
+GPU)."""
 import os
 import re
 
@@ -14,19 +14,24 @@ def _producers():
     return s[s.index("// ---- producers"): s.index("// ---- consumers")]
 
 
-def test_every_wait_of_one_lane_is_broadcast_to_its_warp():
+def test_no_lane_keeps_the_outcome_of_a_wait_for_itself():
     text = _producers()
     waits = [m.start() for m in re.finditer(r"\bbounded\(", text)]
     assert waits
     for at in waits:
-        # the outcome's variable, and what follows the statement that waits: the next
-        # warp-wide instruction has to hand that variable to all lanes
-        name = re.search(r"(\w+) = $", text[:at]).group(1)
+        # up to the next warp-wide instruction; a wait that ran out has set s_fail
         nxt = re.search(r"__(shfl|syncwarp|any|all|ballot|reduce)\w*", text[at:])
-        assert nxt is not None and nxt.group(0).startswith("__shfl"), text[at: at + 200]
-        args = text[at + nxt.end(): at + nxt.end() + 60]
-        assert re.match(r"\(0xffffffffu, \(int\)%s, 0\)" % name, args), args
+        assert nxt is not None
         assert "break" not in text[at: at + nxt.start()] and "continue" not in text[at: at + nxt.start()]
+        kept = re.search(r"(\w+) = $", text[:at])
+        if kept:  # an outcome that is kept is handed to all lanes there
+            args = text[at + nxt.end(): at + nxt.end() + 60]
+            assert nxt.group(0).startswith("__shfl"), text[at: at + 200]
+            assert re.match(r"\(0xffffffffu, \(int\)%s, 0\)" % kept.group(1), args), args
+    # the check that ends the loop for the whole warp once s_fail is set
+    assert re.search(r"if \(failed_flag\(&s_fail\)\) ok = false;\s*\}\s*ok = __shfl_sync\(0xffffffffu, \(int\)ok, 0\)", text)
+    # and the copies in flight are waited for whichever lane or warp failed
+    assert "if (pt == 0 && (!ok || failed_flag(&s_fail)))" in text
 
 
 def test_recorded_wait_error_is_thrown_once(tmp_path):
