@@ -220,8 +220,11 @@ void gram_schmidt(const GSArgs& args, int nactive, cudaStream_t st) {
     // algorithmic bytes: w read and written once; the basis streamed once per
     // pass (two passes with the selective test in its usual outcome, four for CGS2)
     kprof_begin("gram_schmidt", st);
-    const GsShape s = cluster_shape(a.n, a.cnt, passes, nactive);
-    if (s.cost <= gs_grid_cost(a.n, a.cnt, passes, nactive))
+    // (the occupancy query only where its answer matters)
+    const double grid = gs_grid_cost(a.n, a.cnt, passes, nactive);
+    GsShape s = gs_cluster_shape(a.n, a.cnt, passes, nactive, sm_count(), [](int, int, size_t) { return true; });
+    if (s.cost <= grid) s = cluster_shape(a.n, a.cnt, passes, nactive);
+    if (s.cost <= grid)
         launch_cluster(a, nactive, s, st);
     else
         gs_grid(a, nactive, st);
