@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(CL_THREADS, MINB) k_block_solve_cl(Pencil P, J
             if (done()) return true;
             if (it > WAIT_LIMIT) {
                 s_fail = 1;
-                *(volatile int*)err = code;  // pinned host memory
+                atomicExch(err, code);  // pinned host memory
             }
         }
         return false;
